@@ -31,9 +31,6 @@ struct MlpWork {
     float* zd1 = nullptr;        // tangent pass
     float* zd2 = nullptr;
     float* h1b = nullptr;        // dL/dh1
-    float* t0 = nullptr;         // per-sample contributions to the bias / w3 gradients
-    float* t1 = nullptr;
-    float* t2 = nullptr;
     __nv_bfloat16* nu_a = nullptr;  // [cap][Pp]
     __nv_bfloat16* hd1 = nullptr;   // [cap][H]
     __nv_bfloat16* z2b = nullptr;   // [cap][H]
@@ -43,6 +40,7 @@ struct MlpWork {
     __nv_bfloat16* B2T = nullptr;   // [H][2cap]  (h1^T | hd1^T)
     float* ebar = nullptr;          // [cap]
     double* loss_part = nullptr;    // [cap]
+    double* sum_part = nullptr;     // [3][tiles][H] partial sums of the b1, b2 and w3 gradients
 };
 
 // Configurations read with strides: element (m, atom i, coordinate c) at

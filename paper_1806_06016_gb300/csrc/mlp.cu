@@ -133,48 +133,186 @@ __global__ void mlp_adam_kernel(float* p, const float* __restrict__ g, float* m,
 
 // ------------------------------------------------------------- normalisation
 
-__global__ void mlp_feature_stats_kernel(ConfigView cv, long long n, int N, int P,
-                                         const ushort2* __restrict__ pairs, float* mu, float* sd,
-                                         float* inv_sd) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= P) return;
-    const ushort2 ij = pairs[p];
-    auto g_of = [&](long long m) {
-        const float* x = cv.x + m * cv.s_cfg;
-        const double dx = (double)x[ij.x * cv.s_atom] - x[ij.y * cv.s_atom];
-        const double dy = (double)x[ij.x * cv.s_atom + cv.s_coord] - x[ij.y * cv.s_atom + cv.s_coord];
-        const double dz = (double)x[ij.x * cv.s_atom + 2 * cv.s_coord] - x[ij.y * cv.s_atom + 2 * cv.s_coord];
-        return 1.0 / sqrt(dx * dx + dy * dy + dz * dz);
-    };
-    double s = 0.0;
-    for (long long m = 0; m < n; ++m) s += g_of(m);
-    const double mean = s / (double)n;
-    double q = 0.0;
-    for (long long m = 0; m < n; ++m) {
-        const double d = g_of(m) - mean;
-        q += d * d;
+// Mean and sum of squared deviations of every feature g_p = 1 / r over n
+// configurations (and of the energies), merged from slices of the data.
+//
+// The result is that of 64-bit arithmetic, but GB300's FP64 units do a 64th
+// of the FP32 rate, and a reciprocal square root per sample and pair is all
+// the work there is.  So a sample's g is formed in pairs of FP32 numbers
+// (TwoSum: Knuth 1969; exact products by fma): coordinate differences are
+// exact, r^2 carries its rounding errors, and one Newton step on the hardware
+// reciprocal square root leaves g = y0 + corr with a relative error of about
+// 2^-44.  Deviations from the slice's first sample (exactly zero for an equal
+// one, so that a constant feature has no spurious deviation) are summed, with
+// their squares, in compensated FP32; slices become (mean,
+// M2) in FP64 and are merged by Chan, Golub & LeVeque's (1979) formula.
+// A distance outside [1e-10, 1e10] nm (coincident atoms, non-finite input)
+// marks its pair with a NaN, and the merge kernel then does that pair in plain
+// FP64.
+//
+// One thread per pair, the positions of a tile of configurations in shared
+// memory as float4 (consecutive pairs read consecutive atoms: no bank
+// conflicts), the data cut into as many slices as fill the chip.
+// 65536 configurations of 75 atoms: 611 + 29 us, bound by the FP32 issue rate
+// (about 85 instructions per sample and pair); one thread per pair looping
+// twice over all configurations in FP64 (22 blocks) took 151.0 ms.
+constexpr int kStatThreads = 256;
+constexpr int kStatTileBytes = 24 * 1024;
+
+// a + b = s + e exactly
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+    const float s = __fadd_rn(a, b);
+    const float bp = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bp)), __fsub_rn(b, bp));
+    return s;
+}
+// (s, e) with s^2 and its error including 2 s e
+__device__ __forceinline__ float square_err(float s, float e, float& err) {
+    const float p = __fmul_rn(s, s);
+    err = __fmaf_rn(__fadd_rn(s, s), e, __fmaf_rn(s, s, -p));
+    return p;
+}
+// (mean, M2) of na + nb values from those of the parts
+__device__ __forceinline__ void merge_moments(double& na, double& ma, double& qa, double nb, double mb, double qb) {
+    if (nb == 0.0) return;
+    if (na == 0.0) {
+        na = nb; ma = mb; qa = qb;
+        return;
     }
-    double dev = sqrt(q / (double)n);
-    if (!(dev > 0.0)) dev = 1.0;
-    mu[p] = (float)mean;
-    sd[p] = (float)dev;
-    inv_sd[p] = (float)(1.0 / dev);
+    const double n = na + nb, d = mb - ma;
+    ma += d * (nb / n);
+    qa += qb + d * d * (na * (nb / n));
+    na = n;
 }
 
-__global__ void mlp_energy_stats_kernel(const double* __restrict__ E, long long n, double* out) {
+// part[blockIdx.y][p]: (mean, M2) of slice blockIdx.y; the last block column
+// does the energies, entry P.
+__global__ void __launch_bounds__(kStatThreads) mlp_moments_kernel(const float* __restrict__ x,
+                                                                   const double* __restrict__ E, long long n,
+                                                                   long long per, int N, int P, int tile,
+                                                                   const ushort2* __restrict__ pairs,
+                                                                   double2* __restrict__ part) {
+    extern __shared__ float4 sx[];
     __shared__ double red[32];
-    double s = 0.0;
-    for (long long m = threadIdx.x; m < n; m += blockDim.x) s += E[m];
-    const double mean = block_sum(s, red) / (double)n;
-    double q = 0.0;
-    for (long long m = threadIdx.x; m < n; m += blockDim.x) {
-        const double d = E[m] - mean;
-        q += d * d;
+    const long long m0 = blockIdx.y * per, m1 = m0 + per < n ? m0 + per : n;
+    double2* out = part + (size_t)blockIdx.y * (P + 1);
+    if (blockIdx.x == gridDim.x - 1) {
+        double s = 0.0;
+        for (long long m = m0 + threadIdx.x; m < m1; m += kStatThreads) s += E[m];
+        const double mean = block_sum(s, red) / (double)(m1 - m0);
+        double q = 0.0;
+        for (long long m = m0 + threadIdx.x; m < m1; m += kStatThreads) {
+            const double d = E[m] - mean;
+            q += d * d;
+        }
+        q = block_sum(q, red);
+        if (threadIdx.x == 0) out[P] = make_double2(mean, q);
+        return;
     }
-    q = block_sum(q, red);
-    if (threadIdx.x == 0) {
-        out[0] = mean;
-        out[1] = sqrt(q / (double)n);
+    const int p = blockIdx.x * kStatThreads + threadIdx.x;
+    const ushort2 ij = pairs[p < P ? p : 0];
+    float g0 = 0.0f, c0 = 0.0f, s = 0.0f, sl = 0.0f, q = 0.0f, ql = 0.0f;
+    bool first = true, bad = false;
+    for (long long t0 = m0; t0 < m1; t0 += tile) {
+        const int nt = (int)(m1 - t0 < tile ? m1 - t0 : tile);
+        __syncthreads();
+        const float* src = x + (size_t)t0 * 3 * N;
+        for (int a = threadIdx.x; a < nt * N; a += kStatThreads)
+            sx[a] = make_float4(src[3 * a], src[3 * a + 1], src[3 * a + 2], 0.0f);
+        __syncthreads();
+#pragma unroll 2
+        for (int c = 0; c < nt; ++c) {
+            const float4 a = sx[c * N + ij.x], b = sx[c * N + ij.y];
+            float ex, ey, ez, qx, qy, qz, l1, l2;
+            const float dx = two_sum(a.x, -b.x, ex), dy = two_sum(a.y, -b.y, ey), dz = two_sum(a.z, -b.z, ez);
+            const float px = square_err(dx, ex, qx), py = square_err(dy, ey, qy), pz = square_err(dz, ez, qz);
+            const float h = two_sum(two_sum(px, py, l1), pz, l2);
+            const float lo = __fadd_rn(__fadd_rn(l1, l2), __fadd_rn(qx, __fadd_rn(qy, qz)));
+            bad = bad || !(h > 1e-20f && h < 1e20f);
+            const float y = rsqrtf(h);
+            // e = 1 - r^2 y^2
+            const float u = __fmul_rn(h, y), ue = __fmaf_rn(h, y, -u);
+            float e = __fmaf_rn(-u, y, 1.0f);
+            e = __fmaf_rn(-ue, y, e);
+            e = __fmaf_rn(-__fmul_rn(lo, y), y, e);
+            const float corr = __fmul_rn(y, __fmaf_rn(__fmul_rn(0.375f, e), e, __fmul_rn(0.5f, e)));
+            if (first) {
+                g0 = y;
+                c0 = corr;
+                first = false;
+            }
+            const float d = __fadd_rn(__fsub_rn(y, g0), __fsub_rn(corr, c0));
+            float err;
+            s = two_sum(s, d, err);
+            sl = __fadd_rn(sl, err);
+            const float d2 = __fmul_rn(d, d);
+            q = two_sum(q, d2, err);
+            ql = __fadd_rn(ql, __fadd_rn(err, __fmaf_rn(d, d, -d2)));
+        }
+    }
+    if (p < P) {
+        const double cnt = (double)(m1 - m0), S = (double)s + (double)sl, Q = (double)q + (double)ql;
+        const double m2 = Q - S * (S / cnt);
+        out[p] = bad ? make_double2(NAN, NAN) : make_double2(((double)g0 + (double)c0) + S / cnt, m2 > 0.0 ? m2 : 0.0);
+    }
+}
+
+// One warp per feature merges the slices in a fixed order; warp P the
+// energies (out[0] mean, out[1] standard deviation).
+__global__ void __launch_bounds__(128) mlp_moments_merge_kernel(const float* __restrict__ x, long long n,
+                                                                long long per, int slices, int N, int P,
+                                                                const ushort2* __restrict__ pairs,
+                                                                const double2* __restrict__ part, float* mu,
+                                                                float* sd, float* inv_sd, double* out) {
+    const int p = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (p > P) return;
+    double cn = 0.0, mean = 0.0, m2 = 0.0;
+    for (int y = lane; y < slices; y += 32) {
+        const long long m0 = y * per, m1 = m0 + per < n ? m0 + per : n;
+        const double2 v = part[(size_t)y * (P + 1) + p];
+        merge_moments(cn, mean, m2, (double)(m1 - m0), v.x, v.y);
+    }
+    for (int o = 1; o < 32; o <<= 1) {
+        const double bn = __shfl_down_sync(0xffffffffu, cn, o), bm = __shfl_down_sync(0xffffffffu, mean, o),
+                     bq = __shfl_down_sync(0xffffffffu, m2, o);
+        merge_moments(cn, mean, m2, bn, bm, bq);
+    }
+    mean = __shfl_sync(0xffffffffu, mean, 0);
+    m2 = __shfl_sync(0xffffffffu, m2, 0);
+    if (p == P) {
+        if (lane == 0) {
+            out[0] = mean;
+            out[1] = sqrt(m2 / (double)n);
+        }
+        return;
+    }
+    if (isnan(mean)) {  // a distance out of the fast path's range: this pair in FP64
+        const ushort2 ij = pairs[p];
+        auto g_of = [&](long long m) {
+            const float* c = x + m * 3 * N;
+            const double dx = (double)c[3 * ij.x] - c[3 * ij.y];
+            const double dy = (double)c[3 * ij.x + 1] - c[3 * ij.y + 1];
+            const double dz = (double)c[3 * ij.x + 2] - c[3 * ij.y + 2];
+            return 1.0 / sqrt(dx * dx + dy * dy + dz * dz);
+        };
+        double s = 0.0;
+        for (long long m = lane; m < n; m += 32) s += g_of(m);
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        mean = s / (double)n;
+        double q = 0.0;
+        for (long long m = lane; m < n; m += 32) {
+            const double d = g_of(m) - mean;
+            q += d * d;
+        }
+        for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        m2 = q;
+    }
+    if (lane == 0) {
+        double dev = sqrt(m2 / (double)n);
+        if (!(dev > 0.0)) dev = 1.0;
+        mu[p] = (float)mean;
+        sd[p] = (float)dev;
+        inv_sd[p] = (float)(1.0 / dev);
     }
 }
 
@@ -799,12 +937,34 @@ int pamd_mlp_fit_normalization(pamd_mlp* m, const float* x_dev, const double* E_
     int rc = check_model(m);
     if (rc) return rc;
     if (!x_dev || !E_dev || n < 2) return mfail(PAMD_EINVAL, "pamd_mlp_fit_normalization: null pointer or n < 2");
-    ConfigView cv{x_dev, 3LL * m->N, 3, 1, nullptr};
-    mlp_feature_stats_kernel<<<(m->P + 127) / 128, 128, 0, m->stream>>>(cv, n, m->N, m->P, m->pairs,
-                                                                         m->mu, m->sd, m->inv_sd);
+    int dev = 0, sms = 0;
+    MLP_CU(m, cudaGetDevice(&dev));
+    MLP_CU(m, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    // slices: six blocks per SM over all block columns, at least a tile each
+    const int cols = (m->P + kStatThreads - 1) / kStatThreads + 1;
+    const int tile = kStatTileBytes / (16 * m->N) > 0 ? kStatTileBytes / (16 * m->N) : 1;
+    const long long max_slices = (6LL * sms + cols - 1) / cols;
+    long long slices = (n + tile - 1) / tile;
+    if (slices > max_slices) slices = max_slices;
+    const long long per = (n + slices - 1) / slices;
+    slices = (n + per - 1) / per;  // no empty slice
+    if (m->moments_cap < max_slices) {  // kept with the model
+        if (m->moments) cudaFree(m->moments);
+        m->moments = nullptr;
+        m->moments_cap = 0;
+        if (cudaMalloc(&m->moments, sizeof(double2) * (size_t)max_slices * (m->P + 1)) != cudaSuccess) {
+            cudaGetLastError();
+            m->moments = nullptr;
+            return mfail(PAMD_ENOMEM, "pamd_mlp_fit_normalization: workspace");
+        }
+        m->moments_cap = max_slices;
+    }
+    mlp_moments_kernel<<<dim3(cols, (unsigned)slices), kStatThreads, sizeof(float4) * (size_t)tile * m->N, m->stream>>>(
+        x_dev, E_dev, n, per, m->N, m->P, tile, m->pairs, m->moments);
     if ((rc = launch_check(m, "feature statistics"))) return rc;
-    mlp_energy_stats_kernel<<<1, 1024, 0, m->stream>>>(E_dev, n, m->scratch);
-    if ((rc = launch_check(m, "energy statistics"))) return rc;
+    mlp_moments_merge_kernel<<<(m->P + 4) / 4, 128, 0, m->stream>>>(x_dev, n, per, (int)slices, m->N, m->P, m->pairs,
+                                                                    m->moments, m->mu, m->sd, m->inv_sd, m->scratch);
+    if ((rc = launch_check(m, "feature statistics"))) return rc;
     double st[2];
     MLP_CU(m, cudaMemcpyAsync(st, m->scratch, sizeof(st), cudaMemcpyDeviceToHost, m->stream));
     MLP_CU(m, cudaStreamSynchronize(m->stream));
@@ -1090,6 +1250,7 @@ void pamd_mlp_destroy(pamd_mlp* m) {
     if (m->loop_ctr) cudaFree(m->loop_ctr);
     if (m->body_stream) cudaStreamDestroy(m->body_stream);
     if (m->w.base) cudaFree(m->w.base);
+    if (m->moments) cudaFree(m->moments);
     if (m->base) cudaFree(m->base);
     if (m->own_stream && m->stream) cudaStreamDestroy(m->stream);
     delete m;

@@ -553,15 +553,33 @@ int launch_prop(pamd_ctx* c, int theta, double dt, double T, const uint32_t* dev
                           step0, fout);
 }
 
+// Shape of the all-FP64 kernel.  An SM issues one FP64 warp instruction in 16
+// cycles whatever its number of warps, so the time of a step is that of the
+// SM with the most warps: ceil(warps / SMs) times a warp's instructions, which
+// follow the mixed kernel's model (pairs per lane plus 16 pairs' worth per
+// atom for noise, bonded terms and integration).  75 atoms: R = 2048 takes 15
+// lanes x 5 atoms, R = 64 25 x 3.
+void choose_lanes_f64(int N, long long R, int num_sms, int* L, int* B) {
+    double best = 1e300;
+    for (int b = 1; b <= 8; ++b) {
+        const int l = (N + b - 1) / b;
+        if (l > 32) continue;
+        const long long warps = (R + 32 / l - 1) / (32 / l);
+        const double cost = (double)((warps + num_sms - 1) / num_sms) * (0.5 * b * (double)(l * b) + 16.0 * b);
+        if (cost < best) {
+            best = cost;
+            *L = l;
+            *B = b;
+        }
+    }
+}
+
 // Device tables of the all-FP64 mode: one allocation, laid out on the host.
 int build_topo_f64(pamd_ctx* c, const pamd_topology* t, std::vector<unsigned char>& blob) {
     const int N = t->n_atoms, Np = c->Np;
-    std::vector<double> sh(N), ep(N), q(N), im(N), x0(3 * (size_t)Np, 0.0);
+    std::vector<double> im(N), x0(3 * (size_t)Np, 0.0);
     double com[3] = {0, 0, 0}, mt = 0;
     for (int i = 0; i < N; ++i) {
-        sh[i] = 0.5 * t->sigma[i];
-        ep[i] = t->epsilon[i];
-        q[i] = t->charge[i];
         im[i] = 1.0 / t->mass[i];
         for (int k = 0; k < 3; ++k) com[k] += t->mass[i] * t->x0[3 * i + k];
         mt += t->mass[i];
@@ -577,6 +595,31 @@ int build_topo_f64(pamd_ctx* c, const pamd_topology* t, std::vector<unsigned cha
         const int i = t->excl[2 * p], j = t->excl[2 * p + 1];
         kind[(size_t)i * N + j] = kind[(size_t)j * N + i] = 1;
     }
+    // pair table of the half-ring tiles (layout: TopoF64::tab); each pair
+    // that counts appears once
+    int L = c->lay.lanes, B = c->lay.per_lane;
+    if (!c->lanes_req) choose_lanes_f64(N, c->R, c->num_sms, &L, &B);
+    const int TH = L / 2;
+    std::vector<double> tab((size_t)(TH + 1) * B * B * 3 * L, 0.0);
+    std::vector<unsigned long long> offb((size_t)(TH + 1) * L, 0ull);
+    for (int tile = 0; tile <= TH; ++tile)
+        for (int g = 0; g < L; ++g)
+            for (int b = 0; b < B; ++b)
+                for (int a = 0; a < B; ++a) {
+                    double* e = tab.data() + ((((size_t)tile * B + b) * B + a) * 3) * L + g;
+                    const int i = g * B + a, j = ((g + tile) % L) * B + b;
+                    const bool idle = tile == 0 ? a >= b : (2 * tile == L && g >= tile);
+                    if (idle || i >= N || j >= N || kind[(size_t)i * N + j] == 1) {
+                        offb[(size_t)tile * L + g] |= 1ull << (b * B + a);
+                        continue;
+                    }
+                    const bool p14 = kind[(size_t)i * N + j] == 2;
+                    const double sg = 0.5 * t->sigma[i] + 0.5 * t->sigma[j], s6 = sg * sg * sg * sg * sg * sg;
+                    const double e24 = 24.0 * std::sqrt(t->epsilon[i] * t->epsilon[j]) * (p14 ? t->scale14_lj : 1.0);
+                    e[0] = 2.0 * e24 * s6 * s6;
+                    e[L] = e24 * s6;
+                    e[2 * L] = kCoulomb * t->charge[i] * t->charge[j] * (p14 ? t->scale14_coul : 1.0);
+                }
     std::vector<double> bp(2 * (size_t)t->n_bonds), ap(2 * (size_t)t->n_angles), dp(4 * (size_t)t->n_dihedrals);
     for (int b = 0; b < t->n_bonds; ++b) { bp[2 * b] = t->bond_r0[b]; bp[2 * b + 1] = t->bond_k[b]; }
     for (int a = 0; a < t->n_angles; ++a) { ap[2 * a] = t->angle_t0[a]; ap[2 * a + 1] = t->angle_k[a]; }
@@ -594,8 +637,8 @@ int build_topo_f64(pamd_ctx* c, const pamd_topology* t, std::vector<unsigned cha
         if (bytes) std::memcpy(blob.data() + o, src, bytes);
         off.push_back(o);
     };
-    put(sh.data(), 8 * sh.size()); put(ep.data(), 8 * ep.size()); put(q.data(), 8 * q.size());
-    put(im.data(), 8 * im.size()); put(x0.data(), 8 * x0.size()); put(kind.data(), kind.size());
+    put(im.data(), 8 * im.size()); put(x0.data(), 8 * x0.size()); put(tab.data(), 8 * tab.size());
+    put(offb.data(), 8 * offb.size());
     put(t->bond, 8 * (size_t)t->n_bonds); put(bp.data(), 8 * bp.size());
     put(t->angle, 12 * (size_t)t->n_angles); put(ap.data(), 8 * ap.size());
     put(t->dihedral, 16 * (size_t)t->n_dihedrals); put(dp.data(), 8 * dp.size());
@@ -604,23 +647,21 @@ int build_topo_f64(pamd_ctx* c, const pamd_topology* t, std::vector<unsigned cha
     c->top64_blob = d;
     TopoF64& T = c->top64;
     T.n_atoms = N;
-    T.sigma_half = (const double*)(d + off[0]);
-    T.epsilon = (const double*)(d + off[1]);
-    T.charge = (const double*)(d + off[2]);
-    T.inv_mass = (const double*)(d + off[3]);
-    T.x0 = (const double*)(d + off[4]);
-    T.kind = d + off[5];
-    T.s14_lj = t->scale14_lj;
-    T.s14_c = t->scale14_coul;
+    T.lanes = L;
+    T.per_lane = B;
+    T.inv_mass = (const double*)(d + off[0]);
+    T.x0 = (const double*)(d + off[1]);
+    T.tab = (const double*)(d + off[2]);
+    T.off = (const unsigned long long*)(d + off[3]);
     T.n_bonds = t->n_bonds;
     T.n_angles = t->n_angles;
     T.n_dihs = t->n_dihedrals;
-    T.bond = (const int*)(d + off[6]);
-    T.bond_p = (const double*)(d + off[7]);
-    T.angle = (const int*)(d + off[8]);
-    T.angle_p = (const double*)(d + off[9]);
-    T.dih = (const int*)(d + off[10]);
-    T.dih_p = (const double*)(d + off[11]);
+    T.bond = (const int*)(d + off[4]);
+    T.bond_p = (const double*)(d + off[5]);
+    T.angle = (const int*)(d + off[6]);
+    T.angle_p = (const double*)(d + off[7]);
+    T.dih = (const int*)(d + off[8]);
+    T.dih_p = (const double*)(d + off[9]);
     return PAMD_OK;
 }
 

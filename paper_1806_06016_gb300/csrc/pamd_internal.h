@@ -98,13 +98,15 @@ struct PropParams {
 // device allocation.
 struct TopoF64 {
     int n_atoms;
-    const double* sigma_half;   // [N]
-    const double* epsilon;      // [N]
-    const double* charge;       // [N]
+    int lanes, per_lane;        // L lanes per replica, B atoms per lane
     const double* inv_mass;     // [N]
     const double* x0;           // [3][Np] recentred start geometry
-    const unsigned char* kind;  // [N][N]: 0 full, 1 excluded, 2 scaled 1-4 pair
-    double s14_lj, s14_c;
+    // nonbonded pairs, [L/2 + 1 tiles][b][a][3][L]: 48 eps sigma^12, 24 eps
+    // sigma^6 and k_e q q (with 1-4 factors) of atom gB + a against atom b of
+    // block (g + tile) mod L; zeros, and bit b B + a of off [tiles][L], for
+    // pairs that do not count
+    const double* tab;
+    const unsigned long long* off;
     int n_bonds, n_angles, n_dihs;
     const int* bond;            // [nb][2]
     const double* bond_p;       // [nb][2] r0, k

@@ -1143,13 +1143,14 @@ int pamd_init(pamd_ctx** out, const pamd_topology* top, int64_t R, double T0, ui
     b.blk_u64 = (unsigned long long*)dalloc(c, 8 * (size_t)c->n_blk);
     b.blk_f64 = (double*)dalloc(c, 8 * (size_t)c->n_blk);
     b.blk_i32 = (int32_t*)dalloc(c, 8 * (size_t)c->n_blk);
-    b.flags = (unsigned char*)dalloc(c, (size_t)c->R);
-    b.obs_part = (double*)dalloc(c, sizeof(double) * (64 * 5 + 1) * (size_t)c->n_blk);
+    b.fam_stamp = (uint32_t*)dalloc(c, 4 * (size_t)c->R);
+    b.obs_part = (double*)dalloc(c, obs_part_bytes(c->n_blk));
+    b.obs_ctl = dalloc(c, obs_ctl_bytes());
     b.scal = (DevScalars*)dalloc(c, sizeof(DevScalars));
     b.counters = (uint32_t*)dalloc(c, 16);
     if (!b.state || !b.state_alt || !b.E || !b.E_alt || !b.fam || !b.fam_alt || !b.ke || !b.rg ||
         !b.masses || !b.topo || !b.x0 || !b.W || !b.C || !b.cnt || !b.cnt_incl || !b.blk_u64 ||
-        !b.blk_f64 || !b.blk_i32 || !b.flags || !b.obs_part || !b.scal || !b.counters)
+        !b.blk_f64 || !b.blk_i32 || !b.fam_stamp || !b.obs_part || !b.obs_ctl || !b.scal || !b.counters)
         return bail(PAMD_ENOMEM, "device allocation failed");
     if (ensure_obs_cap(c, 2)) return bail(PAMD_ENOMEM, "device allocation failed");
     std::vector<unsigned char> t64;
@@ -1163,6 +1164,8 @@ int pamd_init(pamd_ctx** out, const pamd_topology* top, int64_t R, double T0, ui
               cudaMemcpyAsync(b.topo, blob.data(), blob.size(), cudaMemcpyHostToDevice, c->stream) == cudaSuccess &&
               cudaMemcpyAsync(b.x0, x0.data(), sizeof(float) * 3 * c->Np, cudaMemcpyHostToDevice, c->stream) == cudaSuccess &&
               cudaMemsetAsync(b.state_alt, 0, st_bytes, c->stream) == cudaSuccess &&
+              cudaMemsetAsync(b.fam_stamp, 0, 4 * (size_t)c->R, c->stream) == cudaSuccess &&
+              cudaMemsetAsync(b.obs_ctl, 0, obs_ctl_bytes(), c->stream) == cudaSuccess &&
               cudaMemsetAsync(b.ke, 0, sizeof(double) * c->R, c->stream) == cudaSuccess &&
               cudaMemsetAsync(b.rg, 0, sizeof(double) * c->R, c->stream) == cudaSuccess &&
               (t64.empty() || cudaMemcpyAsync(c->top64_blob, t64.data(), t64.size(),

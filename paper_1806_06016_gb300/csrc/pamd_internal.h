@@ -177,7 +177,8 @@ struct Buffers {
     unsigned long long* blk_u64 = nullptr;
     double* blk_f64 = nullptr;
     int32_t* blk_i32 = nullptr;
-    unsigned char* flags = nullptr;
+    uint32_t* fam_stamp = nullptr;  // [R] last observation that saw a family
+    void* obs_ctl = nullptr;        // counters of the observations (ObsCtl in resample.cu)
     double* obs_part = nullptr;
     DevScalars* scal = nullptr;
     uint32_t* counters = nullptr;
@@ -413,6 +414,8 @@ __global__ void counts_kernel(const unsigned long long* C, long long R, const De
 cudaError_t launch_init(pamd_ctx* c, double T0);
 cudaError_t launch_resample(pamd_ctx* c, double T_prev, double T_next, int do_resample,
                             const uint32_t* dev_counters, uint32_t resample_offset);
+size_t obs_part_bytes(int nblk);  // rows of the observables, one per 1024 replicas
+size_t obs_ctl_bytes();
 cudaError_t launch_observe(pamd_ctx* c, double T, pamd_obs* dst);
 cudaError_t launch_set_counters(pamd_ctx* c, uint32_t step, uint32_t ridx);
 

@@ -629,60 +629,72 @@ __global__ void __launch_bounds__(256) gather_kernel(
 
 // ------------------------------------------------------------------ observables
 
-// Family ids lie in 0 .. R-1 (R the slots of the population buffers); the
-// live replicas are the first live_size(live, R).
-__global__ void mark_kernel(const int32_t* fam, long long R, unsigned char* flags,
-                            const uint32_t* live) {
-    const long long n = live_size(live, R);
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
-         k += (long long)gridDim.x * blockDim.x) {
-        const int32_t f = fam[k];
-        if (f >= 0 && f < R) flags[f] = 1;
-    }
-}
+// One observation is one launch for populations of up to kObsFusedRows chunks
+// of 1024 replicas: every block writes its chunk's sums per family bin and
+// the block that finishes last adds the rows and forms the jackknife errors.
+// Larger populations add the rows in a second launch and finish in a third.
+// Everything is bound by latency, and by FP64 issue (one warp instruction in
+// 16 cycles per SM), so the sums run over short segments side by side and the
+// four jackknife errors in four warps.  R = 256: 15 us; R = 2^20: 40 + 4 + 11
+// us.  Before, with a cleared flag array, a marking pass, one thread per bin
+// walking its replicas and one thread doing the four errors in turn: 2 + 3 +
+// 13 + 87 us at R = 4096 and 5 + 43 + 407 us at R = 2^20.
 
 constexpr int kObsVals = 5;  // count, E, E_kin, R_g, R_g^2
-constexpr int kObsStride = kNumBins * kObsVals + 1;
+constexpr int kObsStride = kNumBins * kObsVals;
+constexpr int kObsSeg = 8;   // replicas a thread adds in a row
+constexpr int kObsFusedRows = 64;
+constexpr int kObsSlices = 16;
 
-// Partial sums per family bin over 1024 replicas, in replica order per bin.
-// Per-bin partial sums of one 1024-replica chunk.  Each bin's sums are
-// accumulated by one thread over the chunk's replicas of that bin in
-// increasing index order.  The replicas are first ordered by bin with a
-// stable counting sort (ranks within 32-replica pieces from
-// __match_any_sync, prefix counts over the pieces), so that the 64 bin
-// threads run side by side over their own segments instead of each scanning
-// the whole chunk.
-__global__ void obs_partial_kernel(const int32_t* fam, const double* E, const double* ke,
-                                   const double* rg, const unsigned char* flags, long long R,
-                                   double* part, const uint32_t* live) {
+// Device state of the observations of one context (zero at the start):
+// stamp[f] is the number of the last observation that saw family f, so that
+// no flag array is cleared between observations.
+struct ObsCtl {
+    uint32_t epoch;   // observations so far
+    uint32_t done;    // blocks that have finished this one
+    uint32_t families;
+    uint32_t pad;
+};
+
+// Per-bin partial sums of one 1024-replica chunk into out[kObsStride], and
+// the families this chunk is the first to see.  The replicas are ordered by
+// bin with a stable counting sort (ranks within 32-replica pieces from
+// __match_any_sync, prefix counts over the pieces), each bin's segment is cut
+// into pieces of at most kObsSeg, one thread each, and one thread per bin
+// adds its pieces in order.  A family id is counted by the first atomic
+// exchange that finds an older stamp; a run of equal ids (copies stand side
+// by side) needs one exchange.
+__device__ __forceinline__ void obs_chunk(const int32_t* fam, const double* E, const double* ke, const double* rg,
+                                          uint32_t* stamp, uint32_t epoch, ObsCtl* ctl, long long base, long long n,
+                                          long long R, double* out) {
     constexpr int kPieces = kScanBlock / 32;
     constexpr int kPerWarp = kPieces / (kScanThreads / 32);
+    constexpr int kSegs = kNumBins + kScanBlock / kObsSeg;  // at most
     static_assert(kPieces % (kScanThreads / 32) == 0, "pieces per warp");
-    const long long n = live_size(live, R);  // replicas; family flags span R
+    static_assert(kSegs <= kScanThreads, "one thread per segment");
     __shared__ int32_t sf[kScanBlock];
     __shared__ double se[kScanBlock], sk[kScanBlock], sr[kScanBlock];
-    __shared__ int32_t famcount[kScanThreads / 32];
     __shared__ int32_t pcount[kPieces][kNumBins];  // per piece and bin: count, then prefix
-    __shared__ int32_t bstart[kNumBins + 1];
+    __shared__ int32_t bstart[kNumBins + 1], sstart[kNumBins + 1];
     __shared__ int16_t order[kScanBlock];          // chunk entries sorted by bin (stable)
-    const long long base = (long long)blockIdx.x * kScanBlock;
-    int fc = 0;
-    for (int t = threadIdx.x; t < kScanBlock; t += blockDim.x) {
+    __shared__ double seg[4][kSegs];
+    int fresh = 0;
+    for (int t = threadIdx.x; t < kScanBlock; t += kScanThreads) {
         const long long k = base + t;
+        int32_t bin = -1;
         if (k < n) {
-            sf[t] = fam[k] & (kNumBins - 1);
+            const int32_t f = fam[k];
+            bin = f & (kNumBins - 1);
             se[t] = E[k];
             sk[t] = ke[k];
             sr[t] = rg[k];
-        } else {
-            sf[t] = -1;
+            if (f >= 0 && f < R && (k == 0 || fam[k - 1] != f) && atomicExch(&stamp[f], epoch) != epoch) ++fresh;
         }
-        if (k < R) fc += flags[k];
+        sf[t] = bin;
     }
-    for (int i = threadIdx.x; i < kPieces * kNumBins; i += blockDim.x) (&pcount[0][0])[i] = 0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) fc += __shfl_xor_sync(0xffffffffu, fc, o);
-    if ((threadIdx.x & 31) == 0) famcount[threadIdx.x >> 5] = fc;
+    for (int i = threadIdx.x; i < kPieces * kNumBins; i += kScanThreads) (&pcount[0][0])[i] = 0;
+    fresh = __reduce_add_sync(0xffffffffu, fresh);
+    if ((threadIdx.x & 31) == 0 && fresh) atomicAdd(&ctl->families, (uint32_t)fresh);
     __syncthreads();
     // ranks within each piece, and the pieces' counts per bin
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -698,6 +710,7 @@ __global__ void obs_partial_kernel(const int32_t* fam, const double* E, const do
     __syncthreads();
     if (threadIdx.x < kNumBins) {  // prefix over the pieces, per bin
         int s = 0;
+#pragma unroll 8
         for (int c = 0; c < kPieces; ++c) {
             const int x = pcount[c][threadIdx.x];
             pcount[c][threadIdx.x] = s;
@@ -706,13 +719,16 @@ __global__ void obs_partial_kernel(const int32_t* fam, const double* E, const do
         bstart[threadIdx.x + 1] = s;  // the bin's size, turned into starts below
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int s = 0;
-        bstart[0] = 0;
-        for (int b = 0; b < kNumBins; ++b) {
-            s += bstart[b + 1];
-            bstart[b + 1] = s;
-        }
+    if (w == 0) {  // starts of the bins and of their segments: two bins per lane
+        const int c0 = bstart[2 * lane + 1], c1 = bstart[2 * lane + 2];
+        const int s0 = (c0 + kObsSeg - 1) / kObsSeg, s1 = (c1 + kObsSeg - 1) / kObsSeg;
+        const int bi = warp_incl_scan(c0 + c1), si = warp_incl_scan(s0 + s1);
+        __syncwarp();
+        bstart[2 * lane + 1] = bi - c1;
+        bstart[2 * lane + 2] = bi;
+        sstart[2 * lane + 1] = si - s1;
+        sstart[2 * lane + 2] = si;
+        if (lane == 0) bstart[0] = sstart[0] = 0;
     }
     __syncthreads();
 #pragma unroll
@@ -723,83 +739,74 @@ __global__ void obs_partial_kernel(const int32_t* fam, const double* E, const do
         if (bin >= 0) order[bstart[bin] + pcount[c][bin] + rank[q]] = (int16_t)t;
     }
     __syncthreads();
-    double* out = part + (size_t)blockIdx.x * kObsStride;
-    if (threadIdx.x < kNumBins) {
-        const int b = threadIdx.x;
-        double c = 0, e = 0, k2 = 0, r = 0, r2 = 0;
-        for (int i = bstart[b]; i < bstart[b + 1]; ++i) {
+    if ((int)threadIdx.x < sstart[kNumBins]) {
+        int b = 0;  // the bin of this segment
+#pragma unroll
+        for (int h = kNumBins / 2; h > 0; h >>= 1)
+            if (sstart[b + h] <= (int)threadIdx.x) b += h;
+        const int i0 = bstart[b] + ((int)threadIdx.x - sstart[b]) * kObsSeg, i1 = min(i0 + kObsSeg, bstart[b + 1]);
+        double e = 0, k2 = 0, r = 0, r2 = 0;
+        for (int i = i0; i < i1; ++i) {
             const int t = order[i];
-            c += 1.0;
             e += se[t];
             k2 += sk[t];
             r += sr[t];
             r2 += sr[t] * sr[t];
         }
-        out[b * kObsVals + 0] = c;
-        out[b * kObsVals + 1] = e;
-        out[b * kObsVals + 2] = k2;
-        out[b * kObsVals + 3] = r;
-        out[b * kObsVals + 4] = r2;
-    }
-    if (threadIdx.x == 0) {
-        int s = 0;
-        for (int i = 0; i < kScanThreads / 32; ++i) s += famcount[i];
-        out[kNumBins * kObsVals] = (double)s;
-    }
-}
-
-// Jackknife standard error over the family bins from the leave-one-bin-out
-// means jk[b] (computed in parallel by the caller), bins that are empty or
-// hold the whole population left out; the sums run over the bins in order.
-__device__ double jackknife_se(const double* cnt, const double* jk, double R) {
-    int nb = 0;
-    double jm = 0.0;
-    for (int b = 0; b < kNumBins; ++b) {
-        if (cnt[b] == 0.0 || cnt[b] == R) continue;
-        jm += jk[b];
-        ++nb;
-    }
-    if (nb < 2) return 0.0;
-    jm /= nb;
-    double ss = 0.0;
-    for (int b = 0; b < kNumBins; ++b) {
-        if (cnt[b] == 0.0 || cnt[b] == R) continue;
-        ss += (jk[b] - jm) * (jk[b] - jm);
-    }
-    return sqrt((double)(nb - 1) / nb * ss);
-}
-
-__global__ void obs_final_kernel(const double* part, int nblk, long long R, int N, double T,
-                                 const DevScalars* s, pamd_obs* dst, const uint32_t* live) {
-    R = live_size(live, R);
-    __shared__ double bins[kObsVals][kNumBins];
-    __shared__ double jk[kObsVals][kNumBins];
-    __shared__ double tot[kObsVals];
-    __shared__ double nfam;
-    if (threadIdx.x < kNumBins) {
-        const int b = threadIdx.x;
-        double acc[kObsVals] = {0, 0, 0, 0, 0};
-        for (int blk = 0; blk < nblk; ++blk)
-            for (int v = 0; v < kObsVals; ++v) acc[v] += part[(size_t)blk * kObsStride + b * kObsVals + v];
-        for (int v = 0; v < kObsVals; ++v) bins[v][b] = acc[v];
-    }
-    if (threadIdx.x == kNumBins) {
-        double f = 0;
-        for (int blk = 0; blk < nblk; ++blk) f += part[(size_t)blk * kObsStride + kNumBins * kObsVals];
-        nfam = f;
+        seg[0][threadIdx.x] = e;
+        seg[1][threadIdx.x] = k2;
+        seg[2][threadIdx.x] = r;
+        seg[3][threadIdx.x] = r2;
     }
     __syncthreads();
-    if (threadIdx.x >= 1 && threadIdx.x < kObsVals) {  // totals over the bins, in bin order
-        const int v = threadIdx.x;
-        double t = 0;
-        for (int b = 0; b < kNumBins; ++b) t += bins[v][b];
-        tot[v] = t;
+    {  // one thread per bin and value
+        const int b = threadIdx.x & (kNumBins - 1), v = threadIdx.x / kNumBins;
+        double s = 0;
+        for (int i = sstart[b]; i < sstart[b + 1]; ++i) s += seg[v][i];
+        out[b * kObsVals + 1 + v] = s;
+        if (v == 0) out[b * kObsVals] = (double)(bstart[b + 1] - bstart[b]);
+    }
+}
+static_assert(kScanThreads == 4 * kNumBins, "one thread per bin and value");
+
+__device__ __forceinline__ double warp_sum_d(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Averages and jackknife standard errors over the family bins from `rows`
+// rows of per-bin sums (whole block, kScanThreads threads).  Warp v takes
+// value v + 1, two bins per lane; bins that are empty or hold the whole
+// population are left out.
+__device__ __forceinline__ void obs_finish(const double* part, int rows, long long R, int N, double T,
+                                           const DevScalars* s, ObsCtl* ctl, pamd_obs* dst) {
+    __shared__ double bins[kObsStride];
+    __shared__ double mean[4], err[4];
+    for (int c = threadIdx.x; c < kObsStride; c += kScanThreads) {
+        double acc = 0.0;
+#pragma unroll 8
+        for (int r = 0; r < rows; ++r) acc += __ldcg(part + (size_t)r * kObsStride + c);
+        bins[c] = acc;
     }
     __syncthreads();
+    const int lane = threadIdx.x & 31, v = threadIdx.x >> 5;
     const double Rd = (double)R;
-    if (threadIdx.x < kNumBins) {  // leave-one-bin-out means
-        const int b = threadIdx.x;
-        for (int v = 1; v < kObsVals; ++v) jk[v][b] = (tot[v] - bins[v][b]) / (Rd - bins[0][b]);
+    if (v < 4) {
+        const double x0 = bins[lane * kObsVals + 1 + v], x1 = bins[(lane + 32) * kObsVals + 1 + v];
+        const double n0 = bins[lane * kObsVals], n1 = bins[(lane + 32) * kObsVals];
+        const double tot = warp_sum_d(x0 + x1);
+        const bool k0 = n0 != 0.0 && n0 != Rd, k1 = n1 != 0.0 && n1 != Rd;
+        // leave-one-bin-out means
+        const double j0 = k0 ? (tot - x0) / (Rd - n0) : 0.0, j1 = k1 ? (tot - x1) / (Rd - n1) : 0.0;
+        const int nb = __popc(__ballot_sync(0xffffffffu, k0)) + __popc(__ballot_sync(0xffffffffu, k1));
+        const double jm = warp_sum_d(j0 + j1) / (double)(nb > 0 ? nb : 1);
+        const double d0 = k0 ? j0 - jm : 0.0, d1 = k1 ? j1 - jm : 0.0;
+        const double ss = warp_sum_d(d0 * d0 + d1 * d1);
+        if (lane == 0) {
+            mean[v] = tot / Rd;
+            err[v] = nb < 2 ? 0.0 : sqrt((double)(nb - 1) / nb * ss);
+        }
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -807,21 +814,76 @@ __global__ void obs_final_kernel(const double* part, int nblk, long long R, int 
         o.T = T;
         o.lnQ = s->lnQ;
         o.sum_lnQ = s->sum_lnQ;
-        o.e_pot = tot[1] / Rd;
-        o.e_pot_se = jackknife_se(bins[0], jk[1], Rd);
-        o.e_kin = tot[2] / Rd;
-        o.e_kin_se = jackknife_se(bins[0], jk[2], Rd);
+        o.e_pot = mean[0];
+        o.e_pot_se = err[0];
+        o.e_kin = mean[1];
+        o.e_kin_se = err[1];
         o.t_meas = 2.0 * o.e_kin / (3.0 * N * kBoltzmann);
-        o.rg = tot[3] / Rd;
-        o.rg_se = jackknife_se(bins[0], jk[3], Rd);
-        o.rg2 = tot[4] / Rd;
-        o.rg2_se = jackknife_se(bins[0], jk[4], Rd);
-        o.n_families = (int64_t)nfam;
+        o.rg = mean[2];
+        o.rg_se = err[2];
+        o.rg2 = mean[3];
+        o.rg2_se = err[3];
+        o.n_families = (int64_t)__ldcg(&ctl->families);
         o.max_copies = s->max_copies;
         o.pad_ = s->status;
         o.R_live = R;
         *dst = o;
+        // ready for the next observation
+        ctl->epoch += 1;
+        ctl->families = 0;
+        ctl->done = 0;
     }
+}
+
+struct ObsArgs {
+    const int32_t* fam;
+    const double *E, *ke, *rg;
+    uint32_t* stamp;
+    ObsCtl* ctl;
+    double* part;          // [blocks][kObsStride], then [kObsSlices][kObsStride]
+    long long R;
+    const uint32_t* live;
+    int N, nblk;
+    double T;
+    const DevScalars* s;
+    pamd_obs* dst;
+};
+
+template <bool FUSED>
+__global__ void __launch_bounds__(kScanThreads) obs_kernel(const ObsArgs g) {
+    __shared__ int last;
+    const long long n = live_size(g.live, g.R);
+    obs_chunk(g.fam, g.E, g.ke, g.rg, g.stamp, g.ctl->epoch + 1, g.ctl, (long long)blockIdx.x * kScanBlock, n, g.R,
+              g.part + (size_t)blockIdx.x * kObsStride);
+    if (!FUSED) return;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&g.ctl->done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    obs_finish(g.part, g.nblk, n, g.N, g.T, g.s, g.ctl, g.dst);
+}
+
+// Rows of slice blockIdx.y added: 32 columns per block, eight row groups.
+__global__ void __launch_bounds__(kScanThreads) obs_rows_kernel(const double* part, int nblk, double* out) {
+    __shared__ double sh[kScanThreads];
+    const int c = blockIdx.x * 32 + (threadIdx.x & 31), q = threadIdx.x >> 5;
+    const int per = (nblk + kObsSlices - 1) / kObsSlices;
+    const int r0 = blockIdx.y * per, r1 = min(r0 + per, nblk);
+    double s = 0.0;
+#pragma unroll 4
+    for (int r = r0 + q; r < r1; r += kScanThreads / 32) s += part[(size_t)r * kObsStride + c];
+    sh[threadIdx.x] = s;
+    __syncthreads();
+    if (q) return;
+    for (int i = 1; i < kScanThreads / 32; ++i) s += sh[threadIdx.x + 32 * i];
+    out[(size_t)blockIdx.y * kObsStride + c] = s;
+}
+static_assert(kObsStride % 32 == 0, "whole column groups");
+
+__global__ void __launch_bounds__(kScanThreads) obs_final_kernel(const ObsArgs g) {
+    obs_finish(g.part + (size_t)g.nblk * kObsStride, kObsSlices, live_size(g.live, g.R), g.N, g.T, g.s, g.ctl, g.dst);
 }
 
 // ------------------------------------------------------------------ host side
@@ -950,19 +1012,36 @@ cudaError_t launch_resample(pamd_ctx* c, double T_prev, double T_next, int do_re
     return cudaGetLastError();
 }
 
+size_t obs_part_bytes(int nblk) { return sizeof(double) * kObsStride * ((size_t)nblk + kObsSlices); }
+size_t obs_ctl_bytes() { return sizeof(ObsCtl); }
+
 cudaError_t launch_observe(pamd_ctx* c, double T, pamd_obs* dst) {
     cudaStream_t s = c->stream;
-    const long long R = c->R;
-    const int32_t* fam = c->cur_is_alt ? c->b.fam_alt : c->b.fam;
-    const double* E = c->cur_is_alt ? c->b.E_alt : c->b.E;
-    cudaError_t e = cudaMemsetAsync(c->b.flags, 0, (size_t)R, s);
-    if (e != cudaSuccess) return e;
-    const uint32_t* live = c->variable ? c->b.counters + 2 : nullptr;
-    mark_kernel<<<grid_for(R, 256, c->num_sms * 16), 256, 0, s>>>(fam, R, c->b.flags, live);
-    obs_partial_kernel<<<c->n_blk, kScanThreads, 0, s>>>(fam, E, c->b.ke, c->b.rg, c->b.flags, R,
-                                                        c->b.obs_part, live);
-    obs_final_kernel<<<1, 128, 0, s>>>(c->b.obs_part, c->n_blk, R, c->N, T, c->b.scal, dst, live);
-    c->launches += 3;
+    ObsArgs g{};
+    g.fam = c->cur_is_alt ? c->b.fam_alt : c->b.fam;
+    g.E = c->cur_is_alt ? c->b.E_alt : c->b.E;
+    g.ke = c->b.ke;
+    g.rg = c->b.rg;
+    g.stamp = c->b.fam_stamp;
+    g.ctl = reinterpret_cast<ObsCtl*>(c->b.obs_ctl);
+    g.part = c->b.obs_part;
+    g.R = c->R;
+    g.live = c->variable ? c->b.counters + 2 : nullptr;
+    g.N = c->N;
+    g.nblk = c->n_blk;
+    g.T = T;
+    g.s = c->b.scal;
+    g.dst = dst;
+    if (g.nblk <= kObsFusedRows) {
+        obs_kernel<true><<<g.nblk, kScanThreads, 0, s>>>(g);
+        c->launches += 1;
+    } else {
+        obs_kernel<false><<<g.nblk, kScanThreads, 0, s>>>(g);
+        obs_rows_kernel<<<dim3(kObsStride / 32, kObsSlices), kScanThreads, 0, s>>>(
+            g.part, g.nblk, g.part + (size_t)g.nblk * kObsStride);
+        obs_final_kernel<<<1, kScanThreads, 0, s>>>(g);
+        c->launches += 3;
+    }
     return cudaGetLastError();
 }
 

@@ -4,6 +4,7 @@
 // weights, velocity rescaling) and step 4 (population averages with
 // family-binned errors).  Everything here is O(R) work between the
 // propagate launches; the gather is the one HBM-bound kernel.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "pamd_device.cuh"
@@ -75,6 +76,12 @@ __device__ __forceinline__ double block_sum_d(double v, double* sh) {
     for (int i = 0; i < nw; ++i) s += sh[i];
     __syncthreads();
     return s;
+}
+
+__device__ __forceinline__ double warp_sum_d(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
 // ------------------------------------------------------------------ init
@@ -277,8 +284,32 @@ __global__ void scan_local_u64_kernel(unsigned long long* W, long long R,
 
 // ------------------------------------------------------------------ counts
 
-// Draw k: u_k from Philox(seed; k, resampling index, 0, RESAMPLE | mol << 8),
-// target t = floor(u_k C_total / 2^64), ancestor = first j with C_j > t.
+// Target of draw k.  Multinomial (rule 1): u_k from Philox(seed; k, resampling
+// index, 0, RESAMPLE | mol << 8), t = floor(u_k C_total / 2^64).  Systematic
+// (rule 2): t_k = floor((k C + V) / R), V = floor(u_0 C / 2^64), by long
+// division in 32-bit digits (the numerator is below 2^84 and the quotient
+// below C).
+__device__ __forceinline__ unsigned long long draw_target(long long k, long long R, unsigned long long total, int rule,
+                                                          unsigned long long seed, uint32_t ridx, uint32_t purpose) {
+    const uint4 o = philox4x32_10(make_uint4(rule == 2 ? 0u : (uint32_t)k, ridx, 0u, purpose), seed_key(seed));
+    const unsigned long long u = (unsigned long long)o.x | ((unsigned long long)o.y << 32);
+    const unsigned long long V = __umul64hi(u, total);
+    if (rule != 2) return V;
+    const unsigned long long plo = (unsigned long long)k * total;  // low 64 bits of k C
+    unsigned long long phi = __umul64hi((unsigned long long)k, total);
+    const unsigned long long lo64 = plo + V;
+    phi += (lo64 < plo) ? 1ull : 0ull;
+    const unsigned long long r64 = (unsigned long long)R;
+    unsigned long long rem = phi % r64;  // phi < R: the quotient's high word is zero
+    unsigned long long cur = (rem << 32) | (lo64 >> 32);
+    const unsigned long long q1 = cur / r64;
+    rem = cur % r64;
+    cur = (rem << 32) | (lo64 & 0xffffffffull);
+    const unsigned long long q0 = cur / r64;
+    return (q1 << 32) | q0;
+}
+
+// Draw k: ancestor = first j with C_j > target.
 __global__ void counts_kernel(const unsigned long long* C, long long R, const DevScalars* s,
                               unsigned long long seed, const uint32_t* dev_counters,
                               uint32_t ridx_off, uint32_t purpose, int do_resample,
@@ -292,31 +323,7 @@ __global__ void counts_kernel(const unsigned long long* C, long long R, const De
             cnt[k] = 1;
             continue;
         }
-        unsigned long long t;
-        if (do_resample == 2) {
-            // systematic: t_k = floor((k C + V) / R), V = floor(u_0 C / 2^64), by
-            // long division in 32-bit digits (the numerator is below 2^84 and
-            // the quotient below C)
-            const uint4 o = philox4x32_10(make_uint4(0u, ridx, 0u, purpose), seed_key(seed));
-            const unsigned long long u0 = (unsigned long long)o.x | ((unsigned long long)o.y << 32);
-            const unsigned long long V = __umul64hi(u0, total);
-            const unsigned long long plo = (unsigned long long)k * total;  // low 64 bits of k C
-            unsigned long long phi = __umul64hi((unsigned long long)k, total);
-            const unsigned long long lo64 = plo + V;
-            phi += (lo64 < plo) ? 1ull : 0ull;
-            const unsigned long long r64 = (unsigned long long)R;
-            unsigned long long rem = phi % r64;  // phi < R: the quotient's high word is zero
-            unsigned long long cur = (rem << 32) | (lo64 >> 32);
-            const unsigned long long q1 = cur / r64;
-            rem = cur % r64;
-            cur = (rem << 32) | (lo64 & 0xffffffffull);
-            const unsigned long long q0 = cur / r64;
-            t = (q1 << 32) | q0;
-        } else {
-            const uint4 o = philox4x32_10(make_uint4((uint32_t)k, ridx, 0u, purpose), seed_key(seed));
-            const unsigned long long u = (unsigned long long)o.x | ((unsigned long long)o.y << 32);
-            t = __umul64hi(u, total);
-        }
+        const unsigned long long t = draw_target(k, R, total, do_resample, seed, ridx, purpose);
         long long lo = 0, hi = R;
         while (lo < hi) {
             const long long mid = lo + ((hi - lo) >> 1);
@@ -327,6 +334,270 @@ __global__ void counts_kernel(const unsigned long long* C, long long R, const De
         // a population whose weights are all zero (all energies non-finite)
         atomicAdd(&cnt[lo < R ? lo : R - 1], 1);
     }
+}
+
+// ------------------------------------------------------------------ one launch
+//
+// Weights, prefix sums, draws, copy counts and ancestors of a population of up
+// to kClusterMaxR replicas in one launch: a cluster of up to eight CTAs, each
+// with a chunk of the population in shared memory, exchanging maxima, totals,
+// search probes and count increments through distributed shared memory.  Same
+// integer weights, targets and ancestors as the kernels above, bit for bit;
+// only the sum behind ln Q is taken in another order.
+// Bound by latency: six cluster barriers, one binary search and, per element,
+// one FP64 exponential (maxima run on integer keys and block sums in one warp:
+// an FP64 instruction of all 16 warps costs 256 cycles).  12 us at R = 256 and
+// 33 us at R = 8192; the separate kernels and a cleared count array take 42
+// and 64 us and eight more launches.  A chunk of more than 2048 would spend
+// longer on its exponentials (5.5 us per 1024) than the launches saved, and
+// eight CTAs are the portable cluster size: above 16384 replicas the separate
+// kernels, spread over all SMs, are used.
+constexpr int kClusterThreads = 512, kClusterCtas = 8, kClusterMaxPer = 4;
+constexpr long long kClusterMaxR = (long long)kClusterThreads * kClusterCtas * kClusterMaxPer;
+
+struct ClusterArgs {
+    const double* E;
+    long long R;
+    double dbeta, two_s;
+    DevScalars* s;
+    ExpCoef cf;
+    unsigned long long seed;
+    const uint32_t* dev_counters;
+    uint32_t ridx_off, purpose;
+    int rule;                // 0: every copy once, 1 multinomial, 2 systematic
+    int32_t *cnt, *incl, *anc;
+};
+
+// Order-preserving map of a double's bits to a signed 64-bit key (no NaN):
+// the maximum then runs on the integer units.  Its own inverse.
+__device__ __forceinline__ long long order_key(double v) {
+    const long long b = __double_as_longlong(v);
+    return b >= 0 ? b : (b ^ 0x7fffffffffffffffLL);
+}
+__device__ __forceinline__ double key_value(long long k) {
+    return __longlong_as_double(k >= 0 ? k : (k ^ 0x7fffffffffffffffLL));
+}
+
+// inclusive scan over the block of PER consecutive values per thread; returns the total
+template <typename T, int PER>
+__device__ __forceinline__ T block_scan(T (&v)[PER], T* sh) {
+#pragma unroll
+    for (int q = 1; q < PER; ++q) v[q] += v[q - 1];
+    const T mine = v[PER - 1];
+    const T incl = warp_incl_scan(mine);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (lane == 31) sh[w] = incl;
+    __syncthreads();
+    T pre = incl - mine, total = 0;
+#pragma unroll
+    for (int i = 0; i < kClusterThreads / 32; ++i) {
+        const T x = sh[i];
+        if (i < w) pre += x;
+        total += x;
+    }
+#pragma unroll
+    for (int q = 0; q < PER; ++q) v[q] += pre;
+    __syncthreads();
+    return total;
+}
+
+template <int PER>
+__global__ void __launch_bounds__(kClusterThreads) resample_cluster_kernel(const ClusterArgs g) {
+    namespace cg = cooperative_groups;
+    constexpr int kChunk = kClusterThreads * PER;
+    __shared__ unsigned long long sC[kChunk];
+    __shared__ int32_t sN[kChunk];
+    __shared__ unsigned long long shw[kClusterThreads / 32];
+    __shared__ double shd[kClusterThreads / 32];
+    __shared__ long long shk[kClusterThreads / 32];
+    __shared__ int32_t shi[kClusterThreads / 32], sht[kClusterThreads / 32];
+    // this CTA's contributions, read by the others
+    __shared__ long long x_max;
+    __shared__ double x_sum;
+    __shared__ unsigned long long x_w;
+    __shared__ int32_t x_n, x_top;
+    __shared__ unsigned long long w_end[kClusterCtas];  // inclusive sums of the CTAs' totals
+    __shared__ int32_t n_end[kClusterCtas];
+    constexpr int kWarps = kClusterThreads / 32;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), ctas = (int)cl.num_blocks();
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    const long long j0 = (long long)rank * kChunk + (long long)threadIdx.x * PER;
+    // a_j and the maximum
+    double a[PER];
+    long long mk = order_key(-INFINITY);
+    bool ok[PER];
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        const bool in = j0 + q < g.R;
+        const double e = in ? g.E[j0 + q] : 0.0;
+        ok[q] = in && isfinite(e);
+        if (in && !ok[q] && atomicCAS(&g.s->status, 0, PAMD_ENONFINITE) == 0)
+            g.s->bad_replica = (int)(j0 + q);  // a non-finite energy gets weight 0
+        a[q] = ok[q] ? __dmul_rn(-g.dbeta, e) : 0.0;
+        if (ok[q]) mk = max(mk, order_key(a[q]));
+        sN[threadIdx.x * PER + q] = 0;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mk = max(mk, __shfl_xor_sync(0xffffffffu, mk, o));
+    if (lane == 0) shk[wp] = mk;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < kWarps; ++i) mk = max(mk, shk[i]);
+        x_max = mk;
+    }
+    cl.sync();
+    mk = order_key(-INFINITY);
+    for (int r = 0; r < ctas; ++r) mk = max(mk, *cl.map_shared_rank(&x_max, r));
+    const double m = key_value(mk);
+    // integer weights and their prefix sums
+    unsigned long long w[PER];
+    double es = 0.0;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        double e = 0.0;
+        w[q] = 0ull;
+        if (ok[q]) {
+            e = exp_det(__dsub_rn(a[q], m), g.cf);
+            w[q] = __double2ull_rz(__dmul_rn(g.two_s, e));
+        }
+        es = q ? es + e : e;
+    }
+    es = warp_sum_d(es);
+    if (lane == 0) shd[wp] = es;
+    const unsigned long long wt = block_scan(w, shw);  // orders the writes of shd as well
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < kWarps; ++i) es += shd[i];
+        x_sum = es;
+        x_w = wt;
+    }
+    cl.sync();
+    if (threadIdx.x == 0) {
+        unsigned long long c = 0;
+        for (int r = 0; r < ctas; ++r) w_end[r] = c += *cl.map_shared_rank(&x_w, r);
+    }
+    __syncthreads();
+    const unsigned long long total = w_end[ctas - 1], woff = rank ? w_end[rank - 1] : 0ull;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) sC[threadIdx.x * PER + q] = woff + w[q];
+    cl.sync();
+    // the last warp forms ln Q while the others search
+    if (rank == 0 && threadIdx.x == kClusterThreads - 1) {
+        double S = 0.0;
+        for (int r = 0; r < ctas; ++r) S += *cl.map_shared_rank(&x_sum, r);
+        const double lnq = m + (log(S) - log((double)g.R));
+        g.s->m = m;
+        g.s->S = S;
+        g.s->C_total = total;
+        g.s->lnQ = lnq;
+        g.s->sum_lnQ += lnq;
+    }
+    // draws: the CTA that holds the ancestor, then a search of its chunk, all
+    // of a thread's draws side by side
+    const uint32_t ridx = (g.dev_counters ? g.dev_counters[1] : 0u) + g.ridx_off;
+    if (!g.rule) {
+#pragma unroll
+        for (int q = 0; q < PER; ++q)
+            if (j0 + q < g.R) sN[threadIdx.x * PER + q] = 1;
+    } else {
+        unsigned long long t[PER];
+        const unsigned long long* chunk[PER];
+        int rr[PER], at[PER];
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            t[q] = draw_target(j0 + q, g.R, total, g.rule, g.seed, ridx, g.purpose);
+            int r = 0;
+            while (r < ctas - 1 && w_end[r] <= t[q]) ++r;
+            rr[q] = r;
+            chunk[q] = cl.map_shared_rank(sC, r);
+            at[q] = 0;  // elements known to be <= t
+        }
+#pragma unroll
+        for (int h = kChunk / 2; h > 0; h >>= 1)
+#pragma unroll
+            for (int q = 0; q < PER; ++q)
+                if (chunk[q][at[q] + h - 1] <= t[q]) at[q] += h;
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            if (j0 + q >= g.R) continue;
+            if (chunk[q][at[q]] <= t[q]) ++at[q];
+            long long j = (long long)rr[q] * kChunk + at[q];
+            // only a population whose weights are all zero reaches the clamp
+            if (j >= g.R) j = g.R - 1;
+            const int r = (int)(j / kChunk);
+            atomicAdd(cl.map_shared_rank(sN, r) + (j - (long long)r * kChunk), 1);
+        }
+    }
+    cl.sync();
+    // copy counts and their prefix sums
+    int32_t n[PER], cnt[PER], top = 0;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        cnt[q] = n[q] = sN[threadIdx.x * PER + q];
+        top = max(top, n[q]);
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    if (lane == 0) sht[wp] = top;
+    const int32_t nt = block_scan(n, shi);
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < kWarps; ++i) top = max(top, sht[i]);
+        x_n = nt;
+        x_top = top;
+    }
+    cl.sync();
+    if (threadIdx.x == 0) {
+        int32_t c = 0, t = 0;
+        for (int r = 0; r < ctas; ++r) {
+            n_end[r] = c += *cl.map_shared_rank(&x_n, r);
+            t = max(t, *cl.map_shared_rank(&x_top, r));
+        }
+        if (rank == 0) {
+            g.s->max_copies = t;
+            g.s->R_new = c;  // size of the new population (sum of the copy counts)
+        }
+    }
+    __syncthreads();
+    const int32_t noff = rank ? n_end[rank - 1] : 0;
+    // ancestors of the new slots: each ancestor fills its own, the whole warp
+    // those of an ancestor with many copies
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        const int32_t end = noff + n[q], c = cnt[q];
+        if (j0 + q < g.R) {
+            g.cnt[j0 + q] = c;
+            g.incl[j0 + q] = end;
+        }
+        if (c <= 4)
+            for (int i = 0; i < c; ++i) g.anc[end - c + i] = (int32_t)(j0 + q);
+        unsigned many = __ballot_sync(0xffffffffu, c > 4);
+        while (many) {
+            const int l = __ffs(many) - 1;
+            many &= many - 1;
+            const int32_t lc = __shfl_sync(0xffffffffu, c, l), le = __shfl_sync(0xffffffffu, end, l);
+            const int32_t lj = (int32_t)__shfl_sync(0xffffffffu, j0 + q, l);
+            for (int i = lane; i < lc; i += 32) g.anc[le - lc + i] = lj;
+        }
+    }
+    cl.sync();  // no CTA leaves while another reads its shared memory
+}
+
+cudaError_t launch_resample_cluster(const ClusterArgs& g, cudaStream_t s) {
+    int ctas = 1;
+    while (ctas < kClusterCtas && (long long)ctas * kClusterThreads < g.R) ctas *= 2;
+    const long long per = (g.R + (long long)ctas * kClusterThreads - 1) / ((long long)ctas * kClusterThreads);
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    cfg.gridDim = dim3((unsigned)ctas);
+    cfg.blockDim = dim3(kClusterThreads);
+    cfg.stream = s;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)ctas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    if (per <= 1) return cudaLaunchKernelEx(&cfg, resample_cluster_kernel<1>, g);
+    if (per <= 2) return cudaLaunchKernelEx(&cfg, resample_cluster_kernel<2>, g);
+    return cudaLaunchKernelEx(&cfg, resample_cluster_kernel<4>, g);
 }
 
 // ------------------------------------------------------------------ copy numbers
@@ -769,12 +1040,6 @@ __device__ __forceinline__ void obs_chunk(const int32_t* fam, const double* E, c
 }
 static_assert(kScanThreads == 4 * kNumBins, "one thread per bin and value");
 
-__device__ __forceinline__ double warp_sum_d(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
 // Averages and jackknife standard errors over the family bins from `rows`
 // rows of per-bin sums (whole block, kScanThreads threads).  Warp v takes
 // value v + 1, two bins per lane; bins that are empty or hold the whole
@@ -948,28 +1213,41 @@ cudaError_t launch_resample(pamd_ctx* c, double T_prev, double T_next, int do_re
 
     // energies of the current population (the ping-pong buffers alternate)
     const double* Ecur = c->cur_is_alt ? c->b.E_alt : c->b.E;
-    amax_kernel<<<nblk, kScanThreads, 0, s>>>(Ecur, R, dbeta, c->b.blk_f64, live);
-    max_top_kernel<<<1, 1024, 0, s>>>(c->b.blk_f64, nblk, c->b.scal);
-    weights_kernel<<<nblk, kScanThreads, 0, s>>>(Ecur, R, dbeta, two_s, c->b.scal, cf, c->b.W,
-                                                 c->b.blk_u64, c->b.blk_f64, live);
-    weights_top_kernel<<<1, kScanThreads, 0, s>>>(c->b.blk_u64, c->b.blk_f64, nblk, R, c->b.scal, live);
-    scan_local_u64_kernel<<<nblk, kScanThreads, 0, s>>>(c->b.W, R, c->b.blk_u64, c->b.C, live);
-    cudaError_t e = cudaMemsetAsync(c->b.cnt, 0, sizeof(int32_t) * (size_t)R, s);
-    if (e != cudaSuccess) return e;
-    if (c->variable && do_resample) {
-        varsize_counts_kernel<<<grid_for(R, 256, c->num_sms * 16), 256, 0, s>>>(
-            c->b.W, R, c->b.scal, c->R_target, c->seed, dev_counters, resample_offset,
-            kPurposeResample | ((uint32_t)c->mol << 8),
-            c->resample_rule == PAMD_RESAMPLE_NEAREST ? 3 : 4, cf, c->b.cnt, live);
+    const int rule = !do_resample ? 0 : (c->resample_rule == PAMD_RESAMPLE_SYSTEMATIC ? 2 : 1);
+    const uint32_t purpose = kPurposeResample | ((uint32_t)c->mol << 8);
+    // ancestors of the new slots (into the weight buffer)
+    int32_t* anc = reinterpret_cast<int32_t*>(c->b.W);
+    if (!c->variable && R <= kClusterMaxR) {
+        const ClusterArgs g{Ecur, R, dbeta, two_s, c->b.scal, cf, c->seed, dev_counters, resample_offset, purpose, rule,
+                            c->b.cnt, c->b.cnt_incl, anc};
+        const cudaError_t e = launch_resample_cluster(g, s);
+        if (e != cudaSuccess) return e;
+        c->launches += 1;
     } else {
-        const int rule = !do_resample ? 0 : (c->resample_rule == PAMD_RESAMPLE_SYSTEMATIC ? 2 : 1);
-        counts_kernel<<<grid_for(R, 256, c->num_sms * 16), 256, 0, s>>>(
-            c->b.C, R, c->b.scal, c->seed, dev_counters, resample_offset,
-            kPurposeResample | ((uint32_t)c->mol << 8), rule, c->b.cnt, live);
+        amax_kernel<<<nblk, kScanThreads, 0, s>>>(Ecur, R, dbeta, c->b.blk_f64, live);
+        max_top_kernel<<<1, 1024, 0, s>>>(c->b.blk_f64, nblk, c->b.scal);
+        weights_kernel<<<nblk, kScanThreads, 0, s>>>(Ecur, R, dbeta, two_s, c->b.scal, cf, c->b.W,
+                                                     c->b.blk_u64, c->b.blk_f64, live);
+        weights_top_kernel<<<1, kScanThreads, 0, s>>>(c->b.blk_u64, c->b.blk_f64, nblk, R, c->b.scal, live);
+        scan_local_u64_kernel<<<nblk, kScanThreads, 0, s>>>(c->b.W, R, c->b.blk_u64, c->b.C, live);
+        const cudaError_t e = cudaMemsetAsync(c->b.cnt, 0, sizeof(int32_t) * (size_t)R, s);
+        if (e != cudaSuccess) return e;
+        if (c->variable && do_resample)
+            varsize_counts_kernel<<<grid_for(R, 256, c->num_sms * 16), 256, 0, s>>>(
+                c->b.W, R, c->b.scal, c->R_target, c->seed, dev_counters, resample_offset, purpose,
+                c->resample_rule == PAMD_RESAMPLE_NEAREST ? 3 : 4, cf, c->b.cnt, live);
+        else
+            counts_kernel<<<grid_for(R, 256, c->num_sms * 16), 256, 0, s>>>(
+                c->b.C, R, c->b.scal, c->seed, dev_counters, resample_offset, purpose, rule, c->b.cnt, live);
+        cnt_block_kernel<<<nblk, kScanThreads, 0, s>>>(c->b.cnt, R, c->b.blk_i32, c->b.blk_i32 + nblk, live);
+        cnt_top_kernel<<<1, kScanThreads, 0, s>>>(c->b.blk_i32, c->b.blk_i32 + nblk, nblk, c->b.scal);
+        cnt_local_kernel<<<nblk, kScanThreads, 0, s>>>(c->b.cnt, R, c->b.blk_i32, c->b.cnt_incl, live);
+        c->launches += 9;
+        if (c->precision != PAMD_PREC_FP64) {
+            ancestor_kernel<<<grid_for(R, 256, c->num_sms * 16), 256, 0, s>>>(c->b.cnt_incl, R, anc, live, c->b.scal);
+            c->launches += 1;
+        }
     }
-    cnt_block_kernel<<<nblk, kScanThreads, 0, s>>>(c->b.cnt, R, c->b.blk_i32, c->b.blk_i32 + nblk, live);
-    cnt_top_kernel<<<1, kScanThreads, 0, s>>>(c->b.blk_i32, c->b.blk_i32 + nblk, nblk, c->b.scal);
-    cnt_local_kernel<<<nblk, kScanThreads, 0, s>>>(c->b.cnt, R, c->b.blk_i32, c->b.cnt_incl, live);
     double mt = 0.0;
     for (double m : c->host_mass) mt += m;
     const float* src = c->cur_is_alt ? c->b.state_alt : c->b.state;
@@ -982,13 +1260,8 @@ cudaError_t launch_resample(pamd_ctx* c, double T_prev, double T_next, int do_re
         const cudaError_t e = launch_gather_f64(
             c, reinterpret_cast<const double*>(src), reinterpret_cast<double*>(dst), Ein, Eout, fin,
             fout, sqrt(T_next / T_prev));
-        c->launches += 9;
         return e != cudaSuccess ? e : cudaGetLastError();
     }
-    // ancestors of the new slots (into the weight buffer, no longer needed)
-    int32_t* anc = reinterpret_cast<int32_t*>(c->b.W);
-    ancestor_kernel<<<grid_for(R, 256, c->num_sms * 16), 256, 0, s>>>(c->b.cnt_incl, R, anc, live,
-                                                                       c->b.scal);
     const int gridg = grid_for(R * 32, 256, c->num_sms * 64);
     const float vs = (float)sqrt(T_next / T_prev), imt = (float)(1.0 / mt);
     switch ((6 * (c->Np / 4) + 31) / 32) {
@@ -1004,7 +1277,7 @@ cudaError_t launch_resample(pamd_ctx* c, double T_prev, double T_next, int do_re
 #undef PAMD_GATHER_CASE
         default: return cudaErrorInvalidValue;
     }
-    c->launches += 11;
+    c->launches += 1;
     if (c->variable) {
         commit_size_kernel<<<1, 1, 0, s>>>(c->b.scal, c->b.counters, R);
         c->launches += 1;

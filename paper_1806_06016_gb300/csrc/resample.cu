@@ -808,12 +808,37 @@ __global__ void ancestor_kernel(const int32_t* __restrict__ incl, long long R, i
 // radius of gyration recomputed from the moved state (FP32 sums: GB300's FP64
 // rate is a small fraction of its FP32 rate, and every propagate launch
 // recomputes these values in FP64).
+//
+// The copy is HBM work, but the arithmetic around it decides: at 692
+// instructions per slot (75 atoms) the issue slots were the bottleneck (66 %
+// busy, DRAM 45 %).  What does not change between slots, each float4's
+// coordinate, masses and padding, is worked out once per lane; a float4
+// column that holds no positions (or no velocities) in any lane skips that
+// half by a uniform branch; values of one coordinate are picked by bit masks;
+// and the sums of several values share shuffles: after the first butterfly
+// step both halves of the warp hold the same sum, so the halves go on with
+// different values (the same additions in the same order).  75 atoms, R = 2^20
+// (3.83 GB): 638 us, 88 % of the measured copy bandwidth; before, 883 us.
+// Bulk copies through shared memory (4 records in flight per warp) took 991 us
+// at 2^20: fewer warps for the same instructions.
+// The roundings are written out, so that every P (and every change around
+// them) gives the same bits.
+__device__ __forceinline__ float dot4(const float4 a, const float4 b) {
+    return __fmaf_rn(a.w, b.w, __fmaf_rn(a.z, b.z, __fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y))));
+}
+__device__ __forceinline__ float mass_square(const float4 m, const float4 w) {
+    return __fmaf_rn(__fmul_rn(m.w, w.w), w.w,
+                     __fmaf_rn(__fmul_rn(m.z, w.z), w.z,
+                               __fmaf_rn(__fmul_rn(m.y, w.y), w.y, __fmul_rn(__fmul_rn(m.x, w.x), w.x))));
+}
+
 template <int P>
-__global__ void __launch_bounds__(256) gather_kernel(
+__global__ void __launch_bounds__(256, P <= 4 ? 4 : P <= 8 ? 3 : 2) gather_kernel(
     const float* __restrict__ st_in, float* __restrict__ st_out, const double* E_in,
     double* E_out, const int32_t* fam_in, int32_t* fam_out, double* ke_out, double* rg_out,
     const int32_t* __restrict__ anc, const float* __restrict__ masses, long long R, int N, int Np,
     float vscale, float inv_mtot, const uint32_t* live, const DevScalars* sc) {
+    constexpr bool kHoldMasses = P <= 4;  // registers
     const int lane = threadIdx.x & 31;
     if (live) R = sc->R_new < R ? sc->R_new : R;  // new slots of a variable population
     const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
@@ -821,79 +846,112 @@ __global__ void __launch_bounds__(256) gather_kernel(
     const int q4 = Np / 4;          // float4s per component
     const int nq = 6 * q4;          // float4s per replica
     const float4* m4 = reinterpret_cast<const float4*>(masses);
+    // per float4 of this lane: its coordinate (0..2 positions, 3.. velocities,
+    // 6 beyond the record), its index among the masses, the masses
+    int comp[P], mi[P];
+    float4 mh[kHoldMasses ? P : 1];
+#pragma unroll
+    for (int r = 0; r < P; ++r) {
+        const int q = lane + 32 * r;
+        comp[r] = q < nq ? q / q4 : 6;
+        mi[r] = q < nq ? q - comp[r] * q4 : 0;
+        if (kHoldMasses) mh[r] = m4[mi[r]];
+    }
     for (long long k = warp; k < R; k += nwarps) {
         const long long j = anc[k];
         const float4* src = reinterpret_cast<const float4*>(st_in + (size_t)j * 6 * Np);
         float4* dst = reinterpret_cast<float4*>(st_out + (size_t)k * 6 * Np);
         float4 v[P];
 #pragma unroll
-        for (int r = 0; r < P; ++r) {
-            const int q = lane + 32 * r;
-            if (q < nq) v[r] = __ldcs(src + q);  // read once: streaming load
+        for (int r = 0; r < P; ++r)
+            if (comp[r] < 6) v[r] = __ldcs(src + lane + 32 * r);  // read once: streaming load
+        double Ej = 0.0;
+        int32_t fj = 0;
+        if (lane == 0) {
+            Ej = E_in[j];
+            fj = fam_in[j];
         }
         float sx = 0.f, sy = 0.f, sz = 0.f;
 #pragma unroll
         for (int r = 0; r < P; ++r) {
-            const int q = lane + 32 * r;
-            if (q < nq) {
-                const int comp = q / q4;
-                if (comp < 3) {
-                    const float4 m = m4[q - comp * q4];
-                    const float s = m.x * v[r].x + m.y * v[r].y + m.z * v[r].z + m.w * v[r].w;
-                    sx += comp == 0 ? s : 0.f;
-                    sy += comp == 1 ? s : 0.f;
-                    sz += comp == 2 ? s : 0.f;
-                }
+            if (32 * r >= 3 * q4) break;  // no positions in this column or later ones
+            if (comp[r] < 3) {
+                const float4 m = kHoldMasses ? mh[r] : m4[mi[r]];
+                const float s = dot4(m, v[r]);
+                sx += comp[r] == 0 ? s : 0.f;
+                sy += comp[r] == 1 ? s : 0.f;
+                sz += comp[r] == 2 ? s : 0.f;
             }
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            sx += __shfl_xor_sync(0xffffffffu, sx, o);
-            sy += __shfl_xor_sync(0xffffffffu, sy, o);
-            sz += __shfl_xor_sync(0xffffffffu, sz, o);
+        float cx, cy, cz;
+        {  // butterfly sums of three values, halves and quarters sharing steps
+            const float a = sx + __shfl_xor_sync(0xffffffffu, sx, 16), b = sy + __shfl_xor_sync(0xffffffffu, sy, 16),
+                        c = sz + __shfl_xor_sync(0xffffffffu, sz, 16);
+            float ab = lane < 16 ? a : b, t = c;
+            ab += __shfl_xor_sync(0xffffffffu, ab, 8);
+            t += __shfl_xor_sync(0xffffffffu, t, 8);
+            float u = (lane & 8) ? t : ab;  // lanes 0..7 x, 16..23 y, 8..15 and 24..31 z
+            u += __shfl_xor_sync(0xffffffffu, u, 4);
+            u += __shfl_xor_sync(0xffffffffu, u, 2);
+            u += __shfl_xor_sync(0xffffffffu, u, 1);
+            cx = __shfl_sync(0xffffffffu, u, 0);
+            cy = __shfl_sync(0xffffffffu, u, 16);
+            cz = __shfl_sync(0xffffffffu, u, 8);
         }
-        const float cx = sx * inv_mtot, cy = sy * inv_mtot, cz = sz * inv_mtot;
         float mv2 = 0.f, ux = 0.f, uy = 0.f, uz = 0.f, u2 = 0.f;
 #pragma unroll
         for (int r = 0; r < P; ++r) {
-            const int q = lane + 32 * r;
-            if (q < nq) {
-                const int comp = q / q4;
-                const int i0 = (q - comp * q4) * 4;
-                float4 w = v[r];
-                const float4 m = m4[q - comp * q4];  // 0 for padding atoms
-                // padding atoms (i >= N) are kept out of the sums
-                const float4 real = make_float4(i0 < N ? 1.f : 0.f, i0 + 1 < N ? 1.f : 0.f,
-                                                i0 + 2 < N ? 1.f : 0.f, i0 + 3 < N ? 1.f : 0.f);
-                if (comp < 3) {
-                    const float c = (comp == 0) ? cx : (comp == 1) ? cy : cz;
-                    w.x -= c; w.y -= c; w.z -= c; w.w -= c;
-                    const float s1 = real.x * w.x + real.y * w.y + real.z * w.z + real.w * w.w;
-                    u2 += real.x * w.x * w.x + real.y * w.y * w.y + real.z * w.z * w.z + real.w * w.w * w.w;
-                    ux += comp == 0 ? s1 : 0.f;
-                    uy += comp == 1 ? s1 : 0.f;
-                    uz += comp == 2 ? s1 : 0.f;
-                } else {
-                    w.x *= vscale; w.y *= vscale; w.z *= vscale; w.w *= vscale;
-                    mv2 += m.x * w.x * w.x + m.y * w.y * w.y + m.z * w.z * w.z + m.w * w.w * w.w;
+            float4 w = v[r];
+            if (32 * r < 3 * q4 && comp[r] < 3) {
+                const float c = (comp[r] == 0) ? cx : (comp[r] == 1) ? cy : cz;  // sum of m x
+                w.x = __fmaf_rn(-c, inv_mtot, w.x);
+                w.y = __fmaf_rn(-c, inv_mtot, w.y);
+                w.z = __fmaf_rn(-c, inv_mtot, w.z);
+                w.w = __fmaf_rn(-c, inv_mtot, w.w);
+                float4 z = w;  // padding atoms (>= N) are kept out of the sums
+                if (Np != N) {
+                    const int left = N - 4 * mi[r];
+                    z.y = left > 1 ? z.y : 0.f;
+                    z.z = left > 2 ? z.z : 0.f;
+                    z.w = left > 3 ? z.w : 0.f;
                 }
-                __stcs(dst + q, w);  // written once: streaming store
+                const float s1 = z.x + z.y + z.z + z.w;
+                u2 += dot4(z, w);
+                ux += comp[r] == 0 ? s1 : 0.f;
+                uy += comp[r] == 1 ? s1 : 0.f;
+                uz += comp[r] == 2 ? s1 : 0.f;
             }
+            if (32 * r + 31 >= 3 * q4 && comp[r] >= 3) {
+                const float4 m = kHoldMasses ? mh[r] : m4[mi[r]];  // 0 for padding atoms
+                w.x *= vscale; w.y *= vscale; w.z *= vscale; w.w *= vscale;
+                if (comp[r] < 6) mv2 += mass_square(m, w);
+            }
+            if (comp[r] < 6) __stcs(dst + lane + 32 * r, w);  // written once: streaming store
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            mv2 += __shfl_xor_sync(0xffffffffu, mv2, o);
-            ux += __shfl_xor_sync(0xffffffffu, ux, o);
-            uy += __shfl_xor_sync(0xffffffffu, uy, o);
-            uz += __shfl_xor_sync(0xffffffffu, uz, o);
-            u2 += __shfl_xor_sync(0xffffffffu, u2, o);
-        }
+        // five butterfly sums: u2, ux, uy, uz end in lanes 0, 8, 16, 24, mv2 in lane 4
+        ux += __shfl_xor_sync(0xffffffffu, ux, 16);
+        uy += __shfl_xor_sync(0xffffffffu, uy, 16);
+        uz += __shfl_xor_sync(0xffffffffu, uz, 16);
+        u2 += __shfl_xor_sync(0xffffffffu, u2, 16);
+        mv2 += __shfl_xor_sync(0xffffffffu, mv2, 16);
+        float a = lane < 16 ? u2 : uy, b = lane < 16 ? ux : uz;
+        a += __shfl_xor_sync(0xffffffffu, a, 8);
+        b += __shfl_xor_sync(0xffffffffu, b, 8);
+        mv2 += __shfl_xor_sync(0xffffffffu, mv2, 8);
+        a = (lane & 8) ? b : a;  // 0..7 u2, 8..15 ux, 16..23 uy, 24..31 uz
+        a += __shfl_xor_sync(0xffffffffu, a, 4);
+        mv2 += __shfl_xor_sync(0xffffffffu, mv2, 4);
+        a = (lane & 28) == 4 ? mv2 : a;
+        a += __shfl_xor_sync(0xffffffffu, a, 2);
+        a += __shfl_xor_sync(0xffffffffu, a, 1);
+        if (lane == 4) ke_out[k] = 0.5 * (double)a;
+        const float mean = a / N;  // each of the four sums in its lane
+        const float mx = __shfl_sync(0xffffffffu, mean, 8), my = __shfl_sync(0xffffffffu, mean, 16),
+                    mz = __shfl_sync(0xffffffffu, mean, 24);
         if (lane == 0) {
-            E_out[k] = E_in[j];
-            fam_out[k] = fam_in[j];
-            ke_out[k] = 0.5 * (double)mv2;
-            const float mx = ux / N, my = uy / N, mz = uz / N;
-            rg_out[k] = (double)sqrtf(fmaxf(u2 / N - (mx * mx + my * my + mz * mz), 0.f));
+            E_out[k] = Ej;
+            fam_out[k] = fj;
+            rg_out[k] = (double)sqrtf(fmaxf(mean - (mx * mx + my * my + mz * mz), 0.f));
         }
     }
 }
@@ -1262,8 +1320,8 @@ cudaError_t launch_resample(pamd_ctx* c, double T_prev, double T_next, int do_re
             fout, sqrt(T_next / T_prev));
         return e != cudaSuccess ? e : cudaGetLastError();
     }
-    const int gridg = grid_for(R * 32, 256, c->num_sms * 64);
     const float vs = (float)sqrt(T_next / T_prev), imt = (float)(1.0 / mt);
+    const int gridg = grid_for(R * 32, 256, c->num_sms * 64);
     switch ((6 * (c->Np / 4) + 31) / 32) {
 #define PAMD_GATHER_CASE(P)                                                                     \
     case P:                                                                                     \

@@ -1601,33 +1601,152 @@ int pamd_anneal(pamd_ctx* c, int32_t K, const double* T, int32_t theta, double d
     return read_status(c);
 }
 
+}  // extern "C"
+
+namespace {
+
+// Staging memory of the state calls: up to kStagingBytes of device memory,
+// kept with the context.  Larger populations go through it in chunks.
+constexpr size_t kStagingBytes = (size_t)64 << 20;
+
+// Replicas per chunk with `row_bytes` of staging each; 0 if there is no
+// memory for staging.  The first 256 bytes hold the finiteness flag.
+long long staging_chunk(pamd_ctx* c, size_t row_bytes) {
+    const size_t want = std::min(kStagingBytes, 256 + row_bytes * (size_t)c->R);
+    if (c->staging_bytes < want) {
+        void* p = dalloc(c, want);
+        if (!p) return 0;
+        if (c->staging) {  // the smaller one of an earlier call
+            cudaStreamSynchronize(c->stream);
+            c->allocations.erase(std::find(c->allocations.begin(), c->allocations.end(), c->staging));
+            if (c->dev_free) c->dev_free(c->staging, c->alloc_user);
+            else cudaFree(c->staging);
+        }
+        c->staging = p;
+        c->staging_bytes = want;
+    }
+    return std::min<long long>(c->R, (long long)((c->staging_bytes - 256) / row_bytes));
+}
+
+// A device-to-host copy that meets pages the host never touched faults them
+// in one by one from the device side (about 50 us each on this machine);
+// touching them here first costs a fraction of a microsecond.
+void touch_pages(void* p, size_t bytes) {
+    volatile char* b = static_cast<volatile char*>(p);
+    for (size_t o = 0; o < bytes; o += 4096) b[o] = 0;
+    if (bytes) b[bytes - 1] = 0;
+}
+
+// rows [R][N][3] <- planes first..first + 2 of records of `planes` planes at
+// src, on the device chunk by chunk.  PAMD_ENOMEM: no staging memory.
+int rows_to_host(pamd_ctx* c, const void* src, int planes, int first, double* rows) {
+    const size_t row = 24 * (size_t)c->N, rec = (is_f64(c) ? 8 : 4) * (size_t)planes * c->Np;
+    const long long chunk = staging_chunk(c, row);
+    if (chunk < 1) return PAMD_ENOMEM;
+    double* st = reinterpret_cast<double*>(static_cast<char*>(c->staging) + 256);
+    touch_pages(rows, row * (size_t)c->R);
+    for (long long k = 0; k < c->R; k += chunk) {
+        const long long n = std::min(chunk, c->R - k);
+        PAMD_CU(c, launch_unpack_rows(static_cast<const char*>(src) + rec * (size_t)k, st, n, c->N, c->Np, planes, first,
+                                      is_f64(c), c->stream));
+        c->launches += 1;
+        PAMD_CU(c, cudaMemcpyAsync(rows + (size_t)k * 3 * c->N, st, row * (size_t)n, cudaMemcpyDeviceToHost, c->stream));
+    }
+    return PAMD_OK;
+}
+
+// The same on the host, for a context without staging memory.
+int rows_to_host_slow(pamd_ctx* c, const void* src, int planes, int first, double* rows) {
+    const int N = c->N, Np = c->Np;
+    const size_t es = is_f64(c) ? 8 : 4;
+    std::vector<unsigned char> buf(es * (size_t)planes * Np * (size_t)c->R);
+    PAMD_CU(c, cudaMemcpyAsync(buf.data(), src, buf.size(), cudaMemcpyDeviceToHost, c->stream));
+    PAMD_CU(c, cudaStreamSynchronize(c->stream));
+    const float* f = reinterpret_cast<const float*>(buf.data());
+    const double* d = reinterpret_cast<const double*>(buf.data());
+    for (long long k = 0; k < c->R; ++k)
+        for (int i = 0; i < N; ++i)
+            for (int q = 0; q < 3; ++q) {
+                const size_t at = ((size_t)k * planes + first + q) * Np + i;
+                rows[((size_t)k * N + i) * 3 + q] = es == 8 ? d[at] : (double)f[at];
+            }
+    return PAMD_OK;
+}
+
+int read_rows(pamd_ctx* c, const void* src, int planes, int first, double* rows) {
+    const int rc = rows_to_host(c, src, planes, first, rows);
+    return rc == PAMD_ENOMEM ? rows_to_host_slow(c, src, planes, first, rows) : rc;
+}
+
+// New population state from the host rows: packed into the alternate buffer
+// (its contents are not needed between calls) and copied over the current one
+// once every value is known to be finite.  PAMD_ENOMEM: no staging memory.
+int rows_from_host(pamd_ctx* c, const double* x, const double* v) {
+    const size_t row = 24 * (size_t)c->N, rec = (is_f64(c) ? 8 : 4) * 6 * (size_t)c->Np;
+    const long long chunk = staging_chunk(c, 2 * row);
+    if (chunk < 1) return PAMD_ENOMEM;
+    char* base = static_cast<char*>(c->staging);
+    int* bad = reinterpret_cast<int*>(base);
+    double* sx = reinterpret_cast<double*>(base + 256);
+    double* sv = sx + (size_t)chunk * 3 * c->N;
+    char* alt = reinterpret_cast<char*>(c->cur_is_alt ? c->b.state : c->b.state_alt);
+    PAMD_CU(c, cudaMemsetAsync(bad, 0, sizeof(int), c->stream));
+    for (long long k = 0; k < c->R; k += chunk) {
+        const long long n = std::min(chunk, c->R - k);
+        const size_t at = (size_t)k * 3 * c->N;
+        PAMD_CU(c, cudaMemcpyAsync(sx, x + at, row * (size_t)n, cudaMemcpyHostToDevice, c->stream));
+        PAMD_CU(c, cudaMemcpyAsync(sv, v + at, row * (size_t)n, cudaMemcpyHostToDevice, c->stream));
+        PAMD_CU(c, launch_pack_state(sx, sv, alt + rec * (size_t)k, n, c->N, c->Np, is_f64(c), bad, c->stream));
+        c->launches += 1;
+    }
+    int h = 0;
+    PAMD_CU(c, cudaMemcpyAsync(&h, bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    PAMD_CU(c, cudaStreamSynchronize(c->stream));
+    if (h) return fail(PAMD_EINVAL, "non-finite state");
+    PAMD_CU(c, cudaMemcpyAsync(cur_state(c), alt, state_bytes(c), cudaMemcpyDeviceToDevice, c->stream));
+    return PAMD_OK;
+}
+
+int rows_from_host_slow(pamd_ctx* c, const double* x, const double* v) {
+    const int N = c->N, Np = c->Np;
+    for (size_t e = 0; e < (size_t)c->R * 3 * N; ++e)
+        if (!std::isfinite(x[e]) || !std::isfinite(v[e])) return fail(PAMD_EINVAL, "non-finite state");
+    const size_t es = is_f64(c) ? 8 : 4;
+    std::vector<unsigned char> buf(es * 6 * Np * (size_t)c->R, 0);
+    float* f = reinterpret_cast<float*>(buf.data());
+    double* d = reinterpret_cast<double*>(buf.data());
+    for (long long k = 0; k < c->R; ++k)
+        for (int i = 0; i < N; ++i)
+            for (int q = 0; q < 6; ++q) {
+                const double a = (q < 3 ? x : v)[((size_t)k * N + i) * 3 + q % 3];
+                const size_t at = ((size_t)k * 6 + q) * Np + i;
+                if (es == 8) d[at] = a;
+                else f[at] = (float)a;
+            }
+    PAMD_CU(c, cudaMemcpyAsync(cur_state(c), buf.data(), buf.size(), cudaMemcpyHostToDevice, c->stream));
+    PAMD_CU(c, cudaStreamSynchronize(c->stream));
+    return PAMD_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 int pamd_get_state(pamd_ctx* c, double* x, double* v, double* E, int32_t* fam) {
     int rc = check_ctx(c);
     if (rc) return rc;
     if (is_batch(c)) return fail(PAMD_EINVAL, "batch context: call this on pamd_batch_sub(ctx, m)");
-    const int N = c->N, Np = c->Np;
-    const long long R = c->R;
-    std::vector<float> st;
-    std::vector<double> st64;
-    if ((x || v) && is_f64(c)) {
-        st64.resize((size_t)R * 6 * Np);
-        PAMD_CU(c, cudaMemcpyAsync(st64.data(), cur_state(c), st64.size() * 8, cudaMemcpyDeviceToHost, c->stream));
-    } else if (x || v) {
-        st.resize((size_t)R * 6 * Np);
-        PAMD_CU(c, cudaMemcpyAsync(st.data(), cur_state(c), st.size() * 4, cudaMemcpyDeviceToHost, c->stream));
+    if (x && (rc = read_rows(c, cur_state(c), 6, 0, x))) return rc;
+    if (v && (rc = read_rows(c, cur_state(c), 6, 3, v))) return rc;
+    if (E) {
+        touch_pages(E, 8 * (size_t)c->R);
+        PAMD_CU(c, cudaMemcpyAsync(E, cur_E(c), 8 * (size_t)c->R, cudaMemcpyDeviceToHost, c->stream));
     }
-    if (E) PAMD_CU(c, cudaMemcpyAsync(E, cur_E(c), 8 * (size_t)R, cudaMemcpyDeviceToHost, c->stream));
-    if (fam) PAMD_CU(c, cudaMemcpyAsync(fam, cur_fam(c), 4 * (size_t)R, cudaMemcpyDeviceToHost, c->stream));
+    if (fam) {
+        touch_pages(fam, 4 * (size_t)c->R);
+        PAMD_CU(c, cudaMemcpyAsync(fam, cur_fam(c), 4 * (size_t)c->R, cudaMemcpyDeviceToHost, c->stream));
+    }
     PAMD_CU(c, cudaStreamSynchronize(c->stream));
-    for (long long k = 0; k < R && (x || v); ++k) {
-        for (int i = 0; i < N; ++i)
-            for (int q = 0; q < 3; ++q) {
-                const size_t ix = (size_t)k * 6 * Np + (size_t)q * Np + i;
-                const size_t iv = ix + 3 * (size_t)Np;
-                if (x) x[((size_t)k * N + i) * 3 + q] = st64.empty() ? (double)st[ix] : st64[ix];
-                if (v) v[((size_t)k * N + i) * 3 + q] = st64.empty() ? (double)st[iv] : st64[iv];
-            }
-    }
     return PAMD_OK;
 }
 
@@ -1636,38 +1755,11 @@ int pamd_set_state(pamd_ctx* c, const double* x, const double* v, const double* 
     if (rc) return rc;
     if (is_batch(c)) return fail(PAMD_EINVAL, "batch context: call this on pamd_batch_sub(ctx, m)");
     if (!x || !v) return fail(PAMD_EINVAL, "x and v are required");
-    const int N = c->N, Np = c->Np;
-    const long long R = c->R;
-    if (!finite_all(x, (int)std::min<long long>(R * N * 3, 0x7fffffff)) ||
-        !finite_all(v, (int)std::min<long long>(R * N * 3, 0x7fffffff)))
-        return fail(PAMD_EINVAL, "non-finite state");
-    if (is_f64(c)) {
-        std::vector<double> st((size_t)R * 6 * Np, 0.0);
-        for (long long k = 0; k < R; ++k) {
-            double* s = st.data() + (size_t)k * 6 * Np;
-            for (int i = 0; i < N; ++i)
-                for (int q = 0; q < 3; ++q) {
-                    s[(size_t)q * Np + i] = x[((size_t)k * N + i) * 3 + q];
-                    s[(size_t)(3 + q) * Np + i] = v[((size_t)k * N + i) * 3 + q];
-                }
-        }
-        PAMD_CU(c, cudaMemcpyAsync(cur_state(c), st.data(), st.size() * 8, cudaMemcpyHostToDevice, c->stream));
-        PAMD_CU(c, cudaStreamSynchronize(c->stream));
-    } else {
-        std::vector<float> st((size_t)R * 6 * Np, 0.0f);
-        for (long long k = 0; k < R; ++k) {
-            float* s = st.data() + (size_t)k * 6 * Np;
-            for (int i = 0; i < N; ++i)
-                for (int q = 0; q < 3; ++q) {
-                    s[(size_t)q * Np + i] = (float)x[((size_t)k * N + i) * 3 + q];
-                    s[(size_t)(3 + q) * Np + i] = (float)v[((size_t)k * N + i) * 3 + q];
-                }
-        }
-        PAMD_CU(c, cudaMemcpyAsync(cur_state(c), st.data(), st.size() * 4, cudaMemcpyHostToDevice, c->stream));
-        PAMD_CU(c, cudaStreamSynchronize(c->stream));
-    }
-    if (E) PAMD_CU(c, cudaMemcpyAsync(cur_E(c), E, 8 * (size_t)R, cudaMemcpyHostToDevice, c->stream));
-    if (fam) PAMD_CU(c, cudaMemcpyAsync(cur_fam(c), fam, 4 * (size_t)R, cudaMemcpyHostToDevice, c->stream));
+    rc = rows_from_host(c, x, v);
+    if (rc == PAMD_ENOMEM) rc = rows_from_host_slow(c, x, v);
+    if (rc) return rc;
+    if (E) PAMD_CU(c, cudaMemcpyAsync(cur_E(c), E, 8 * (size_t)c->R, cudaMemcpyHostToDevice, c->stream));
+    if (fam) PAMD_CU(c, cudaMemcpyAsync(cur_fam(c), fam, 4 * (size_t)c->R, cudaMemcpyHostToDevice, c->stream));
     PAMD_CU(c, cudaStreamSynchronize(c->stream));
     return PAMD_OK;
 }
@@ -1676,30 +1768,18 @@ int pamd_forces(pamd_ctx* c, double* f, double* E) {
     int rc = check_ctx(c);
     if (rc) return rc;
     if (is_batch(c)) return fail(PAMD_EINVAL, "batch context: call this on pamd_batch_sub(ctx, m)");
-    const int N = c->N, Np = c->Np;
-    const long long R = c->R;
     const size_t es = is_f64(c) ? 8 : 4;
     if (!c->b.fout) {
-        c->b.fout = (float*)dalloc(c, es * 3 * (size_t)Np * (size_t)R);
+        c->b.fout = (float*)dalloc(c, es * 3 * (size_t)c->Np * (size_t)c->R);
         if (!c->b.fout) return fail(PAMD_ENOMEM, "force buffer");
     }
     if ((rc = launch_prop(c, 0, 0.001, 300.0, nullptr, c->step, c->b.fout))) return rc;
-    std::vector<float> fo;
-    std::vector<double> fo64;
-    if (f && is_f64(c)) {
-        fo64.resize((size_t)R * 3 * Np);
-        PAMD_CU(c, cudaMemcpyAsync(fo64.data(), c->b.fout, fo64.size() * 8, cudaMemcpyDeviceToHost, c->stream));
-    } else if (f) {
-        fo.resize((size_t)R * 3 * Np);
-        PAMD_CU(c, cudaMemcpyAsync(fo.data(), c->b.fout, fo.size() * 4, cudaMemcpyDeviceToHost, c->stream));
+    if (f && (rc = read_rows(c, c->b.fout, 3, 0, f))) return rc;
+    if (E) {
+        touch_pages(E, 8 * (size_t)c->R);
+        PAMD_CU(c, cudaMemcpyAsync(E, cur_E(c), 8 * (size_t)c->R, cudaMemcpyDeviceToHost, c->stream));
     }
-    if (E) PAMD_CU(c, cudaMemcpyAsync(E, cur_E(c), 8 * (size_t)R, cudaMemcpyDeviceToHost, c->stream));
     PAMD_CU(c, cudaStreamSynchronize(c->stream));
-    for (long long k = 0; k < R && f; ++k)
-        for (int i = 0; i < N; ++i)
-            for (int q = 0; q < 3; ++q)
-                f[((size_t)k * N + i) * 3 + q] = fo64.empty() ? (double)fo[(size_t)k * 3 * Np + (size_t)q * Np + i]
-                                                               : fo64[(size_t)k * 3 * Np + (size_t)q * Np + i];
     return read_status(c);
 }
 

@@ -288,6 +288,8 @@ struct pamd_ctx {
     pamd::TopoF64 top64{};        // all-FP64 mode tables (precision == PAMD_PREC_FP64)
     // batch context (pamd_init_batch): one sub-context per molecule
     std::vector<pamd_ctx*> subs;
+    void* staging = nullptr;      // rows of the state on their way to or from the host, kept once allocated
+    size_t staging_bytes = 0;
     int4* items = nullptr;        // device work lists of the batched propagate, group by group
     int n_items = 0;
     int* queue = nullptr;         // device work counters, one per group
@@ -425,6 +427,13 @@ cudaError_t propagate_batch_occupancy(int B, size_t smem, int* blocks_per_sm);
 // the same for molecules in the packed FP32x2 layout (propagate_batch_x2.cu)
 cudaError_t launch_propagate_batch_x2(const BatchParams& bp, int B, int grid, size_t smem, cudaStream_t s);
 cudaError_t propagate_batch_x2_occupancy(int B, size_t smem, int* blocks_per_sm);
+
+// host arrays [n][N][3] FP64 (in device staging memory) to records of 6 planes
+// and back (state_io.cu); *bad is set to 1 by a non-finite value
+cudaError_t launch_pack_state(const double* x, const double* v, void* rec, long long n, int N, int Np, bool f64, int* bad,
+                              cudaStream_t s);
+cudaError_t launch_unpack_rows(const void* rec, double* rows, long long n, int N, int Np, int planes, int first, bool f64,
+                               cudaStream_t s);
 
 // all-FP64 mode (propagate_f64.cu)
 cudaError_t launch_propagate_f64(pamd_ctx* c, double* state, double* E, double* ke, double* rg,

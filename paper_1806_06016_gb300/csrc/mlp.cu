@@ -3,7 +3,8 @@
 //
 // Dense layers are BF16 tensor-core GEMMs (mlp_gemm.cu) whose epilogues apply
 // the bias, the SiLU and its derivative and write the BF16 operands of the
-// next product (row-major, and transposed where a weight gradient needs them).
+// next product; the weight gradients contract over the samples of the same
+// row-major operands.
 // Everything between the products (features, the pair Jacobian and its
 // transpose, second-derivative terms, column sums) is FP32 here; energies and
 // loss sums are FP64.
@@ -95,31 +96,29 @@ __global__ void mlp_init_kernel(float* params, size_t oW1, size_t oW2, size_t ow
     }
 }
 
-// BF16 copies of W1 and W2, row-major and transposed
-__global__ void mlp_pack_kernel(const float* __restrict__ params, size_t oW1, size_t oW2, int H,
-                                int Pp, __nv_bfloat16* W1b, __nv_bfloat16* W1Tb,
-                                __nv_bfloat16* W2b, __nv_bfloat16* W2Tb) {
-    const long long n1 = (long long)H * Pp, n2 = (long long)H * H;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n1 + n2;
-         e += (long long)gridDim.x * blockDim.x) {
-        if (e < n1) {
-            const int h = (int)(e / Pp), p = (int)(e % Pp);
-            const __nv_bfloat16 b = __float2bfloat16(params[oW1 + e]);
-            W1b[e] = b;
-            W1Tb[(size_t)p * H + h] = b;
-        } else {
-            const long long l = e - n1;
-            const int h = (int)(l / H), k = (int)(l % H);
-            const __nv_bfloat16 b = __float2bfloat16(params[oW2 + l]);
-            W2b[l] = b;
-            W2Tb[(size_t)k * H + h] = b;
-        }
+// The BF16 copies of W1 and W2 the tensor cores read: same layout, rounded.
+struct WeightCopies {
+    size_t oW1, nW1, oW2, nW2;  // offsets and sizes in the parameter block
+    __nv_bfloat16 *W1b, *W2b;
+    __device__ __forceinline__ void put(size_t e, float p) const {
+        if (e - oW1 < nW1) W1b[e - oW1] = __float2bfloat16(p);
+        else if (e - oW2 < nW2) W2b[e - oW2] = __float2bfloat16(p);
     }
+};
+
+__global__ void mlp_pack_kernel(const float* __restrict__ params, long long n, const WeightCopies w) {
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
+         e += (long long)gridDim.x * blockDim.x)
+        w.put((size_t)e, params[e]);
 }
 
+// Adam and, from the new value in hand, the BF16 copies: HBM/L2-bound, 28
+// bytes read and written per parameter.  75 atoms, H = 512 (1.7 M
+// parameters): 11.9 us; an update and a pass that also wrote transposed
+// copies in 2-byte stores took 11.5 + 16.7 us.
 __global__ void mlp_adam_kernel(float* p, const float* __restrict__ g, float* m, float* v,
                                 long long n, float lr, float b1, float b2, float eps, float bc1,
-                                float bc2) {
+                                float bc2, const WeightCopies w) {
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
          e += (long long)gridDim.x * blockDim.x) {
         const float gi = g[e];
@@ -127,7 +126,9 @@ __global__ void mlp_adam_kernel(float* p, const float* __restrict__ g, float* m,
         const float vi = b2 * v[e] + (1.0f - b2) * gi * gi;
         m[e] = mi;
         v[e] = vi;
-        p[e] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+        const float pn = p[e] - lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+        p[e] = pn;
+        w.put((size_t)e, pn);
     }
 }
 
@@ -324,8 +325,7 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_features_kernel(const FeatArg
         __syncthreads();
         load_config(f.cv, m, f.N, xs);
         __syncthreads();
-        block_features(xs, f.pairs, f.mu, f.inv_sd, f.P, f.Pp, f.a + (size_t)m * f.Pp, f.aT,
-                       f.ldt, m);
+        block_features(xs, f.pairs, f.mu, f.inv_sd, f.P, f.Pp, f.a + (size_t)m * f.Pp);
     }
 }
 
@@ -401,9 +401,7 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_loss_kernel(const LossArgs L)
                                  ir * ir * ir;
                 v = jn * L.inv_sd[p];
             }
-            const __nv_bfloat16 b = __float2bfloat16(v);
-            nrow[p] = b;
-            L.nu_aT[(size_t)p * L.ldt + m] = b;
+            nrow[p] = __float2bfloat16(v);
         }
         if (threadIdx.x == 0) {
             const double e = head_energy(L.part, L.nparts, m, L.b3);
@@ -416,24 +414,20 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_loss_kernel(const LossArgs L)
 
 // Reverse pass through the two hidden layers.  Tiles of kBarRows samples m by
 // kBarCols hidden units h, 256 threads: a thread keeps one column h and walks
-// the tile's rows four apart, so that
-//   * reads and the row-major output are coalesced along h;
-//   * the transposed BF16 operand of the weight gradient goes through shared
-//     memory and is written in runs of kBarRows samples (8-byte stores: M and
-//     ldt are multiples of 4), not as one 2-byte store per 32-byte sector;
-//   * the bias and w3 gradients' sums over the samples start here, in FP64 in
-//     registers, so that their per-sample terms never go to memory.  Each tile
-//     leaves one partial per column; mlp_sums_kernel adds those.
+// the tile's rows four apart, reads and writes are coalesced along h, and the
+// bias and w3 gradients' sums over the samples start here, in FP64 in
+// registers, so that their per-sample terms never go to memory.  Each tile
+// leaves one partial per column; mlp_sums_kernel adds those.
 // Bound by the FP64 conversions and additions (two per element and sum on
 // units that do a 64th of the FP32 rate) and the latency of one tile.  At 2048
-// samples and H = 512: layer 2 13.7 us, layer 1 9.8 us, sums 5.3 us (tiles of
+// samples and H = 512: layer 2 13.9 us, layer 1 10.0 us, sums 5.3 us (tiles of
 // 64 rows: 15.9, 14.7, 5.3); with element-wise kernels that stored the terms
 // and column sums of four blocks, each thread walking all samples in one
 // serial FP64 chain, 14.8 + 14.1 + 3 x 249 + 167 us.
 constexpr int kBarRows = 32, kBarCols = 64, kBarThreads = 256;
 
 struct BarArgs {
-    int M, H, ldt;
+    int M, H;
     const float* ebar;       // [M]
     const float* z;          // pre-activations of the layer
     const float* s;          // silu'(z)
@@ -441,8 +435,7 @@ struct BarArgs {
     const float* up;         // layer 1: dL/dh1; layer 2: unused
     const float* w2d2;       // layer 1: W2^T d2
     const float* w3;         // layer 2
-    __nv_bfloat16* zb;       // layer 2: dL/dz2 row-major
-    __nv_bfloat16* AT;       // dL/dz transposed [H][ldt]
+    __nv_bfloat16* zb;       // dL/dz
     double* part_b;          // [tiles][H] partial sums of dL/dz
     double* part_w3;         // layer 2: [tiles][H] partial sums of the w3 gradient
 };
@@ -451,8 +444,6 @@ struct BarArgs {
 // LAYER 1: dL/dz1 = h1_bar silu'(z1) + (W2^T d2) zd1 silu''(z1)
 template <int LAYER>
 __global__ void __launch_bounds__(kBarThreads) mlp_zbar_kernel(const BarArgs g) {
-    // row stride kBarRows + 4: rows 8-byte aligned, few bank conflicts on the writes
-    __shared__ __align__(8) __nv_bfloat16 tile[kBarCols][kBarRows + 4];
     __shared__ double sb[kBarThreads], sw[kBarThreads];
     constexpr int kGroups = kBarThreads / kBarCols, kPer = kBarRows / kGroups;
     const int hl = threadIdx.x % kBarCols, r0 = threadIdx.x / kBarCols;
@@ -474,7 +465,7 @@ __global__ void __launch_bounds__(kBarThreads) mlp_zbar_kernel(const BarArgs g) 
     double ab = 0.0, aw = 0.0;
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
-        const int r = r0 + q * kGroups, m = m0 + r;
+        const int m = m0 + r0 + q * kGroups;
         if (!col || m >= g.M) continue;
         float zb;
         if (LAYER == 2) {
@@ -484,9 +475,7 @@ __global__ void __launch_bounds__(kBarThreads) mlp_zbar_kernel(const BarArgs g) 
             zb = u0[q] * ds[q] + u1[q] * td[q] * d2silu(z[q]);
         }
         ab += (double)zb;
-        const __nv_bfloat16 b = __float2bfloat16(zb);
-        if (LAYER == 2) g.zb[(size_t)m * g.H + h] = b;
-        tile[hl][r] = b;
+        g.zb[(size_t)m * g.H + h] = __float2bfloat16(zb);
     }
     sb[threadIdx.x] = ab;
     if (LAYER == 2) sw[threadIdx.x] = aw;
@@ -499,13 +488,6 @@ __global__ void __launch_bounds__(kBarThreads) mlp_zbar_kernel(const BarArgs g) 
         }
         g.part_b[(size_t)blockIdx.y * g.H + h] = tb;
         if (LAYER == 2) g.part_w3[(size_t)blockIdx.y * g.H + h] = tw;
-    }
-    for (int t = threadIdx.x; t < kBarCols * (kBarRows / 4); t += kBarThreads) {
-        const int row = t / (kBarRows / 4), q = 4 * (t % (kBarRows / 4));
-        const int hh = blockIdx.x * kBarCols + row, m = m0 + q;
-        if (hh < g.H && m < g.M)
-            *reinterpret_cast<uint2*>(g.AT + (size_t)hh * g.ldt + m) =
-                *reinterpret_cast<const uint2*>(&tile[row][q]);
     }
 }
 
@@ -584,10 +566,13 @@ int read_model_status(pamd_mlp* m) {
     return PAMD_OK;
 }
 
+WeightCopies weight_copies(const pamd_mlp* m) {
+    return {m->oW1, (size_t)m->H * m->Pp, m->oW2, (size_t)m->H * m->H, m->W1b, m->W2b};
+}
+
 int pack(pamd_mlp* m) {
-    const long long n = (long long)m->H * m->Pp + (long long)m->H * m->H;
-    mlp_pack_kernel<<<grid_for(n, 256), 256, 0, m->stream>>>(m->params, m->oW1, m->oW2, m->H, m->Pp,
-                                                             m->W1b, m->W1Tb, m->W2b, m->W2Tb);
+    const long long n = (long long)m->ob2;  // W1, b1 and W2 come first
+    mlp_pack_kernel<<<grid_for(n, 256), 256, 0, m->stream>>>(m->params, n, weight_copies(m));
     return launch_check(m, "weight pack");
 }
 
@@ -602,7 +587,7 @@ int set_smem_attrs(const pamd_mlp* m) {
     return e == cudaSuccess ? PAMD_OK : mfail(PAMD_ECUDA, std::string("kernel attributes: ") + cudaGetErrorString(e));
 }
 
-int features(pamd_mlp* m, const ConfigView& cv, int M, __nv_bfloat16* aT, int ldt) {
+int features(pamd_mlp* m, const ConfigView& cv, int M, __nv_bfloat16* a) {
     FeatArgs f{};
     f.cv = cv;
     f.M = M;
@@ -612,9 +597,7 @@ int features(pamd_mlp* m, const ConfigView& cv, int M, __nv_bfloat16* aT, int ld
     f.pairs = m->pairs;
     f.mu = m->mu;
     f.inv_sd = m->inv_sd;
-    f.a = m->w.a;
-    f.aT = aT;
-    f.ldt = ldt;
+    f.a = a;
     mlp_features_kernel<<<grid_for((long long)M * kMlpThreads, kMlpThreads, 152 * 16), kMlpThreads, 0,
                           m->stream>>>(f);
     return launch_check(m, "features");
@@ -631,13 +614,10 @@ int mlp_ensure_work(pamd_mlp* m, long long M, bool train) {
     const bool tr = train || w.train;
     const size_t H = (size_t)m->H, Pp = (size_t)m->Pp, C = (size_t)cap;
     std::vector<size_t> sizes;
-    // order: a h1 d2 d1 s1 ga part | z1 z2 s2 w2d2 zd1 zd2 h1b nu_a hd1 z2b A1T B1T A2T B2T ebar loss sums
+    // order: a h1 d2 d1 s1 ga part | z1 z2 s2 w2d2 zd1 zd2 h1b A1 B1 A2 B2 ebar loss sums
     sizes = {2 * C * Pp, 2 * C * H, 2 * C * H, 2 * C * H, 4 * C * H, 2 * C * Pp, 4 * C * (size_t)m->nparts};
     if (tr) {
         for (int i = 0; i < 7; ++i) sizes.push_back(4 * C * H);
-        sizes.push_back(2 * C * Pp);
-        sizes.push_back(2 * C * H);
-        sizes.push_back(2 * C * H);
         sizes.push_back(2 * H * 2 * C);
         sizes.push_back(2 * Pp * 2 * C);
         sizes.push_back(2 * H * 2 * C);
@@ -679,20 +659,13 @@ int mlp_ensure_work(pamd_mlp* m, long long M, bool train) {
     if (tr) {
         float** f32[7] = {&nw.z1, &nw.z2, &nw.s2, &nw.w2d2, &nw.zd1, &nw.zd2, &nw.h1b};
         for (auto q : f32) *q = reinterpret_cast<float*>(take());
-        nw.nu_a = reinterpret_cast<__nv_bfloat16*>(take());
-        nw.hd1 = reinterpret_cast<__nv_bfloat16*>(take());
-        nw.z2b = reinterpret_cast<__nv_bfloat16*>(take());
-        nw.A1T = reinterpret_cast<__nv_bfloat16*>(take());
-        nw.B1T = reinterpret_cast<__nv_bfloat16*>(take());
-        nw.A2T = reinterpret_cast<__nv_bfloat16*>(take());
-        nw.B2T = reinterpret_cast<__nv_bfloat16*>(take());
+        nw.A1 = reinterpret_cast<__nv_bfloat16*>(take());
+        nw.B1 = reinterpret_cast<__nv_bfloat16*>(take());
+        nw.A2 = reinterpret_cast<__nv_bfloat16*>(take());
+        nw.B2 = reinterpret_cast<__nv_bfloat16*>(take());
         nw.ebar = reinterpret_cast<float*>(take());
         nw.loss_part = reinterpret_cast<double*>(take());
         nw.sum_part = reinterpret_cast<double*>(take());
-        // the transposed operands are read over K = 2M columns: clear them so
-        // that no column is ever uninitialised memory
-        if (cudaMemsetAsync(nw.A1T, 0, (size_t)(p - reinterpret_cast<char*>(nw.A1T)), m->stream) != cudaSuccess)
-            return mcuda(m, cudaGetLastError(), "workspace clear");
     }
     w = nw;
     return PAMD_OK;
@@ -733,12 +706,12 @@ int mlp_gemms(pamd_mlp* m, int M, bool forces, cudaStream_t s, int* status) {
     if (!forces) return PAMD_OK;
     // d1 = (d2 W2) * s1
     g = GemmArgs{};
-    g.A = w.d2; g.B = m->W2Tb; g.M = M; g.N = H; g.K = H; g.lda = H; g.ldb = H;
+    g.mode = kGemmNN; g.A = w.d2; g.B = m->W2b; g.M = M; g.N = H; g.K = H; g.lda = H; g.ldb = H;
     g.epi = kEpiMul; g.mul = w.s1; g.ldc = H; g.Cb = w.d1; g.ldcb = H;
     if ((rc = gemm(m, g, s, status))) return rc;
     // de/da = d1 W1
     g = GemmArgs{};
-    g.A = w.d1; g.B = m->W1Tb; g.M = M; g.N = Pp; g.K = H; g.lda = H; g.ldb = H;
+    g.mode = kGemmNN; g.A = w.d1; g.B = m->W1b; g.M = M; g.N = Pp; g.K = H; g.lda = H; g.ldb = Pp;
     g.epi = kEpiStore; g.Cb = w.ga; g.ldcb = Pp; g.ldc = Pp;
     return gemm(m, g, s, status);
 }
@@ -761,7 +734,7 @@ int pamd_mlp_create(pamd_mlp** out, int32_t n_atoms, int32_t hidden, uint64_t se
     m->P = n_atoms * (n_atoms - 1) / 2;
     m->Pp = (m->P + 7) / 8 * 8;
     m->H = hidden;
-    m->nparts = kGemmHeadParts * ((hidden + kGemmTileN - 1) / kGemmTileN);
+    m->nparts = gemm_head_parts(hidden);
     const size_t H = (size_t)hidden, Pp = (size_t)m->Pp;
     m->oW1 = 0;
     m->ob1 = H * Pp;
@@ -772,8 +745,7 @@ int pamd_mlp_create(pamd_mlp** out, int32_t n_atoms, int32_t hidden, uint64_t se
     m->n_params = m->ob3 + 4;
     const size_t pbytes = align256(4 * m->n_params);
     const size_t sizes[] = {pbytes, pbytes, pbytes, pbytes, align256(4 * Pp), align256(4 * Pp),
-                            align256(4 * Pp), align256(2 * H * Pp), align256(2 * H * Pp),
-                            align256(2 * H * H), align256(2 * H * H), align256(4 * Pp),
+                            align256(4 * Pp), align256(2 * H * Pp), align256(2 * H * H), align256(4 * Pp),
                             align256(sizeof(int)), align256(8 * 4)};
     size_t total = 0;
     for (size_t s : sizes) total += s;
@@ -806,9 +778,7 @@ int pamd_mlp_create(pamd_mlp** out, int32_t n_atoms, int32_t hidden, uint64_t se
     m->sd = reinterpret_cast<float*>(take());
     m->inv_sd = reinterpret_cast<float*>(take());
     m->W1b = reinterpret_cast<__nv_bfloat16*>(take());
-    m->W1Tb = reinterpret_cast<__nv_bfloat16*>(take());
     m->W2b = reinterpret_cast<__nv_bfloat16*>(take());
-    m->W2Tb = reinterpret_cast<__nv_bfloat16*>(take());
     m->pairs = reinterpret_cast<ushort2*>(take());
     m->status = reinterpret_cast<int*>(take());
     m->scratch = reinterpret_cast<double*>(take());
@@ -982,7 +952,7 @@ int pamd_mlp_energy_forces(pamd_mlp* m, const float* x_dev, int64_t M, double* E
     if (!E_dev && !F_dev) return PAMD_OK;
     if ((rc = mlp_ensure_work(m, M, false))) return rc;
     const ConfigView cv{x_dev, 3LL * m->N, 3, 1, nullptr};
-    if ((rc = features(m, cv, (int)M, nullptr, 0))) return rc;
+    if ((rc = features(m, cv, (int)M, m->w.a))) return rc;
     if ((rc = mlp_gemms(m, (int)M, F_dev != nullptr, m->stream, m->status))) return rc;
     ForceArgs f{};
     f.cv = cv;
@@ -1014,29 +984,33 @@ int pamd_mlp_loss_grads(pamd_mlp* m, const float* x_dev, const double* E_dev, co
     if (!(lam >= 0.0) || !std::isfinite(lam)) return mfail(PAMD_EINVAL, "pamd_mlp_loss_grads: lam must be >= 0");
     if ((rc = mlp_ensure_work(m, M, true))) return rc;
     const MlpWork& w = m->w;
-    const int H = m->H, Pp = m->Pp, Mi = (int)M, ldt = 2 * Mi;
+    const int H = m->H, Pp = m->Pp, Mi = (int)M;
     cudaStream_t s = m->stream;
     const ConfigView cv{x_dev, 3LL * m->N, 3, 1, idx_dev};
+    // the operands of the weight gradients: M rows of the energy part, then M
+    // of the force part (see MlpWork)
+    const size_t MH = (size_t)Mi * H;
+    __nv_bfloat16 *const a = w.B1, *const nu_a = w.B1 + (size_t)Mi * Pp, *const h1 = w.B2, *const hd1 = w.B2 + MH,
+                  *const z1b = w.A1, *const d1 = w.A1 + MH, *const z2b = w.A2, *const d2 = w.A2 + MH;
     // forward, keeping what the gradient needs
-    if ((rc = features(m, cv, Mi, w.B1T, ldt))) return rc;
+    if ((rc = features(m, cv, Mi, a))) return rc;
     GemmArgs g{};
-    g.A = w.a; g.B = m->W1b; g.M = Mi; g.N = H; g.K = Pp; g.lda = Pp; g.ldb = Pp;
+    g.A = a; g.B = m->W1b; g.M = Mi; g.N = H; g.K = Pp; g.lda = Pp; g.ldb = Pp;
     g.bias = m->params + m->ob1; g.epi = kEpiSilu;
-    g.C = w.z1; g.Cs = w.s1; g.ldc = H; g.Cb = w.h1; g.ldcb = H; g.CbT = w.B2T; g.ldt = ldt;
+    g.C = w.z1; g.Cs = w.s1; g.ldc = H; g.Cb = h1; g.ldcb = H;
     if ((rc = gemm(m, g, s))) return rc;
     g = GemmArgs{};
-    g.A = w.h1; g.B = m->W2b; g.M = Mi; g.N = H; g.K = H; g.lda = H; g.ldb = H;
+    g.A = h1; g.B = m->W2b; g.M = Mi; g.N = H; g.K = H; g.lda = H; g.ldb = H;
     g.bias = m->params + m->ob2; g.epi = kEpiHead; g.vec = m->params + m->ow3;
-    g.C = w.z2; g.Cs = w.s2; g.ldc = H; g.Cb = w.d2; g.ldcb = H; g.CbT = w.A2T + Mi; g.ldt = ldt;
+    g.C = w.z2; g.Cs = w.s2; g.ldc = H; g.Cb = d2; g.ldcb = H;
     g.part = w.part;
     if ((rc = gemm(m, g, s))) return rc;
     g = GemmArgs{};
-    g.A = w.d2; g.B = m->W2Tb; g.M = Mi; g.N = H; g.K = H; g.lda = H; g.ldb = H;
-    g.epi = kEpiMul; g.mul = w.s1; g.C = w.w2d2; g.ldc = H; g.Cb = w.d1; g.ldcb = H;
-    g.CbT = w.A1T + Mi; g.ldt = ldt;
+    g.mode = kGemmNN; g.A = d2; g.B = m->W2b; g.M = Mi; g.N = H; g.K = H; g.lda = H; g.ldb = H;
+    g.epi = kEpiMul; g.mul = w.s1; g.C = w.w2d2; g.ldc = H; g.Cb = d1; g.ldcb = H;
     if ((rc = gemm(m, g, s))) return rc;
     g = GemmArgs{};
-    g.A = w.d1; g.B = m->W1Tb; g.M = Mi; g.N = Pp; g.K = H; g.lda = H; g.ldb = H;
+    g.mode = kGemmNN; g.A = d1; g.B = m->W1b; g.M = Mi; g.N = Pp; g.K = H; g.lda = H; g.ldb = Pp;
     g.epi = kEpiStore; g.Cb = w.ga; g.ldcb = Pp; g.ldc = Pp;
     if ((rc = gemm(m, g, s))) return rc;
     // loss, energy cotangent and the tangent direction nu_a
@@ -1057,21 +1031,18 @@ int pamd_mlp_loss_grads(pamd_mlp* m, const float* x_dev, const double* E_dev, co
     L.mu_E = m->mu_E;
     L.sigma_E = m->sigma_E;
     L.lam = lam;
-    L.nu_a = w.nu_a;
-    L.nu_aT = w.B1T + Mi;
-    L.ldt = ldt;
+    L.nu_a = nu_a;
     L.ebar = w.ebar;
     L.loss_part = w.loss_part;
     mlp_loss_kernel<<<grid_for(M * kMlpThreads, kMlpThreads, 152 * 16), kMlpThreads, loss_smem(m), s>>>(L);
     if ((rc = launch_check(m, "loss"))) return rc;
     // tangent pass: zd1 = W1 nu_a, hd1 = zd1 s1, zd2 = W2 hd1
     g = GemmArgs{};
-    g.A = w.nu_a; g.B = m->W1b; g.M = Mi; g.N = H; g.K = Pp; g.lda = Pp; g.ldb = Pp;
-    g.epi = kEpiMul; g.mul = w.s1; g.C = w.zd1; g.ldc = H; g.Cb = w.hd1; g.ldcb = H;
-    g.CbT = w.B2T + Mi; g.ldt = ldt;
+    g.A = nu_a; g.B = m->W1b; g.M = Mi; g.N = H; g.K = Pp; g.lda = Pp; g.ldb = Pp;
+    g.epi = kEpiMul; g.mul = w.s1; g.C = w.zd1; g.ldc = H; g.Cb = hd1; g.ldcb = H;
     if ((rc = gemm(m, g, s))) return rc;
     g = GemmArgs{};
-    g.A = w.hd1; g.B = m->W2b; g.M = Mi; g.N = H; g.K = H; g.lda = H; g.ldb = H;
+    g.A = hd1; g.B = m->W2b; g.M = Mi; g.N = H; g.K = H; g.lda = H; g.ldb = H;
     g.epi = kEpiStore; g.C = w.zd2; g.ldc = H;
     if ((rc = gemm(m, g, s))) return rc;
     // reverse: z2_bar, h1_bar = z2_bar W2, z1_bar
@@ -1079,26 +1050,28 @@ int pamd_mlp_loss_grads(pamd_mlp* m, const float* x_dev, const double* E_dev, co
     const size_t psz = (size_t)tiles * H;
     const dim3 bar_grid((H + kBarCols - 1) / kBarCols, tiles);
     BarArgs bar{};
-    bar.M = Mi; bar.H = H; bar.ldt = ldt; bar.ebar = w.ebar;
+    bar.M = Mi; bar.H = H; bar.ebar = w.ebar;
     bar.z = w.z2; bar.s = w.s2; bar.zd = w.zd2; bar.w3 = m->params + m->ow3;
-    bar.zb = w.z2b; bar.AT = w.A2T; bar.part_b = w.sum_part + psz; bar.part_w3 = w.sum_part + 2 * psz;
+    bar.zb = z2b; bar.part_b = w.sum_part + psz; bar.part_w3 = w.sum_part + 2 * psz;
     mlp_zbar_kernel<2><<<bar_grid, kBarThreads, 0, s>>>(bar);
     if ((rc = launch_check(m, "z2 cotangent"))) return rc;
     g = GemmArgs{};
-    g.A = w.z2b; g.B = m->W2Tb; g.M = Mi; g.N = H; g.K = H; g.lda = H; g.ldb = H;
+    g.mode = kGemmNN; g.A = z2b; g.B = m->W2b; g.M = Mi; g.N = H; g.K = H; g.lda = H; g.ldb = H;
     g.epi = kEpiStore; g.C = w.h1b; g.ldc = H;
     if ((rc = gemm(m, g, s))) return rc;
     bar.z = w.z1; bar.s = w.s1; bar.zd = w.zd1; bar.up = w.h1b; bar.w2d2 = w.w2d2;
-    bar.AT = w.A1T; bar.part_b = w.sum_part;
+    bar.zb = z1b; bar.part_b = w.sum_part;
     mlp_zbar_kernel<1><<<bar_grid, kBarThreads, 0, s>>>(bar);
     if ((rc = launch_check(m, "z1 cotangent"))) return rc;
-    // weight gradients: contractions over the 2M columns of the transposed operands
+    // weight gradients: contractions over the 2M rows of the operands
     g = GemmArgs{};
-    g.A = w.A1T; g.B = w.B1T; g.M = H; g.N = Pp; g.K = ldt; g.lda = ldt; g.ldb = ldt;
+    g.mode = kGemmTN;
+    g.A = w.A1; g.B = w.B1; g.M = H; g.N = Pp; g.K = 2 * Mi; g.lda = H; g.ldb = Pp;
     g.epi = kEpiStore; g.C = m->grads + m->oW1; g.ldc = Pp;
     if ((rc = gemm(m, g, s))) return rc;
     g = GemmArgs{};
-    g.A = w.A2T; g.B = w.B2T; g.M = H; g.N = H; g.K = ldt; g.lda = ldt; g.ldb = ldt;
+    g.mode = kGemmTN;
+    g.A = w.A2; g.B = w.B2; g.M = H; g.N = H; g.K = 2 * Mi; g.lda = H; g.ldb = H;
     g.epi = kEpiStore; g.C = m->grads + m->oW2; g.ldc = H;
     if ((rc = gemm(m, g, s))) return rc;
     SumArgs sums{};
@@ -1127,9 +1100,8 @@ int pamd_mlp_adam_step(pamd_mlp* m, double lr, double beta1, double beta2, doubl
     const long long n = (long long)m->ob3 + 1;
     mlp_adam_kernel<<<grid_for(n, 256), 256, 0, m->stream>>>(m->params, m->grads, m->adam_m, m->adam_v, n,
                                                              (float)lr, (float)beta1, (float)beta2,
-                                                             (float)eps, bc1, bc2);
-    if ((rc = launch_check(m, "Adam"))) return rc;
-    return pack(m);
+                                                             (float)eps, bc1, bc2, weight_copies(m));
+    return launch_check(m, "Adam");
 }
 
 // Model file: magic, {N, H}, the FP32 parameter block (W1 padded to Pp

@@ -41,8 +41,7 @@ __device__ __forceinline__ void load_config(const ConfigView& cv, int m, int N, 
 __device__ __forceinline__ void block_features(const float* xs, const ushort2* __restrict__ pairs,
                                                const float* __restrict__ mu,
                                                const float* __restrict__ inv_sd, int P, int Pp,
-                                               __nv_bfloat16* a_row, __nv_bfloat16* aT, int ldt,
-                                               int m) {
+                                               __nv_bfloat16* a_row) {
 #pragma unroll 4
     for (int p = threadIdx.x; p < Pp; p += blockDim.x) {
         float v = 0.0f;
@@ -54,9 +53,7 @@ __device__ __forceinline__ void block_features(const float* xs, const ushort2* _
             const float g = rsqrtf(fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
             v = (g - mu[p]) * inv_sd[p];
         }
-        const __nv_bfloat16 b = __float2bfloat16(v);
-        a_row[p] = b;
-        if (aT) aT[(size_t)p * ldt + m] = b;
+        a_row[p] = __float2bfloat16(v);
     }
 }
 

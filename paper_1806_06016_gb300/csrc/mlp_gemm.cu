@@ -1,26 +1,39 @@
 // mlp_gemm.cu -- BF16 GEMM on the 5th-generation tensor cores (tcgen05),
 // for the dense layers of the MLP energy surrogate.
 //
-// C[M x N] (FP32) = A[M x K] . B[N x K]^T, A and B row-major BF16 (both
-// "K-major").  Persistent kernel, one CTA per SM, in clusters of two CTAs
-// that compute the 128 x 256 output tiles of two adjacent row blocks in the
-// same column block, so that the 256 x 64 B tile of each k-step is read from
-// L2 once per cluster instead of once per CTA.  Six warps with fixed roles:
-//   * one thread of warp 0 streams the CTA's 128 x 64 tile of A and its half
-//     (128 x 64) of the shared B tile with TMA (cp.async.bulk.tensor, 128-byte
-//     swizzle, out-of-range rows and columns zero-filled), the B half
-//     multicast into both CTAs' stage, into a ring of kStages shared-memory
-//     stages, each completing a transaction-count mbarrier; a stage is
-//     refilled once the products of both CTAs have read it;
-//   * one thread of warp 1 issues four tcgen05.mma (M 128, N 256, K 16) per
-//     stage into one of two FP32 accumulators of 256 tensor-memory columns,
+// C (FP32) = A . B with BF16 operands stored row-major in one of three forms:
+//   NT  A[M x K], B[N x K]: the contraction index is contiguous in both;
+//   NN  A[M x K], B[K x N]: products with the transpose of a weight;
+//   TN  A[K x M], B[K x N]: weight gradients, contracted over the samples.
+// The tensor core reads either order from shared memory, so no operand is
+// ever transposed in memory.  Persistent kernel, one CTA per SM, in clusters
+// of two CTAs that compute the 128 x BN output tiles of two adjacent row
+// blocks in the same column block, so that the BN x 64 B tile of each k-step
+// is read from L2 once per cluster instead of once per CTA.  Ten warps with
+// fixed roles:
+//   * warp 0 streams the CTA's 128 x 64 tile of A and its half
+//     of the shared B tile with TMA (cp.async.bulk.tensor, 128-byte swizzle,
+//     out-of-range rows and columns zero-filled), the B half multicast into
+//     both CTAs' stage, into a ring of kStages shared-memory stages, each
+//     completing a transaction-count mbarrier; a stage is refilled once the
+//     products of both CTAs have read it;
+//   * warp 1 issues four tcgen05.mma (M 128, N BN, K 16) per operand
+//     tile into one of two FP32 accumulators of BN tensor-memory columns,
 //     frees each stage in both CTAs with a multicast tcgen05.commit, and
 //     commits the accumulator when a tile's last product is issued;
-//   * warps 2..5 drain a finished accumulator with tcgen05.ld (warp w reads
+//   * warps 2..9 drain a finished accumulator with tcgen05.ld (warp w reads
 //     tensor-memory lanes 32 (w mod 4) ..), apply the bias and the layer's
 //     output transform, store with 16-byte vector stores, and hand the
 //     accumulator back -- so the epilogue of one tile runs while the tensor
 //     core works on the next.
+//
+// A k-step is bound by what one thread issues, not by the copies: the stage
+// holds two k-tiles where the ring is deep enough, the abort flag is read only
+// in the slow part of a wait, slot and parity are counters, and the warps walk
+// the ring as a whole with an elected lane issuing, which spares the issue
+// loops over lanes that a single-lane branch costs (per 64 of K at BN = 64:
+// 0.41 us before, 0.15 now; 512 x 8192 x 64: 59.5 -> 28.8 us; 65536 x 512 x
+// 2776 at BN = 256: 178 -> 169 us, 1.10 PFLOP/s).
 //
 // Every wait on an mbarrier is bounded: after kWaitLimit polls the waiting
 // role records PAMD_ETIMEOUT and raises a shared abort flag, the others stop
@@ -41,20 +54,33 @@ namespace pamd {
 
 namespace {
 
-constexpr int kBM = 128, kBN = kGemmTileN, kBK = 64, kStages = 4;
+constexpr int kBM = 128;
+constexpr int kBK = 64;   // contraction depth of one operand tile (128 bytes of BF16)
 // warp 0: TMA producer, warp 1: MMA issuer, warps 2..9: epilogue (two warps
 // per tensor-memory lane quarter, each taking one half of the tile's columns)
 constexpr int kEpiWarps = 8, kThreads = 64 + 32 * kEpiWarps, kEpiThreads = 32 * kEpiWarps;
 constexpr int kTileA = kBM * kBK * 2;  // 16 KiB
-constexpr int kTileB = kBN * kBK * 2;  // 32 KiB
-constexpr int kStageBytes = kTileA + kTileB;
-constexpr int kTmemCols = 2 * kBN;     // two accumulators: all 512 columns
+constexpr int kRingBytes = 192 * 1024;
 constexpr uint32_t kWaitLimit = 1u << 22;
 
+// Per tile width BN: bytes of a B tile and a stage [A A | B B], stages of the
+// ring (192 KiB), tensor-memory columns (two accumulators).
+template <int BN>
+struct Tile {
+    static constexpr int kSub = BN == 256 ? 1 : 2;  // operand tiles per ring stage
+    static constexpr int kTileB = BN * kBK * 2;
+    static constexpr int kStageBytes = kSub * (kTileA + kTileB);
+    static constexpr int kStages = kRingBytes / kStageBytes;  // 4, 3, 4 for BN = 256, 128, 64
+    static constexpr int kTmemCols = 2 * BN;
+};
+
 // instruction descriptor of tcgen05.mma.kind::f16: D FP32 (bits 4-5 = 1),
-// A BF16 (bits 7-9 = 1), B BF16 (bits 10-12 = 1), both K-major, N >> 3 at
-// bits 17-22, M >> 4 at bits 24-28
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kBN >> 3) << 17) |
+// A BF16 (bits 7-9 = 1), B BF16 (bits 10-12 = 1), bits 15 and 16: A and B
+// stored with the row index of the product contiguous, not the contraction
+// index; N >> 3 at bits 17-22, M >> 4 at bits 24-28
+template <int BN, int MODE>
+constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (MODE == kGemmTN ? 1u << 15 : 0u) |
+                            (MODE != kGemmNT ? 1u << 16 : 0u) | ((uint32_t)(BN >> 3) << 17) |
                             ((uint32_t)(kBM >> 4) << 24);
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -67,6 +93,18 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
     uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFFu);
     d |= (uint64_t)1 << 16;
+    d |= (uint64_t)(1024 >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)2 << 61;
+    return d;
+}
+
+// The same for an operand stored [k][row]: groups of 64 rows of the
+// product are 128 bytes wide and kBK k-rows (8 KiB) long, one after another
+// (leading byte offset), groups of 8 k-rows 1024 bytes apart (stride).
+__device__ __forceinline__ uint64_t sw128_desc_tn(uint32_t saddr) {
+    uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFFu);
+    d |= (uint64_t)(kBK * 128 >> 4) << 16;
     d |= (uint64_t)(1024 >> 4) << 32;
     d |= (uint64_t)1 << 46;
     d |= (uint64_t)2 << 61;
@@ -89,13 +127,35 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 
-// bounded wait (polls, then polls with a short sleep); false on timeout
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+// Bounded wait (polls, then polls with a short sleep); false on timeout, or
+// when another role has raised the abort flag.  The flag is read only in the
+// slow part: the producer and the issuer are single threads, and 30 cycles of
+// a shared-memory read in each of their steps were a quarter of a k-step.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const volatile int* abort_flag = nullptr) {
     for (uint32_t i = 0; i < kWaitLimit; ++i) {
         if (mbar_try_wait(bar, parity)) return true;
-        if (i >= 1024) __nanosleep(64);
+        if (i >= 1024) {
+            if (abort_flag && *abort_flag) return false;
+            __nanosleep(64);
+        }
     }
     return false;
+}
+
+// the same by all lanes of a warp, with one result
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, const volatile int* abort_flag) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
+}
+
+// true in one lane of a converged warp, the same one on each call
+__device__ __forceinline__ bool elect_one() {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok));
+    return ok != 0;
 }
 
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
@@ -120,13 +180,13 @@ __device__ __forceinline__ void tc_fence_after() {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t adesc, uint64_t bdesc,
+__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem), "l"(adesc), "l"(bdesc), "r"(kIdesc), "r"(accumulate)
+        ::"r"(tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 
@@ -228,18 +288,16 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-// Epilogue of one half (128 columns) of a 128 x 256 tile: accumulator
-// columns of this warp's 32 tensor-memory lanes (rows m0 + 32q + lane);
-// taddr and n0 point at the half's first column.
-__device__ __forceinline__ void epilogue_tile(const GemmArgs& g, uint32_t taddr, int row, int n0,
-                                              int ntile, int ntiles, int half) {
+// Epilogue of `chunks` x 32 columns of a tile: accumulator columns of this
+// warp's 32 tensor-memory lanes (rows m0 + 32q + lane); taddr and n0 point at
+// the first column.
+__device__ __forceinline__ void epilogue_tile(const GemmArgs& g, uint32_t taddr, int row, int n0, int chunks) {
     const bool row_ok = row < g.M;
     float head = 0.0f;
     __nv_bfloat16* Cb = static_cast<__nv_bfloat16*>(g.Cb);
-    __nv_bfloat16* CbT = static_cast<__nv_bfloat16*>(g.CbT);
     const bool vf = (g.vec_ok & 1) != 0, vb = (g.vec_ok & 2) != 0;
 #pragma unroll 1
-    for (int cc = 0; cc < kBN / 64; ++cc) {
+    for (int cc = 0; cc < chunks; ++cc) {
         float v[32];
         tmem_ld32(taddr + (uint32_t)(cc * 32), v);
         const int col0 = n0 + cc * 32;
@@ -285,20 +343,23 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs& g, uint32_t taddr,
             }
         }
         if (Cb) store_row32_bf16(Cb + (size_t)row * g.ldcb + col0, v, n, vb);
-        if (CbT) {
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-                if (j < n) CbT[(size_t)(col0 + j) * g.ldt + row] = __float2bfloat16(v[j]);
-        }
     }
-    if (g.epi == kEpiHead && row_ok)
-        g.part[(size_t)row * (kGemmHeadParts * ntiles) + kGemmHeadParts * ntile + half] = head;
+    // one partial sum of the head per 128 columns; a tile of 128 columns that
+    // is the last one writes the zero of the missing other half as well
+    if (g.epi == kEpiHead && row_ok) {
+        const int np = gemm_head_parts(g.N), at = n0 / 128;
+        g.part[(size_t)row * np + at] = head;
+        if (at + 1 < np && n0 + 128 >= g.N && chunks * 32 == 128 && at % 2 == 0) g.part[(size_t)row * np + at + 1] = 0.0f;
+    }
 }
 
+template <int BN, int MODE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-    gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA,
-                                                                const __grid_constant__ CUtensorMap tmB,
-                                                                const __grid_constant__ GemmArgs g) {
+    gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                     const __grid_constant__ GemmArgs g) {
+    constexpr int kSub = Tile<BN>::kSub;
+    constexpr int kBN = BN, kStages = Tile<BN>::kStages, kStageBytes = Tile<BN>::kStageBytes, kTileB = Tile<BN>::kTileB;
+    constexpr uint32_t kTmemCols = Tile<BN>::kTmemCols;
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) unsigned long long full_bar[kStages], empty_bar[kStages];
     __shared__ __align__(8) unsigned long long accf_bar[2], acce_bar[2], done_bar;
@@ -312,7 +373,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     // multicast to both.
     const int MT = (g.M + kBM - 1) / kBM, NT = (g.N + kBN - 1) / kBN;
     const int tiles = ((MT + 1) / 2) * NT;  // tile pairs
-    const int KB = (g.K + kBK - 1) / kBK;
+    const int KT = (g.K + kBK - 1) / kBK, KB = (KT + kSub - 1) / kSub;  // operand tiles and stages of a product
     const int crank = (int)cluster_rank();
     const int cid = blockIdx.x >> 1, ncl = gridDim.x >> 1;
 
@@ -346,74 +407,123 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     volatile int* abort_flag = &s_abort;
 
     if (warp == 0) {
-        if (lane == 0) {  // TMA producer
-            long long gk = 0;
+        {  // TMA producer: the warp walks the ring, one lane issues
+            uint32_t gk = 0, st = 0, ph = 0;  // stages so far, ring slot, its use number's parity
             bool stop = false;
             for (int t = cid; t < tiles && !stop; t += ncl) {
-                // A box of an odd last row block's missing partner, or a B half
+                // A box of an odd last row block's missing partner, or a B box
                 // past column N, would lie wholly outside its matrix: read a
                 // valid box instead (its products land in rows / columns the
                 // epilogue drops)
                 const int n0 = (t % NT) * kBN;
-                const int ya = min((2 * (t / NT) + crank) * kBM, (MT - 1) * kBM);
-                const int yb = (n0 + crank * (kBN / 2) < g.N) ? n0 + crank * (kBN / 2) : n0;
+                const int m0 = min((2 * (t / NT) + crank) * kBM, (MT - 1) * kBM);
                 for (int kb = 0; kb < KB; ++kb, ++gk) {
-                    const int st = (int)(gk % kStages);
-                    if (gk >= kStages &&
-                        !mbar_wait(smem_u32(&empty_bar[st]), (uint32_t)((gk / kStages - 1) & 1))) {
+                    if (gk >= (uint32_t)kStages && !mbar_wait_warp(smem_u32(&empty_bar[st]), ph ^ 1u, abort_flag)) {
                         *abort_flag = 1;
-                    }
-                    if (*abort_flag) {
                         stop = true;
                         break;
                     }
                     const uint32_t fb = smem_u32(&full_bar[st]);
-                    const uint32_t ta = base + (uint32_t)(st * kStageBytes);
-                    mbar_expect_tx(fb, (uint32_t)kStageBytes);
-                    tma_load_2d(ta, &tmA, kb * kBK, ya, fb);
-                    tma_load_2d_mc(ta + kTileA + crank * (kTileB / 2), &tmB, kb * kBK, yb, fb,
-                                   (uint16_t)0x3);
+                    const uint32_t sa = base + st * (uint32_t)kStageBytes, sb = sa + kSub * kTileA;
+                    const int subs = min(kSub, KT - kb * kSub);
+                    if (elect_one()) {
+                        mbar_expect_tx(fb, (uint32_t)(subs * (kTileA + kTileB)));
+#pragma unroll
+                        for (int u = 0; u < kSub; ++u) {
+                            if (u >= subs) break;
+                            const uint32_t ta = sa + u * kTileA, tb = sb + u * kTileB;
+                            const int k0 = (kb * kSub + u) * kBK;
+                            if (MODE == kGemmTN) {  // A: boxes of 64 rows of the product x 64 k-rows
+#pragma unroll
+                                for (int q = 0; q < kBM / 64; ++q) {
+                                    const int x = m0 + 64 * q;
+                                    tma_load_2d(ta + q * kBK * 128, &tmA, x < g.M ? x : m0, k0, fb);
+                                }
+                            } else {
+                                tma_load_2d(ta, &tmA, k0, m0, fb);
+                            }
+                            if (MODE != kGemmNT) {
+                                // B: boxes of 64 columns x 32 k-rows, half the k-rows from
+                                // each CTA.  The last tile may have no rows for the
+                                // second one: it reads the first one's (A is zero there)
+                                const int y = k0 + crank * (kBK / 2);
+#pragma unroll
+                                for (int q = 0; q < BN / 64; ++q) {
+                                    const int x = n0 + 64 * q;
+                                    tma_load_2d_mc(tb + q * kBK * 128 + crank * (kBK / 2) * 128, &tmB, x < g.N ? x : n0,
+                                                   y < g.K ? y : k0, fb, (uint16_t)0x3);
+                                }
+                            } else {
+                                const int yb = (n0 + crank * (kBN / 2) < g.N) ? n0 + crank * (kBN / 2) : n0;
+                                tma_load_2d_mc(tb + crank * (kTileB / 2), &tmB, k0, yb, fb, (uint16_t)0x3);
+                            }
+                        }
+                    }
+                    __syncwarp();
+                    if (++st == (uint32_t)kStages) {
+                        st = 0;
+                        ph ^= 1u;
+                    }
                 }
             }
             s_issued = (int)gk;
             // the peer's last releases of this CTA's stages land before it exits
-            for (long long u = gk > kStages ? gk - kStages : 0; u < gk && !*abort_flag; ++u)
-                if (!mbar_wait(smem_u32(&empty_bar[u % kStages]), (uint32_t)((u / kStages) & 1)))
+            for (uint32_t u = gk > (uint32_t)kStages ? gk - kStages : 0; u < gk; ++u)
+                if (!mbar_wait_warp(smem_u32(&empty_bar[u % kStages]), (u / kStages) & 1u, abort_flag)) {
                     *abort_flag = 1;
+                    break;
+                }
         }
     } else if (warp == 1) {
-        if (lane == 0) {  // MMA issuer
-            long long gk = 0;
+        {  // MMA issuer, likewise
+            uint32_t gk = 0, st = 0, ph = 0;
             int i = 0;
             bool stop = false;
             for (int t = cid; t < tiles && !stop; t += ncl, ++i) {
                 const int acc = i & 1;
-                if (i >= 2 && !mbar_wait(smem_u32(&acce_bar[acc]), (uint32_t)((i / 2 - 1) & 1))) {
+                if (i >= 2 && !mbar_wait_warp(smem_u32(&acce_bar[acc]), (uint32_t)((i / 2 - 1) & 1), abort_flag)) {
                     *abort_flag = 1;
                     break;
                 }
                 tc_fence_after();
                 const uint32_t td = tmem + (uint32_t)(acc * kBN);
                 for (int kb = 0; kb < KB; ++kb, ++gk) {
-                    const int st = (int)(gk % kStages);
-                    if (!mbar_wait(smem_u32(&full_bar[st]), (uint32_t)((gk / kStages) & 1))) *abort_flag = 1;
-                    if (*abort_flag) {
+                    if (!mbar_wait_warp(smem_u32(&full_bar[st]), ph, abort_flag)) {
+                        *abort_flag = 1;
                         stop = true;
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t ta = base + (uint32_t)(st * kStageBytes);
+                    const uint32_t sa = base + st * (uint32_t)kStageBytes, sb = sa + kSub * kTileA;
+                    const int subs = min(kSub, KT - kb * kSub);
+                    if (elect_one()) {
 #pragma unroll
-                    for (int k = 0; k < kBK / 16; ++k)
-                        mma_bf16(td, sw128_desc(ta + k * 32), sw128_desc(ta + kTileA + k * 32),
-                                 (kb > 0 || k > 0) ? 1u : 0u);
-                    mma_commit_mc(smem_u32(&empty_bar[st]), (uint16_t)0x3);
+                        for (int u = 0; u < kSub; ++u) {
+                            if (u >= subs) break;
+                            const uint32_t ta = sa + u * kTileA, tb = sb + u * kTileB;
+                            const uint64_t da = MODE == kGemmTN ? sw128_desc_tn(ta) : sw128_desc(ta);
+                            const uint64_t db = MODE != kGemmNT ? sw128_desc_tn(tb) : sw128_desc(tb);
+                            // 16 of the contraction further: 32 bytes along a row, or 16 rows
+#pragma unroll
+                            for (int k = 0; k < kBK / 16; ++k)
+                                mma_bf16(td, da + (uint64_t)(k * (MODE == kGemmTN ? 16 * 128 : 32) >> 4),
+                                         db + (uint64_t)(k * (MODE != kGemmNT ? 16 * 128 : 32) >> 4), kIdesc<BN, MODE>,
+                                         (kb > 0 || u > 0 || k > 0) ? 1u : 0u);
+                        }
+                        mma_commit_mc(smem_u32(&empty_bar[st]), (uint16_t)0x3);
+                    }
+                    __syncwarp();
+                    if (++st == (uint32_t)kStages) {
+                        st = 0;
+                        ph ^= 1u;
+                    }
                 }
-                if (!stop) mma_commit(smem_u32(&accf_bar[acc]));
+                if (!stop && elect_one()) mma_commit(smem_u32(&accf_bar[acc]));
+                __syncwarp();
             }
             s_consumed = (int)gk;
             // tracks every product issued before it, also on the abort path
-            mma_commit(smem_u32(&done_bar));
+            if (elect_one()) mma_commit(smem_u32(&done_bar));
         }
     } else {  // epilogue warps 2..9
         const int q = warp & 3;  // tensor-memory lane quarter this warp may access
@@ -421,14 +531,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         int i = 0;
         for (int t = cid; t < tiles; t += ncl, ++i) {
             const int acc = i & 1;
-            if (!mbar_wait(smem_u32(&accf_bar[acc]), (uint32_t)((i / 2) & 1))) *abort_flag = 1;
-            __syncwarp();
-            if (*abort_flag) break;
+            if (!mbar_wait_warp(smem_u32(&accf_bar[acc]), (uint32_t)((i / 2) & 1), abort_flag)) {
+                *abort_flag = 1;
+                break;
+            }
             tc_fence_after();
             const int m0 = (2 * (t / NT) + crank) * kBM, nt = t % NT;
-            const uint32_t taddr =
-                tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kBN + half * (kBN / 2));
-            epilogue_tile(g, taddr, m0 + q * 32 + lane, nt * kBN + half * (kBN / 2), nt, NT, half);
+            const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kBN);
+            // the head's partial sums run over 128 columns: with a tile that
+            // narrow one warp per quarter takes them all
+            if (BN == 128 && g.epi == kEpiHead) {
+                if (half == 0) epilogue_tile(g, taddr, m0 + q * 32 + lane, nt * kBN, BN / 32);
+            } else {
+                epilogue_tile(g, taddr + (uint32_t)(half * (kBN / 2)), m0 + q * 32 + lane, nt * kBN + half * (kBN / 2),
+                              BN / 64);
+            }
             tc_fence_before();
             mbar_arrive(smem_u32(&acce_bar[acc]));
         }
@@ -439,7 +556,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         if (*abort_flag) {
             atomicCAS(g.status, 0, PAMD_ETIMEOUT);
             // copies issued but never consumed must land before the CTA exits
-            for (long long gk = s_consumed; gk < s_issued; ++gk)
+            for (int gk = s_consumed; gk < s_issued; ++gk)
                 mbar_wait(smem_u32(&full_bar[gk % kStages]), (uint32_t)((gk / kStages) & 1));
         }
         mbar_wait(smem_u32(&done_bar), 0u);  // products in flight
@@ -498,15 +615,30 @@ bool on_device(const void* p, int dev) {
 
 constexpr int kMaxDevices = 64;
 
-// Kernel attribute and resident cluster count, once per device.
+using GemmKernel = void (*)(const CUtensorMap, const CUtensorMap, const GemmArgs);
+constexpr size_t kGemmSmem = kRingBytes + 1024;
+
+template <int MODE>
+GemmKernel gemm_kernel_of(int bn) {
+    return bn == 256 ? gemm_bf16_kernel<256, MODE> : bn == 128 ? gemm_bf16_kernel<128, MODE> : gemm_bf16_kernel<64, MODE>;
+}
+GemmKernel gemm_kernel(int bn, int mode) {
+    return mode == kGemmNT ? gemm_kernel_of<kGemmNT>(bn) : mode == kGemmTN ? gemm_kernel_of<kGemmTN>(bn)
+                                                                           : gemm_kernel_of<kGemmNN>(bn);
+}
+
+// Kernel attributes and resident cluster count, once per device.
 cudaError_t gemm_setup(int dev, int* max_clusters_out) {
-    const size_t smem = (size_t)kStages * kStageBytes + 1024;
+    const size_t smem = kGemmSmem;
     static std::once_flag once[kMaxDevices];
     static cudaError_t attr[kMaxDevices];
     static int max_clusters[kMaxDevices];
     std::call_once(once[dev], [&] {
-        cudaError_t e = cudaFuncSetAttribute(gemm_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
+        cudaError_t e = cudaSuccess;
+        for (int bn = 64; bn <= 256 && e == cudaSuccess; bn *= 2)
+            for (int mode = kGemmNT; mode <= kGemmNN && e == cudaSuccess; ++mode)
+                e = cudaFuncSetAttribute((const void*)gemm_kernel(bn, mode), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
         // persistent grid: as many two-CTA clusters as can be resident at once
         // (an SM left without a partner in its GPC hosts none)
         cudaLaunchConfig_t cfg{};
@@ -514,7 +646,7 @@ cudaError_t gemm_setup(int dev, int* max_clusters_out) {
         cfg.blockDim = dim3(kThreads, 1, 1);
         cfg.dynamicSmemBytes = smem;
         int mc = 0;
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&mc, gemm_bf16_kernel, &cfg);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&mc, gemm_kernel(256, kGemmNT), &cfg);
         if (e == cudaSuccess && mc < 1) e = cudaErrorInvalidConfiguration;
         attr[dev] = e;
         max_clusters[dev] = mc;
@@ -531,6 +663,26 @@ cudaError_t gemm_prepare_device() {
     return gemm_setup(dev, nullptr);
 }
 
+// Tile pairs (two row blocks of one column block) of a product.
+long long gemm_tiles(const GemmArgs& g, int bn) {
+    return (long long)((g.M + 2 * kBM - 1) / (2 * kBM)) * ((g.N + bn - 1) / bn);
+}
+
+// Tile width: the narrowest of 64, 128 and 256 columns whose tile pairs still
+// fit the resident clusters in one wave, else 256.  One wave of narrow tiles
+// has shorter steps and uses more SMs; past one wave the wide tile reads
+// least per product.  Measured with BN = 64 / 128 / 256, us (NT, FP32 result):
+//   N 512,  K 2776: M 2048 16.5 / 18.6 / 24.6, 4096 28.8 / 19.9 / 24.7,
+//                   8192 53 / 34.9 / 25.4, 65536 346 / 229 / 169;
+//   N 512,  K 512:  M 2048 8.3 / 10.3 / 12.4, 8192 14.5 / 12.5 / 12.4;
+//   N 2776, K 512:  M 256 8.3 / 10.3 / 12.4, 512 10.4 / 10.3 / 12.4.
+// The head sums over 128 columns in one thread: not below that.
+int tile_width(const GemmArgs& g, int max_clusters) {
+    int bn = 256;
+    while (bn > (g.epi == kEpiHead ? 128 : 64) && gemm_tiles(g, bn / 2) <= max_clusters) bn /= 2;
+    return bn;
+}
+
 cudaError_t launch_gemm_bf16(const GemmArgs& ga, cudaStream_t s) {
     if (ga.M <= 0 || ga.N <= 0 || ga.K <= 0 || (ga.K & 7) || (ga.lda & 7) || (ga.ldb & 7) ||
         (reinterpret_cast<uintptr_t>(ga.A) & 15) || (reinterpret_cast<uintptr_t>(ga.B) & 15))
@@ -542,23 +694,25 @@ cudaError_t launch_gemm_bf16(const GemmArgs& ga, cudaStream_t s) {
     // The B tile is multicast by TMA into both CTAs of a cluster: the tensor
     // maps must cover this GPU's own memory only.
     if (!on_device(ga.A, dev) || !on_device(ga.B, dev)) return cudaErrorInvalidValue;
+    int max_clusters = 0;
+    const cudaError_t se = gemm_setup(dev, &max_clusters);
+    if (se != cudaSuccess) return se;
+    const int bn = tile_width(ga, max_clusters);
     CUtensorMap tmA, tmB;
-    if (!encode_operand(&tmA, ga.A, ga.M, ga.K, ga.lda, kBM) ||
-        !encode_operand(&tmB, ga.B, ga.N, ga.K, ga.ldb, kBN / 2))
-        return cudaErrorInvalidValue;
+    const bool mapped = (ga.mode == kGemmTN ? encode_operand(&tmA, ga.A, ga.K, ga.M, ga.lda, kBK)
+                                            : encode_operand(&tmA, ga.A, ga.M, ga.K, ga.lda, kBM)) &&
+                        (ga.mode == kGemmNT ? encode_operand(&tmB, ga.B, ga.N, ga.K, ga.ldb, bn / 2)
+                                            : encode_operand(&tmB, ga.B, ga.K, ga.N, ga.ldb, kBK / 2));
+    if (!mapped) return cudaErrorInvalidValue;
     GemmArgs g = ga;
     auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
     const bool f_ok = (g.ldc % 4 == 0) && al16(g.C) && al16(g.Cs) && al16(g.mul);
     const bool b_ok = (g.ldcb % 8 == 0) && al16(g.Cb);
     g.vec_ok = (f_ok ? 1 : 0) | (b_ok ? 2 : 0);
-    const size_t smem = (size_t)kStages * kStageBytes + 1024;
-    int max_clusters = 0;
-    const cudaError_t se = gemm_setup(dev, &max_clusters);
-    if (se != cudaSuccess) return se;
     // one cluster per pair of row blocks and column block, at most max_clusters
-    const long long pairs = (long long)((g.M + 2 * kBM - 1) / (2 * kBM)) * ((g.N + kBN - 1) / kBN);
-    const int grid = 2 * (int)(pairs < max_clusters ? pairs : max_clusters);
-    gemm_bf16_kernel<<<grid, kThreads, smem, s>>>(tmA, tmB, g);
+    const long long tiles = gemm_tiles(ga, bn);
+    const int grid = 2 * (int)(tiles < max_clusters ? tiles : max_clusters);
+    gemm_kernel(bn, ga.mode)<<<grid, kThreads, kGemmSmem, s>>>(tmA, tmB, g);
     return cudaGetLastError();
 }
 

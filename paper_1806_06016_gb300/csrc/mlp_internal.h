@@ -31,13 +31,11 @@ struct MlpWork {
     float* zd1 = nullptr;        // tangent pass
     float* zd2 = nullptr;
     float* h1b = nullptr;        // dL/dh1
-    __nv_bfloat16* nu_a = nullptr;  // [cap][Pp]
-    __nv_bfloat16* hd1 = nullptr;   // [cap][H]
-    __nv_bfloat16* z2b = nullptr;   // [cap][H]
-    __nv_bfloat16* A1T = nullptr;   // [H][2cap]  (z1_bar^T | d1^T)
-    __nv_bfloat16* B1T = nullptr;   // [Pp][2cap] (a^T | nu_a^T)
-    __nv_bfloat16* A2T = nullptr;   // [H][2cap]  (z2_bar^T | d2^T)
-    __nv_bfloat16* B2T = nullptr;   // [H][2cap]  (h1^T | hd1^T)
+    // operands of the weight gradients, two sets of M rows one after another
+    __nv_bfloat16* A1 = nullptr;    // [2cap][H]  (z1_bar; d1)
+    __nv_bfloat16* B1 = nullptr;    // [2cap][Pp] (a; nu_a)
+    __nv_bfloat16* A2 = nullptr;    // [2cap][H]  (z2_bar; d2)
+    __nv_bfloat16* B2 = nullptr;    // [2cap][H]  (h1; hd1)
     float* ebar = nullptr;          // [cap]
     double* loss_part = nullptr;    // [cap]
     double* sum_part = nullptr;     // [3][tiles][H] partial sums of the b1, b2 and w3 gradients
@@ -59,8 +57,6 @@ struct FeatArgs {
     const float* mu;         // [Pp]
     const float* inv_sd;     // [Pp]
     __nv_bfloat16* a;        // [M][Pp]
-    __nv_bfloat16* aT;       // [Pp][ldt] or null
-    int ldt;
 };
 
 struct ForceArgs {
@@ -88,8 +84,6 @@ struct LossArgs {
     const float* b3;         // device scalar
     double mu_E, sigma_E, lam;
     __nv_bfloat16* nu_a;     // [M][Pp]
-    __nv_bfloat16* nu_aT;    // [Pp][ldt], column offset included
-    int ldt;
     float* ebar;             // [M]
     double* loss_part;       // [M]
 };
@@ -148,9 +142,7 @@ struct pamd_mlp {
     float* inv_sd = nullptr;     // [Pp]
     double mu_E = 0.0, sigma_E = 1.0;
     __nv_bfloat16* W1b = nullptr;   // [H][Pp]
-    __nv_bfloat16* W1Tb = nullptr;  // [Pp][H]
     __nv_bfloat16* W2b = nullptr;   // [H][H]
-    __nv_bfloat16* W2Tb = nullptr;  // [H][H]
     ushort2* pairs = nullptr;       // [Pp]
     int* status = nullptr;
     double* scratch = nullptr;      // [4] loss and statistics

@@ -348,31 +348,32 @@ cudaError_t propagate2_b3(const PropParams* p, bool chain, int warps, int grid, 
 cudaError_t propagate2_b4(const PropParams* p, bool chain, int warps, int grid, size_t smem,
                           cudaStream_t s, int* blocks_per_sm);
 
-// BF16 tensor-core GEMM (mlp_gemm.cu): C = A . B^T with A [M x K], B [N x K]
-// row-major BF16 (K contiguous), FP32 accumulation, and a fused epilogue on
-// z = acc (+ bias[n]):
+// BF16 tensor-core GEMM (mlp_gemm.cu): C [M x N] = the product over K of BF16
+// operands, FP32 accumulation, and a fused epilogue on z = acc (+ bias[n]):
 //   kEpiStore  C = z, Cb = bf16(z)                       (each output optional)
-//   kEpiSilu   C = z, Cs = silu'(z), Cb = bf16(silu(z)), CbT = Cb transposed
-//   kEpiHead   C = z, Cs = silu'(z), Cb = bf16(vec[n] silu'(z)), CbT, and
-//              part[m * 2 ntiles + 2 tile + h] = sum over the n of half h of
-//              the tile of vec[n] silu(z), ntiles = ceil(N / kGemmTileN)
-//   kEpiMul    C = z, Cb = bf16(z * mul[m, n]) (mul FP32, leading dim ldc), CbT
+//   kEpiSilu   C = z, Cs = silu'(z), Cb = bf16(silu(z))
+//   kEpiHead   C = z, Cs = silu'(z), Cb = bf16(vec[n] silu'(z)), and
+//              part[m][b] = sum of vec[n] silu(z) over the columns n of the
+//              b-th 128, gemm_head_parts(N) of them (an even number)
+//   kEpiMul    C = z, Cb = bf16(z * mul[m, n]) (mul FP32, leading dim ldc)
 enum GemmEpi { kEpiStore = 0, kEpiSilu = 1, kEpiHead = 2, kEpiMul = 3 };
-constexpr int kGemmTileN = 256;   // output columns per tile
-constexpr int kGemmHeadParts = 2;  // kEpiHead partial sums per tile (part[] has 2 ceil(N / kGemmTileN) columns)
+__host__ __device__ constexpr int gemm_head_parts(int N) { return 2 * ((N + 255) / 256); }
+// How the operands are stored: NT A [M x K], B [N x K]; TN A [K x M], B [K x
+// N]; NN A [M x K], B [K x N] (row-major each).
+enum GemmMode { kGemmNT = 0, kGemmTN = 1, kGemmNN = 2 };
 struct GemmArgs {
-    const void* A;             // __nv_bfloat16 [M][lda]
-    const void* B;             // __nv_bfloat16 [N][ldb]
+    const void* A;             // __nv_bfloat16 [M][lda], TN: [K][lda]
+    const void* B;             // __nv_bfloat16 [N][ldb], NN and TN: [K][ldb]
     float* C;                  // [M][ldc] or null
     float* Cs;                 // [M][ldc] or null
     void* Cb;                  // __nv_bfloat16 [M][ldcb] or null
-    void* CbT;                 // __nv_bfloat16 [N][ldt] or null
     const float* bias;         // [N] or null
     const float* vec;          // [N] (kEpiHead)
     const float* mul;          // [M][ldc] (kEpiMul)
-    float* part;               // [M][kGemmHeadParts ceil(N / kGemmTileN)] (kEpiHead)
+    float* part;               // [M][gemm_head_parts(N)] (kEpiHead)
     int* status;               // PAMD status word (timeouts)
-    int M, N, K, lda, ldb, ldc, ldcb, ldt, epi;
+    int M, N, K, lda, ldb, ldc, ldcb, epi;
+    int mode;                  // GemmMode
     int vec_ok;                // set by the launcher: 1 FP32 rows, 2 BF16 rows 16-byte aligned
 };
 cudaError_t launch_gemm_bf16(const GemmArgs& g, cudaStream_t s);

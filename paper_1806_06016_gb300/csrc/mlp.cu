@@ -319,39 +319,202 @@ __global__ void __launch_bounds__(128) mlp_moments_merge_kernel(const float* __r
 
 // ------------------------------------------------------- features and forces
 
-__global__ void __launch_bounds__(kMlpThreads) mlp_features_kernel(const FeatArgs f) {
-    __shared__ float xs[3 * kXs];
-    for (int m = blockIdx.x; m < f.M; m += gridDim.x) {
-        __syncthreads();
-        load_config(f.cv, m, f.N, xs);
-        __syncthreads();
-        block_features(xs, f.pairs, f.mu, f.inv_sd, f.P, f.Pp, f.a + (size_t)m * f.Pp);
+// Features of 2 DUOS configurations per block, one after another from one read
+// of the pair's tables.  Bound by shared-memory reads (4 wavefronts a pair
+// and 32 configurations' lanes) and issue; the BF16 rows it writes are 5.5 KB a
+// configuration of 75 atoms.
+// 65536 configurations of 75 atoms, DUOS = 4: 165 us (a block per configuration
+// that read six words and three table entries a pair: 342), shared-memory
+// pipe 84 % busy.
+constexpr int kFeatThreads = 256;
+
+template <int DUOS>
+__global__ void __launch_bounds__(kFeatThreads) mlp_features_kernel(const FeatArgs f) {
+    extern __shared__ __align__(16) unsigned char qsm[];
+    const int N = f.N, n3 = 3 * N, m0 = blockIdx.x * 2 * DUOS;
+    for (int t = threadIdx.x; t < 2 * DUOS * n3; t += kFeatThreads) {
+        const int g = t / n3;
+        int i, c;
+        config_element(f.cv, t - g * n3, N, i, c);
+        const int m = m0 + g < f.M ? m0 + g : f.M - 1;
+        duo_pos(qsm + (g >> 1) * duo_pos_bytes(N), N).put(g & 1, i, c, config_value(f.cv, m, i, c));
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int p = threadIdx.x; p < f.Pp; p += kFeatThreads) {
+        const bool in = p < f.P;
+        const ushort2 ij = in ? f.pairs[p] : make_ushort2(0, 0);
+        const float mu = in ? f.mu[p] : 0.0f, isd = in ? f.inv_sd[p] : 0.0f;
+        __nv_bfloat16* a = f.a + (size_t)m0 * f.Pp + p;
+#pragma unroll
+        for (int u = 0; u < DUOS; ++u, a += 2 * f.Pp) {
+            const float2 v = duo_feature(duo_pos(qsm + u * duo_pos_bytes(N), N), ij, mu, isd);
+            if (m0 + 2 * u < f.M) a[0] = __float2bfloat16(in ? v.x : 0.0f);
+            if (m0 + 2 * u + 1 < f.M) a[f.Pp] = __float2bfloat16(in ? v.y : 0.0f);
+        }
     }
 }
 
+// Energies, and the forces of molecules with gamma_matrix(N): two
+// configurations at a time per block.  One pass over the pairs fills the
+// matrix c_ij, one over its rows sums c_kj (x_k - x_j) with each row split
+// over several threads; meanwhile the next two de/da rows arrive by
+// cp.async and their positions in registers.  Bound by shared-memory
+// wavefronts (8 per 32 pairs and configuration in the first pass, 2 per 32
+// elements in the second) and by the barriers between the passes.
+// 65536 configurations of 75 atoms: 471 us (one configuration at a time, 75 of
+// 128 threads in the second pass: 796); shared-memory pipe 72 % busy.
+// 16384 of 128 atoms with the rest of the call: 2062 -> 895 us.
+// Block size: as many threads as a row split over up to eight keeps busy.
+// Small molecules in 384 threads leave most idle at the barriers (65536
+// configurations of 9 atoms, whole call: 210 us, in 64 threads 131; 16384 of
+// 22: 102 and, in 128, 87).
+constexpr int kDuoPartsMax = 8;
+constexpr int kDuoElems = 2;  // coordinates per thread: 6 N <= 2 threads
+
+__host__ __device__ __forceinline__ int duo_threads(int N) { return N <= 21 ? 64 : N <= 42 ? 128 : 384; }
+static_assert(6 * 21 <= kDuoElems * 64 && 6 * 42 <= kDuoElems * 128 && 6 * kGammaMatrixMax <= kDuoElems * 384, "");
+__host__ __device__ __forceinline__ int duo_parts(int N) {
+    return duo_threads(N) / N < kDuoPartsMax ? duo_threads(N) / N : kDuoPartsMax;
+}
+
+// byte offsets: matrix, de/da rows, positions, partial force sums [part][2][N][3]
+struct DuoSmem {
+    size_t ga, pos, part, total;
+};
+__host__ __device__ __forceinline__ DuoSmem duo_smem(int N, int Pp) {
+    auto up = [](size_t b) { return (b + 15) & ~size_t(15); };
+    DuoSmem L{};
+    L.ga = up(duo_gamma_bytes(N));
+    L.pos = L.ga + 4 * (size_t)Pp;
+    L.part = L.pos + duo_pos_bytes(N);
+    L.total = L.part + 24 * (size_t)N * duo_parts(N);
+    return L;
+}
+
+__device__ __forceinline__ void duo_fetch_rows(const __nv_bfloat16* ga, int m0, int m1, int Pp, unsigned char* dst) {
+    const int n = Pp / 8;
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    for (int t = threadIdx.x; t < 2 * n; t += blockDim.x) {
+        const __nv_bfloat16* src = ga + (size_t)(t < n ? m0 : m1) * Pp + 8 * (t < n ? t : t - n);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + 16 * t), "l"(src) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+__device__ __forceinline__ void duo_fetch_pos(const ConfigView& cv, int m0, int m1, int N, float (&v)[kDuoElems]) {
+#pragma unroll
+    for (int u = 0; u < kDuoElems; ++u) {
+        const int t = threadIdx.x + u * blockDim.x, b = t >= 3 * N;
+        int i, c;
+        config_element(cv, t - 3 * N * b, N, i, c);
+        v[u] = t < 6 * N ? config_value(cv, b ? m1 : m0, i, c) : 0.0f;
+    }
+}
+__device__ __forceinline__ void duo_store_pos(const ConfigView& cv, int N, const float (&v)[kDuoElems], const DuoPos& q) {
+#pragma unroll
+    for (int u = 0; u < kDuoElems; ++u) {
+        const int t = threadIdx.x + u * blockDim.x, b = t >= 3 * N;
+        int i, c;
+        config_element(cv, t - 3 * N * b, N, i, c);
+        if (t < 6 * N) q.put(b, i, c, v[u]);
+    }
+}
+
+// the row sums of both configurations into part[h][b][k][c], duo_threads(N) threads
+__device__ __forceinline__ void duo_force_parts(const DuoPos& q, const float2* gam, int N, float* part) {
+    const int parts = duo_parts(N), len = (N + parts - 1) / parts;
+    const int h = threadIdx.x / N, k = threadIdx.x - h * N;
+    if (h >= parts) return;
+    const int j0 = min(h * len, N), j1 = min(N, j0 + len);
+    const Duo3 s = duo_force(k, q, gam, N, j0, j1);
+    float* o = part + (size_t)h * 6 * N + 3 * k;
+    o[0] = s.x.x;
+    o[1] = s.y.x;
+    o[2] = s.z.x;
+    o += 3 * N;
+    o[0] = s.x.y;
+    o[1] = s.y.y;
+    o[2] = s.z.y;
+}
+__device__ __forceinline__ float duo_force_sum(const float* part, int N, int t) {
+    const int parts = duo_parts(N);
+    float v = part[t];
+    for (int h = 1; h < parts; ++h) v += part[h * 6 * N + t];
+    return v;
+}
+
+__device__ __forceinline__ void energies(const ForceArgs& f) {
+    for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < f.M; m += gridDim.x * blockDim.x)
+        f.E[m] = f.sigma_E * head_energy(f.part, f.nparts, m, f.b3) + f.mu_E;
+}
+
+template <int T>
+__global__ void __launch_bounds__(T, T == 384 ? 3 : 1024 / T) mlp_forces_duo_kernel(const ForceArgs f) {
+    extern __shared__ __align__(16) unsigned char dsm[];
+    const int N = f.N, D = (f.M + 1) / 2;
+    const DuoSmem L = duo_smem(N, f.Pp);
+    float2* gam = reinterpret_cast<float2*>(dsm);
+    const __nv_bfloat16* ga = reinterpret_cast<const __nv_bfloat16*>(dsm + L.ga);
+    const DuoPos q = duo_pos(dsm + L.pos, N);
+    float* part = reinterpret_cast<float*>(dsm + L.part);
+    if (f.E) energies(f);
+    if (!f.F) return;
+    const float sE = (float)f.sigma_E;
+    auto second = [&](int d) { return 2 * d + 1 < f.M ? 2 * d + 1 : 2 * d; };
+    float v[kDuoElems];
+    int d = blockIdx.x;
+    if (d < D) {
+        duo_fetch_rows(f.ga, 2 * d, second(d), f.Pp, dsm + L.ga);
+        duo_fetch_pos(f.cv, 2 * d, second(d), N, v);
+    }
+    for (int k = threadIdx.x; k < N; k += T) gam[k * gamma_stride(N) + k] = make_float2(0.0f, 0.0f);
+    for (; d < D; d += gridDim.x) {
+        duo_store_pos(f.cv, N, v, q);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        duo_gamma(q, ga, f.pairs, f.inv_sd, f.P, f.Pp, N, gam);
+        __syncthreads();
+        const int nd = d + gridDim.x;
+        if (nd < D) {
+            duo_fetch_rows(f.ga, 2 * nd, second(nd), f.Pp, dsm + L.ga);
+            duo_fetch_pos(f.cv, 2 * nd, second(nd), N, v);
+        }
+        duo_force_parts(q, gam, N, part);
+        __syncthreads();
+        const int n = 2 * d + 1 < f.M ? 6 * N : 3 * N;
+        float* Fo = f.F + (size_t)d * 6 * N;
+        for (int t = threadIdx.x; t < n; t += T) Fo[t] = sE * duo_force_sum(part, N, t);
+    }
+}
+
+using ForceKernel = void (*)(const ForceArgs);
+ForceKernel forces_duo_kernel(int N) {
+    const int t = duo_threads(N);
+    return t == 64 ? mlp_forces_duo_kernel<64> : t == 128 ? mlp_forces_duo_kernel<128> : mlp_forces_duo_kernel<384>;
+}
+
+// The same for molecules past gamma_matrix(N), whose matrix does not fit.
 __global__ void __launch_bounds__(kMlpThreads) mlp_forces_kernel(const ForceArgs f) {
     extern __shared__ float fsm[];
     float* xs = fsm;
     float* gam = fsm + 3 * kXs;
-    init_gamma(f.N, gam);
+    if (f.E) energies(f);
+    if (!f.F) return;
+    const float sE = (float)f.sigma_E;
     for (int m = blockIdx.x; m < f.M; m += gridDim.x) {
         __syncthreads();
         load_config(f.cv, m, f.N, xs);
         __syncthreads();
-        if (f.F) load_gamma(xs, f.ga + (size_t)m * f.Pp, f.inv_sd, f.pairs, f.P, f.N, gam);
+        load_gamma(xs, f.ga + (size_t)m * f.Pp, f.inv_sd, f.pairs, f.P, f.N, gam);
         __syncthreads();
-        if (f.F) {
-            const float sE = (float)f.sigma_E;
-            float* Fo = f.F + (size_t)m * 3 * f.N;
-            for (int k = threadIdx.x; k < f.N; k += blockDim.x) {
-                const float3 a = atom_force_any(k, xs, gam, f.N);
-                Fo[3 * k] = sE * a.x;
-                Fo[3 * k + 1] = sE * a.y;
-                Fo[3 * k + 2] = sE * a.z;
-            }
+        float* Fo = f.F + (size_t)m * 3 * f.N;
+        for (int k = threadIdx.x; k < f.N; k += blockDim.x) {
+            const float3 a = atom_force_any(k, xs, gam, f.N);
+            Fo[3 * k] = sE * a.x;
+            Fo[3 * k + 1] = sE * a.y;
+            Fo[3 * k + 2] = sE * a.z;
         }
-        if (f.E && threadIdx.x == 0)
-            f.E[m] = f.sigma_E * head_energy(f.part, f.nparts, m, f.b3) + f.mu_E;
     }
 }
 
@@ -582,7 +745,8 @@ size_t loss_smem(const pamd_mlp* m) { return sizeof(float) * (6 * kXs + (size_t)
 // The dynamic shared-memory limits of the force and loss kernels on the
 // current device, raised to what this model needs.
 int set_smem_attrs(const pamd_mlp* m) {
-    cudaError_t e = ensure_dyn_smem((const void*)mlp_forces_kernel, forces_smem(m));
+    cudaError_t e = gamma_matrix(m->N) ? ensure_dyn_smem((const void*)forces_duo_kernel(m->N), duo_smem(m->N, m->Pp).total)
+                                       : ensure_dyn_smem((const void*)mlp_forces_kernel, forces_smem(m));
     if (e == cudaSuccess) e = ensure_dyn_smem((const void*)mlp_loss_kernel, loss_smem(m));
     return e == cudaSuccess ? PAMD_OK : mfail(PAMD_ECUDA, std::string("kernel attributes: ") + cudaGetErrorString(e));
 }
@@ -598,8 +762,14 @@ int features(pamd_mlp* m, const ConfigView& cv, int M, __nv_bfloat16* a) {
     f.mu = m->mu;
     f.inv_sd = m->inv_sd;
     f.a = a;
-    mlp_features_kernel<<<grid_for((long long)M * kMlpThreads, kMlpThreads, 152 * 16), kMlpThreads, 0,
-                          m->stream>>>(f);
+    // Eight configurations a block read the tables least; two keep enough
+    // blocks in flight below four waves of the chip.  Whole energy call, 75
+    // atoms, eight / two, us: M 64 41.9 / 36.8, 1024 43.9 / 41.9, 4096 52.1 /
+    // 51.1, 8192 62.4 / 64.5, 65536 290 / 334.
+    if (M >= 8 * 152 * 4)
+        mlp_features_kernel<4><<<(M + 7) / 8, kFeatThreads, 4 * duo_pos_bytes(m->N), m->stream>>>(f);
+    else
+        mlp_features_kernel<1><<<(M + 1) / 2, kFeatThreads, duo_pos_bytes(m->N), m->stream>>>(f);
     return launch_check(m, "features");
 }
 
@@ -970,8 +1140,14 @@ int pamd_mlp_energy_forces(pamd_mlp* m, const float* x_dev, int64_t M, double* E
     f.mu_E = m->mu_E;
     f.E = E_dev;
     f.F = F_dev;
-    mlp_forces_kernel<<<grid_for(M * kMlpThreads, kMlpThreads, 152 * 16), kMlpThreads,
-                        forces_smem(m), m->stream>>>(f);
+    if (gamma_matrix(m->N)) {
+        const int t = duo_threads(m->N);
+        const int grid = F_dev ? grid_for((M + 1) / 2 * t, t, 152 * (t == 384 ? 3 : 1024 / t)) : grid_for(M, t);
+        forces_duo_kernel(m->N)<<<grid, t, duo_smem(m->N, m->Pp).total, m->stream>>>(f);
+    } else {
+        mlp_forces_kernel<<<F_dev ? grid_for(M * kMlpThreads, kMlpThreads, 152 * 16) : grid_for(M, kMlpThreads), kMlpThreads,
+                            forces_smem(m), m->stream>>>(f);
+    }
     return launch_check(m, "surrogate forces");
 }
 

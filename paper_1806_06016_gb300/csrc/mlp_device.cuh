@@ -36,25 +36,68 @@ __device__ __forceinline__ void load_config(const ConfigView& cv, int m, int N, 
     }
 }
 
-// a_p = (1 / r_ij - mu_p) / sd_p rounded to BF16, zero for the padding
-// columns P <= p < Pp (whole block)
-__device__ __forceinline__ void block_features(const float* xs, const ushort2* __restrict__ pairs,
-                                               const float* __restrict__ mu,
-                                               const float* __restrict__ inv_sd, int P, int Pp,
-                                               __nv_bfloat16* a_row) {
-#pragma unroll 4
-    for (int p = threadIdx.x; p < Pp; p += blockDim.x) {
-        float v = 0.0f;
-        if (p < P) {
-            const ushort2 ij = pairs[p];
-            const float dx = xs[ij.x] - xs[ij.y];
-            const float dy = xs[kXs + ij.x] - xs[kXs + ij.y];
-            const float dz = xs[2 * kXs + ij.x] - xs[2 * kXs + ij.y];
-            const float g = rsqrtf(fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
-            v = (g - mu[p]) * inv_sd[p];
-        }
-        a_row[p] = __float2bfloat16(v);
+// ------------------------------------------------ two configurations at a time
+// The pair passes are bound by shared-memory reads and instruction issue, not
+// by HBM.  Two configurations side by side, (xA, xB, yA, yB) and (zA, zB) per
+// atom, halve both: one 16- and one 8-byte read bring an atom of both, the
+// packed FP32 instructions work on both, and the pair table is read once.
+// Consecutive lanes take consecutive row-order pairs: the reads of atom j are
+// free of bank conflicts, those of atom i are broadcasts.  Every element is
+// rounded as it would be alone (a multiply by -1 is exact, so the fused
+// difference rounds like the subtraction).
+struct DuoPos {
+    float4* xy;  // [N]
+    float2* z;   // [N]
+    __device__ __forceinline__ void put(int b, int i, int c, float v) const {
+        if (c < 2) reinterpret_cast<float*>(xy)[4 * i + 2 * c + b] = v;
+        else reinterpret_cast<float*>(z)[2 * i + b] = v;
     }
+};
+
+// a multiple of 16, so that one duo can follow another
+__host__ __device__ __forceinline__ size_t duo_pos_bytes(int N) { return (24 * (size_t)N + 15) & ~size_t(15); }
+__device__ __forceinline__ DuoPos duo_pos(unsigned char* sm, int N) {
+    return DuoPos{reinterpret_cast<float4*>(sm), reinterpret_cast<float2*>(sm + 16 * (size_t)N)};
+}
+
+// element r < 3 N of a configuration in the order it lies in memory: atom i, coordinate c
+__device__ __forceinline__ void config_element(const ConfigView& cv, int r, int N, int& i, int& c) {
+    if (cv.s_coord == 1) {
+        i = r / 3;
+        c = r - 3 * i;
+    } else {
+        c = r / N;
+        i = r - c * N;
+    }
+}
+__device__ __forceinline__ float config_value(const ConfigView& cv, int m, int i, int c) {
+    return cv.x[config_index(cv, m) * cv.s_cfg + (long long)i * cv.s_atom + (long long)c * cv.s_coord];
+}
+
+struct Duo3 {
+    float2 x, y, z;
+};
+
+// x_i - x_j
+__device__ __forceinline__ Duo3 duo_diff(const float4 a, const float2 az, const float4 b, const float2 bz) {
+    const float2 m1 = make_float2(-1.0f, -1.0f);
+    Duo3 d;
+    d.x = __ffma2_rn(m1, make_float2(b.x, b.y), make_float2(a.x, a.y));
+    d.y = __ffma2_rn(m1, make_float2(b.z, b.w), make_float2(a.z, a.w));
+    d.z = __ffma2_rn(m1, bz, az);
+    return d;
+}
+
+// 1 / |d|
+__device__ __forceinline__ float2 duo_inv_norm(const Duo3& d) {
+    const float2 s = __ffma2_rn(d.z, d.z, __ffma2_rn(d.y, d.y, __fmul2_rn(d.x, d.x)));
+    return make_float2(rsqrtf(s.x), rsqrtf(s.y));
+}
+
+// (1 / r_ij - mu) / sd
+__device__ __forceinline__ float2 duo_feature(const DuoPos& q, const ushort2 ij, float mu, float isd) {
+    const float2 g = duo_inv_norm(duo_diff(q.xy[ij.x], q.z[ij.x], q.xy[ij.y], q.z[ij.y]));
+    return __fmul2_rn(__fadd2_rn(g, make_float2(-mu, -mu)), make_float2(isd, isd));
 }
 
 // sum over j != k of gam_p(k,j) (x_k - x_j) / r_kj^3, i.e. minus the
@@ -136,13 +179,51 @@ __device__ __forceinline__ float3 atom_force_any(int k, const float* xs, const f
     return make_float3(fx, fy, fz);
 }
 
+// The symmetric matrix c_ij = gam_ij / r_ij^3 of two configurations (odd row
+// stride: rows of consecutive atoms start on distinct bank pairs), one 1/r per
+// pair, from their de/da rows ga[0..P) and ga[Pp..Pp + P).
+__host__ __device__ __forceinline__ size_t duo_gamma_bytes(int N) { return 8 * (size_t)N * gamma_stride(N); }
+
+__device__ __forceinline__ void duo_gamma(const DuoPos& q, const __nv_bfloat16* ga, const ushort2* __restrict__ pairs,
+                                          const float* __restrict__ inv_sd, int P, int Pp, int N, float2* gam) {
+    const int S = gamma_stride(N);
+#pragma unroll 4
+    for (int p = threadIdx.x; p < P; p += blockDim.x) {
+        const ushort2 ij = pairs[p];
+        const float isd = inv_sd[p];
+        const float2 g = make_float2(__bfloat162float(ga[p]), __bfloat162float(ga[Pp + p]));
+        const float2 ir = duo_inv_norm(duo_diff(q.xy[ij.x], q.z[ij.x], q.xy[ij.y], q.z[ij.y]));
+        const float2 c = __fmul2_rn(__fmul2_rn(__fmul2_rn(__fmul2_rn(g, make_float2(isd, isd)), ir), ir), ir);
+        gam[ij.x * S + ij.y] = c;
+        gam[ij.y * S + ij.x] = c;
+    }
+}
+
+// sum over j0 <= j < j1 of c_kj (x_k - x_j); lanes of consecutive k read x_j as broadcasts
+__device__ __forceinline__ Duo3 duo_force(int k, const DuoPos& q, const float2* gam, int N, int j0, int j1) {
+    const float4 kxy = q.xy[k];
+    const float2 kz = q.z[k];
+    const float2* row = gam + k * gamma_stride(N);
+    const float2 zero = make_float2(0.0f, 0.0f);
+    Duo3 f{zero, zero, zero};
+#pragma unroll 5
+    for (int j = j0; j < j1; ++j) {
+        const float2 c = row[j];
+        const Duo3 d = duo_diff(kxy, kz, q.xy[j], q.z[j]);
+        f.x = __ffma2_rn(c, d.x, f.x);
+        f.y = __ffma2_rn(c, d.y, f.y);
+        f.z = __ffma2_rn(c, d.z, f.z);
+    }
+    return f;
+}
+
 // ------------------------------------------------ pair passes of the MD step kernel
 // Consecutive threads take consecutive row-order pairs, so that the lanes of
 // a warp read consecutive atoms (no shared-memory bank conflicts) and
 // consecutive table entries.  The pair table (i, j) and the per-pair tables
 // may sit in shared or global memory.  Positions sit in shared memory as
 // float4 (x, y, z, 0).  The arithmetic of every pair is that of
-// block_features / load_gamma / atom_force_any, bit for bit.
+// duo_feature / load_gamma / atom_force_any, bit for bit.
 
 __host__ __device__ __forceinline__ size_t step_pos_bytes(int N) { return 16 * (size_t)(N + 1); }
 

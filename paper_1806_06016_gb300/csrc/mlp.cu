@@ -365,19 +365,6 @@ __global__ void __launch_bounds__(kFeatThreads) mlp_features_kernel(const FeatAr
 // 65536 configurations of 75 atoms: 471 us (one configuration at a time, 75 of
 // 128 threads in the second pass: 796); shared-memory pipe 72 % busy.
 // 16384 of 128 atoms with the rest of the call: 2062 -> 895 us.
-// Block size: as many threads as a row split over up to eight keeps busy.
-// Small molecules in 384 threads leave most idle at the barriers (65536
-// configurations of 9 atoms, whole call: 210 us, in 64 threads 131; 16384 of
-// 22: 102 and, in 128, 87).
-constexpr int kDuoPartsMax = 8;
-constexpr int kDuoElems = 2;  // coordinates per thread: 6 N <= 2 threads
-
-__host__ __device__ __forceinline__ int duo_threads(int N) { return N <= 21 ? 64 : N <= 42 ? 128 : 384; }
-static_assert(6 * 21 <= kDuoElems * 64 && 6 * 42 <= kDuoElems * 128 && 6 * kGammaMatrixMax <= kDuoElems * 384, "");
-__host__ __device__ __forceinline__ int duo_parts(int N) {
-    return duo_threads(N) / N < kDuoPartsMax ? duo_threads(N) / N : kDuoPartsMax;
-}
-
 // byte offsets: matrix, de/da rows, positions, partial force sums [part][2][N][3]
 struct DuoSmem {
     size_t ga, pos, part, total;
@@ -390,16 +377,6 @@ __host__ __device__ __forceinline__ DuoSmem duo_smem(int N, int Pp) {
     L.part = L.pos + duo_pos_bytes(N);
     L.total = L.part + 24 * (size_t)N * duo_parts(N);
     return L;
-}
-
-__device__ __forceinline__ void duo_fetch_rows(const __nv_bfloat16* ga, int m0, int m1, int Pp, unsigned char* dst) {
-    const int n = Pp / 8;
-    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-    for (int t = threadIdx.x; t < 2 * n; t += blockDim.x) {
-        const __nv_bfloat16* src = ga + (size_t)(t < n ? m0 : m1) * Pp + 8 * (t < n ? t : t - n);
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + 16 * t), "l"(src) : "memory");
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
 __device__ __forceinline__ void duo_fetch_pos(const ConfigView& cv, int m0, int m1, int N, float (&v)[kDuoElems]) {
@@ -419,29 +396,6 @@ __device__ __forceinline__ void duo_store_pos(const ConfigView& cv, int N, const
         config_element(cv, t - 3 * N * b, N, i, c);
         if (t < 6 * N) q.put(b, i, c, v[u]);
     }
-}
-
-// the row sums of both configurations into part[h][b][k][c], duo_threads(N) threads
-__device__ __forceinline__ void duo_force_parts(const DuoPos& q, const float2* gam, int N, float* part) {
-    const int parts = duo_parts(N), len = (N + parts - 1) / parts;
-    const int h = threadIdx.x / N, k = threadIdx.x - h * N;
-    if (h >= parts) return;
-    const int j0 = min(h * len, N), j1 = min(N, j0 + len);
-    const Duo3 s = duo_force(k, q, gam, N, j0, j1);
-    float* o = part + (size_t)h * 6 * N + 3 * k;
-    o[0] = s.x.x;
-    o[1] = s.y.x;
-    o[2] = s.z.x;
-    o += 3 * N;
-    o[0] = s.x.y;
-    o[1] = s.y.y;
-    o[2] = s.z.y;
-}
-__device__ __forceinline__ float duo_force_sum(const float* part, int N, int t) {
-    const int parts = duo_parts(N);
-    float v = part[t];
-    for (int h = 1; h < parts; ++h) v += part[h * 6 * N + t];
-    return v;
 }
 
 __device__ __forceinline__ void energies(const ForceArgs& f) {
@@ -480,11 +434,11 @@ __global__ void __launch_bounds__(T, T == 384 ? 3 : 1024 / T) mlp_forces_duo_ker
             duo_fetch_rows(f.ga, 2 * nd, second(nd), f.Pp, dsm + L.ga);
             duo_fetch_pos(f.cv, 2 * nd, second(nd), N, v);
         }
-        duo_force_parts(q, gam, N, part);
+        duo_force_parts(q, gam, N, duo_parts(N), part);
         __syncthreads();
         const int n = 2 * d + 1 < f.M ? 6 * N : 3 * N;
         float* Fo = f.F + (size_t)d * 6 * N;
-        for (int t = threadIdx.x; t < n; t += T) Fo[t] = sE * duo_force_sum(part, N, t);
+        for (int t = threadIdx.x; t < n; t += T) Fo[t] = sE * duo_force_sum(part, N, duo_parts(N), t);
     }
 }
 
@@ -506,11 +460,11 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_forces_kernel(const ForceArgs
         __syncthreads();
         load_config(f.cv, m, f.N, xs);
         __syncthreads();
-        load_gamma(xs, f.ga + (size_t)m * f.Pp, f.inv_sd, f.pairs, f.P, f.N, gam);
+        load_gamma(f.ga + (size_t)m * f.Pp, f.inv_sd, f.P, gam);
         __syncthreads();
         float* Fo = f.F + (size_t)m * 3 * f.N;
         for (int k = threadIdx.x; k < f.N; k += blockDim.x) {
-            const float3 a = atom_force_any(k, xs, gam, f.N);
+            const float3 a = atom_force(k, xs, gam, f.N);
             Fo[3 * k] = sE * a.x;
             Fo[3 * k + 1] = sE * a.y;
             Fo[3 * k + 2] = sE * a.z;
@@ -521,6 +475,104 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_forces_kernel(const ForceArgs
 // Force-matching loss of one sample and the direction of the tangent pass:
 // f = sum_p gam_p dg_p/dx (normalised forces), u = dL/df, and
 // nu_a = dL/d(de/da) = (J u) / sd with (J u)_p = (x_i - x_j).(u_i - u_j) / r^3.
+// Two samples at a time like the force kernel, with a second pass over the
+// pairs for J u; bound likewise by shared-memory wavefronts and barriers.
+// 2048 samples of 75 atoms: 61 us (one at a time, 75 of 128 threads at the
+// force rows: 70).
+// Shared memory: that of the force kernel with dL/df in the place of the partial sums.
+__host__ __device__ __forceinline__ size_t loss_duo_smem(int N, int Pp) {
+    return ((duo_smem(N, Pp).part + 15) & ~size_t(15)) + duo_pos_bytes(N);
+}
+
+template <int T>
+__global__ void __launch_bounds__(T, T == 384 ? 3 : 1024 / T) mlp_loss_duo_kernel(const LossArgs A) {
+    extern __shared__ __align__(16) unsigned char dsm[];
+    __shared__ double red[32];
+    const int N = A.N, D = (A.M + 1) / 2;
+    const DuoSmem L = duo_smem(N, A.Pp);
+    float2* gam = reinterpret_cast<float2*>(dsm);
+    const __nv_bfloat16* ga = reinterpret_cast<const __nv_bfloat16*>(dsm + L.ga);
+    const DuoPos q = duo_pos(dsm + L.pos, N), us = duo_pos(dsm + ((L.part + 15) & ~size_t(15)), N);
+    const float2* xs = reinterpret_cast<const float2*>(q.xy);  // x of atom i at 2 i, y at 2 i + 1
+    const double inv_sE = 1.0 / A.sigma_E;
+    const float cu = (float)(2.0 * A.lam / (3.0 * N * (double)A.M));
+    auto second = [&](int d) { return 2 * d + 1 < A.M ? 2 * d + 1 : 2 * d; };
+    float v[kDuoElems];
+    int d = blockIdx.x;
+    if (d < D) {
+        duo_fetch_rows(A.ga, 2 * d, second(d), A.Pp, dsm + L.ga);
+        duo_fetch_pos(A.cv, 2 * d, second(d), N, v);
+    }
+    for (int k = threadIdx.x; k < N; k += T) gam[k * gamma_stride(N) + k] = make_float2(0.0f, 0.0f);
+    for (; d < D; d += gridDim.x) {
+        const int m0 = 2 * d, m1 = second(d);
+        duo_store_pos(A.cv, N, v, q);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        const long long src0 = config_index(A.cv, m0), src1 = config_index(A.cv, m1);
+        duo_gamma(q, ga, A.pairs, A.inv_sd, A.P, A.Pp, N, gam);
+        __syncthreads();
+        const int nd = d + gridDim.x;
+        if (nd < D) {
+            duo_fetch_rows(A.ga, 2 * nd, second(nd), A.Pp, dsm + L.ga);
+            duo_fetch_pos(A.cv, 2 * nd, second(nd), N, v);
+        }
+        // One thread per atom and coordinate sums a whole row in order: the BF16
+        // rounding of nu_a turns a different order into flips of a bit.
+        double sq0 = 0.0, sq1 = 0.0;
+        if (threadIdx.x < 3 * N) {
+            const int c = threadIdx.x / N, k = threadIdx.x - c * N;
+            const float2* xc = c == 0 ? xs : c == 1 ? xs + 1 : q.z;
+            const int sx = c < 2 ? 2 : 1;
+            const float2 xk = xc[sx * k], m1 = make_float2(-1.0f, -1.0f);
+            const float2* row = gam + k * gamma_stride(N);
+            float2 f = make_float2(0.0f, 0.0f);
+#pragma unroll 5
+            for (int j = 0; j < N; ++j) f = __ffma2_rn(row[j], __ffma2_rn(m1, xc[sx * j], xk), f);
+            const float d0 = f.x - (float)(A.F_ref[src0 * 3 * N + 3 * k + c] * inv_sE);
+            const float d1 = f.y - (float)(A.F_ref[src1 * 3 * N + 3 * k + c] * inv_sE);
+            us.put(0, k, c, cu * d0);
+            us.put(1, k, c, cu * d1);
+            sq0 = (double)d0 * d0;
+            sq1 = (double)d1 * d1;
+        }
+        sq0 = block_sum(sq0, red);
+        sq1 = block_sum(sq1, red);  // also orders the writes of us before the reads below
+        if ((threadIdx.x & 31) == 0 && threadIdx.x < 64 && (threadIdx.x == 0 || m1 != m0)) {
+            const int m = threadIdx.x ? m1 : m0;
+            const double e = head_energy(A.part, A.nparts, m, A.b3);
+            const double de = e - (A.E_ref[threadIdx.x ? src1 : src0] - A.mu_E) * inv_sE;
+            A.ebar[m] = (float)(2.0 * de / (double)A.M);
+            A.loss_part[m] = de * de + A.lam / (3.0 * N) * (threadIdx.x ? sq1 : sq0);
+        }
+        __nv_bfloat16* nrow = A.nu_a + (size_t)m0 * A.Pp;
+#pragma unroll 2
+        for (int p = threadIdx.x; p < A.Pp; p += T) {
+            float2 w = make_float2(0.0f, 0.0f);
+            if (p < A.P) {
+                const ushort2 ij = A.pairs[p];
+                const float isd = A.inv_sd[p];
+                const Duo3 dx = duo_diff(q.xy[ij.x], q.z[ij.x], q.xy[ij.y], q.z[ij.y]);
+                const Duo3 du = duo_diff(us.xy[ij.x], us.z[ij.x], us.xy[ij.y], us.z[ij.y]);
+                const float2 r2 = __ffma2_rn(dx.z, dx.z, __ffma2_rn(dx.x, dx.x, __fmul2_rn(dx.y, dx.y)));
+                const float2 ir = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+                w = __ffma2_rn(dx.z, du.z, __ffma2_rn(dx.x, du.x, __fmul2_rn(dx.y, du.y)));
+                w = __fmul2_rn(__fmul2_rn(__fmul2_rn(__fmul2_rn(w, ir), ir), ir), make_float2(isd, isd));
+            }
+            nrow[p] = __float2bfloat16(w.x);
+            if (m1 != m0) nrow[A.Pp + p] = __float2bfloat16(w.y);
+        }
+        __syncthreads();  // q and us are read until here
+    }
+}
+
+using LossKernel = void (*)(const LossArgs);
+LossKernel loss_duo_kernel(int N) {
+    const int t = duo_threads(N);
+    return t == 64 ? mlp_loss_duo_kernel<64> : t == 128 ? mlp_loss_duo_kernel<128> : mlp_loss_duo_kernel<384>;
+}
+
+// The same for molecules past gamma_matrix(N).
 __global__ void __launch_bounds__(kMlpThreads) mlp_loss_kernel(const LossArgs L) {
     extern __shared__ float lsm[];
     __shared__ double red[32];
@@ -529,18 +581,17 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_loss_kernel(const LossArgs L)
     float* gam = lsm + 6 * kXs;
     const double inv_sE = 1.0 / L.sigma_E;
     const float cu = (float)(2.0 * L.lam / (3.0 * L.N * (double)L.M));
-    init_gamma(L.N, gam);
     for (int m = blockIdx.x; m < L.M; m += gridDim.x) {
         __syncthreads();
         load_config(L.cv, m, L.N, xs);
         __syncthreads();
-        load_gamma(xs, L.ga + (size_t)m * L.Pp, L.inv_sd, L.pairs, L.P, L.N, gam);
+        load_gamma(L.ga + (size_t)m * L.Pp, L.inv_sd, L.P, gam);
         __syncthreads();
         const long long src = config_index(L.cv, m);
         const float* Fr = L.F_ref + src * 3 * L.N;
         double sq = 0.0;
         for (int k = threadIdx.x; k < L.N; k += blockDim.x) {
-            const float3 a = atom_force_any(k, xs, gam, L.N);
+            const float3 a = atom_force(k, xs, gam, L.N);
             const float dfx = a.x - (float)(Fr[3 * k] * inv_sE);
             const float dfy = a.y - (float)(Fr[3 * k + 1] * inv_sE);
             const float dfz = a.z - (float)(Fr[3 * k + 2] * inv_sE);
@@ -739,15 +790,17 @@ int pack(pamd_mlp* m) {
     return launch_check(m, "weight pack");
 }
 
-size_t forces_smem(const pamd_mlp* m) { return sizeof(float) * (3 * kXs + (size_t)gamma_floats(m->N, m->Pp)); }
-size_t loss_smem(const pamd_mlp* m) { return sizeof(float) * (6 * kXs + (size_t)gamma_floats(m->N, m->Pp)); }
+size_t forces_smem(const pamd_mlp* m) { return sizeof(float) * (3 * kXs + (size_t)m->Pp); }
+size_t loss_smem(const pamd_mlp* m) { return sizeof(float) * (6 * kXs + (size_t)m->Pp); }
 
 // The dynamic shared-memory limits of the force and loss kernels on the
 // current device, raised to what this model needs.
 int set_smem_attrs(const pamd_mlp* m) {
     cudaError_t e = gamma_matrix(m->N) ? ensure_dyn_smem((const void*)forces_duo_kernel(m->N), duo_smem(m->N, m->Pp).total)
                                        : ensure_dyn_smem((const void*)mlp_forces_kernel, forces_smem(m));
-    if (e == cudaSuccess) e = ensure_dyn_smem((const void*)mlp_loss_kernel, loss_smem(m));
+    if (e == cudaSuccess)
+        e = gamma_matrix(m->N) ? ensure_dyn_smem((const void*)loss_duo_kernel(m->N), loss_duo_smem(m->N, m->Pp))
+                               : ensure_dyn_smem((const void*)mlp_loss_kernel, loss_smem(m));
     return e == cudaSuccess ? PAMD_OK : mfail(PAMD_ECUDA, std::string("kernel attributes: ") + cudaGetErrorString(e));
 }
 
@@ -1210,7 +1263,13 @@ int pamd_mlp_loss_grads(pamd_mlp* m, const float* x_dev, const double* E_dev, co
     L.nu_a = nu_a;
     L.ebar = w.ebar;
     L.loss_part = w.loss_part;
-    mlp_loss_kernel<<<grid_for(M * kMlpThreads, kMlpThreads, 152 * 16), kMlpThreads, loss_smem(m), s>>>(L);
+    if (gamma_matrix(m->N)) {
+        const int t = duo_threads(m->N);
+        loss_duo_kernel(m->N)<<<grid_for((M + 1) / 2 * t, t, 152 * (t == 384 ? 3 : 1024 / t)), t,
+                                loss_duo_smem(m->N, m->Pp), s>>>(L);
+    } else {
+        mlp_loss_kernel<<<grid_for(M * kMlpThreads, kMlpThreads, 152 * 16), kMlpThreads, loss_smem(m), s>>>(L);
+    }
     if ((rc = launch_check(m, "loss"))) return rc;
     // tangent pass: zd1 = W1 nu_a, hd1 = zd1 s1, zd2 = W2 hd1
     g = GemmArgs{};

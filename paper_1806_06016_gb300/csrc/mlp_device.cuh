@@ -119,64 +119,19 @@ __device__ __forceinline__ float3 atom_force(int k, const float* xs, const float
 }
 
 // Molecules of up to kGammaMatrixMax atoms use a symmetric N x N shared-
-// memory matrix (odd row stride: the atoms of a warp hit distinct banks)
-// holding c_ij = gam_ij / r_ij^3, filled by one pass over the pairs (one
-// rsqrt per pair), so that the force of atom k is the plain row sum
-// F_k = sum_j c_kj (x_k - x_j).  Larger molecules keep gam per pair and use
-// atom_force.  The diagonal is zero (set once per block, never written by
-// the pair pass).
+// memory matrix c_ij = gam_ij / r_ij^3 per configuration, filled by one pass
+// over the pairs (one rsqrt per pair), so that the force of atom k is the
+// plain row sum F_k = sum_j c_kj (x_k - x_j).  Larger molecules keep gam per
+// pair and use atom_force.
 constexpr int kGammaMatrixMax = 128;
 
 __host__ __device__ __forceinline__ bool gamma_matrix(int N) { return N <= kGammaMatrixMax; }
 __host__ __device__ __forceinline__ int gamma_stride(int N) { return N | 1; }
 
-// floats of shared memory the table of an N-atom molecule takes
-__host__ __device__ __forceinline__ int gamma_floats(int N, int Pp) {
-    return gamma_matrix(N) ? N * gamma_stride(N) : Pp;
-}
-
-// zero diagonal of the matrix (whole block; once per block)
-__device__ __forceinline__ void init_gamma(int N, float* gam) {
-    if (gamma_matrix(N))
-        for (int k = threadIdx.x; k < N; k += blockDim.x) gam[k * gamma_stride(N) + k] = 0.0f;
-}
-
-// fill the table from de/da of one configuration (whole block)
-__device__ __forceinline__ void load_gamma(const float* xs, const __nv_bfloat16* __restrict__ ga_row,
-                                           const float* __restrict__ inv_sd,
-                                           const ushort2* __restrict__ pairs, int P, int N, float* gam) {
-    if (gamma_matrix(N)) {
-        const int S = gamma_stride(N);
-#pragma unroll 4
-        for (int p = threadIdx.x; p < P; p += blockDim.x) {
-            const ushort2 ij = pairs[p];
-            const float dx = xs[ij.x] - xs[ij.y];
-            const float dy = xs[kXs + ij.x] - xs[kXs + ij.y];
-            const float dz = xs[2 * kXs + ij.x] - xs[2 * kXs + ij.y];
-            const float ir = rsqrtf(fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
-            const float c = __bfloat162float(ga_row[p]) * inv_sd[p] * ir * ir * ir;
-            gam[ij.x * S + ij.y] = c;
-            gam[ij.y * S + ij.x] = c;
-        }
-    } else {
-        for (int p = threadIdx.x; p < P; p += blockDim.x) gam[p] = __bfloat162float(ga_row[p]) * inv_sd[p];
-    }
-}
-
-// sum over j != k of gam_kj (x_k - x_j) / r_kj^3 with the table of load_gamma
-__device__ __forceinline__ float3 atom_force_any(int k, const float* xs, const float* gam, int N) {
-    if (!gamma_matrix(N)) return atom_force(k, xs, gam, N);
-    const float xk = xs[k], yk = xs[kXs + k], zk = xs[2 * kXs + k];
-    const float* row = gam + k * gamma_stride(N);
-    float fx = 0.0f, fy = 0.0f, fz = 0.0f;
-#pragma unroll 4
-    for (int j = 0; j < N; ++j) {
-        const float c = row[j];
-        fx = fmaf(c, xk - xs[j], fx);
-        fy = fmaf(c, yk - xs[kXs + j], fy);
-        fz = fmaf(c, zk - xs[2 * kXs + j], fz);
-    }
-    return make_float3(fx, fy, fz);
+// gam_p = de/dg_p of one configuration (whole block)
+__device__ __forceinline__ void load_gamma(const __nv_bfloat16* __restrict__ ga_row, const float* __restrict__ inv_sd,
+                                           int P, float* gam) {
+    for (int p = threadIdx.x; p < P; p += blockDim.x) gam[p] = __bfloat162float(ga_row[p]) * inv_sd[p];
 }
 
 // The symmetric matrix c_ij = gam_ij / r_ij^3 of two configurations (odd row
@@ -217,13 +172,55 @@ __device__ __forceinline__ Duo3 duo_force(int k, const DuoPos& q, const float2* 
     return f;
 }
 
+// Block size: as many threads as a row split over up to eight keeps busy.
+// Small molecules in 384 threads leave most idle at the barriers (65536
+// configurations of 9 atoms, whole call: 210 us, in 64 threads 131; 16384 of
+// 22: 102 and, in 128, 87).
+constexpr int kDuoPartsMax = 8;
+constexpr int kDuoElems = 2;  // coordinates per thread: 6 N <= 2 threads
+
+__host__ __device__ __forceinline__ int duo_threads(int N) { return N <= 21 ? 64 : N <= 42 ? 128 : 384; }
+static_assert(6 * 21 <= kDuoElems * 64 && 6 * 42 <= kDuoElems * 128 && 6 * kGammaMatrixMax <= kDuoElems * 384, "");
+__host__ __device__ __forceinline__ int duo_parts(int N) {
+    return duo_threads(N) / N < kDuoPartsMax ? duo_threads(N) / N : kDuoPartsMax;
+}
+
+// queue the copies of two rows of Pp BF16 values (16-byte multiples) to dst
+__device__ __forceinline__ void duo_fetch_rows(const __nv_bfloat16* ga, int m0, int m1, int Pp, unsigned char* dst) {
+    const int n = Pp / 8;
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    for (int t = threadIdx.x; t < 2 * n; t += blockDim.x) {
+        const __nv_bfloat16* src = ga + (size_t)(t < n ? m0 : m1) * Pp + 8 * (t < n ? t : t - n);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + 16 * t), "l"(src) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// the row sums of both configurations, each row in `parts` consecutive pieces:
+// part[h][b][k][c], parts N <= blockDim.x
+__device__ __forceinline__ void duo_force_parts(const DuoPos& q, const float2* gam, int N, int parts, float* part) {
+    const int len = (N + parts - 1) / parts;
+    const int h = threadIdx.x / N, k = threadIdx.x - h * N;
+    if (h >= parts) return;
+    const int j0 = min(h * len, N), j1 = min(N, j0 + len);
+    const Duo3 s = duo_force(k, q, gam, N, j0, j1);
+    float* o = part + (size_t)h * 6 * N + 3 * k;
+    o[0] = s.x.x;
+    o[1] = s.y.x;
+    o[2] = s.z.x;
+    o += 3 * N;
+    o[0] = s.x.y;
+    o[1] = s.y.y;
+    o[2] = s.z.y;
+}
+__device__ __forceinline__ float duo_force_sum(const float* part, int N, int parts, int t) {
+    float v = part[t];
+    for (int h = 1; h < parts; ++h) v += part[h * 6 * N + t];
+    return v;
+}
+
 // ------------------------------------------------ pair passes of the MD step kernel
-// Consecutive threads take consecutive row-order pairs, so that the lanes of
-// a warp read consecutive atoms (no shared-memory bank conflicts) and
-// consecutive table entries.  The pair table (i, j) and the per-pair tables
-// may sit in shared or global memory.  Positions sit in shared memory as
-// float4 (x, y, z, 0).  The arithmetic of every pair is that of
-// duo_feature / load_gamma / atom_force_any, bit for bit.
+// past gamma_matrix(N).  Positions sit in shared memory as float4 (x, y, z, 0).
 
 __host__ __device__ __forceinline__ size_t step_pos_bytes(int N) { return 16 * (size_t)(N + 1); }
 
@@ -252,75 +249,22 @@ __device__ __forceinline__ void pass_features(const float4* xs4, const ushort2* 
     }
 }
 
-// the table of load_gamma from de/da of the configuration in xs4 (whole block)
-__device__ __forceinline__ void pass_gamma(const float4* xs4, const ushort2* pij, int P, int N,
-                                           const __nv_bfloat16* ga_row, const float* inv_sd, float* gam) {
-    if (!gamma_matrix(N)) {
-        for (int p = threadIdx.x; p < P; p += blockDim.x) gam[p] = __bfloat162float(ga_row[p]) * inv_sd[p];
-        return;
-    }
-    const int S = gamma_stride(N);
-#pragma unroll 4
-    for (int p = threadIdx.x; p < P; p += blockDim.x) {
-        const ushort2 ij = pij[p];
-        const float ir = inv_dist4(xs4[ij.x], xs4[ij.y]);
-        const float c = __bfloat162float(ga_row[p]) * inv_sd[p] * ir * ir * ir;
-        gam[ij.x * S + ij.y] = c;
-        gam[ij.y * S + ij.x] = c;
-    }
-}
-
-// sum over j != k of gam_kj (x_k - x_j) / r_kj^3 (atom_force_any on xs4)
+// sum over j != k of gam_kj (x_k - x_j) / r_kj^3 (atom_force on xs4)
 __device__ __forceinline__ float3 atom_force4(int k, const float4* xs4, const float* gam, int N) {
     const float4 xk = xs4[k];
     float fx = 0.0f, fy = 0.0f, fz = 0.0f;
-    if (!gamma_matrix(N)) {
-        for (int j = 0; j < N; ++j) {
-            if (j == k) continue;
-            const int p = k < j ? pair_id(k, j, N) : pair_id(j, k, N);
-            const float4 xj = xs4[j];
-            const float dx = xk.x - xj.x, dy = xk.y - xj.y, dz = xk.z - xj.z;
-            const float ir = rsqrtf(fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
-            const float c = gam[p] * ir * ir * ir;
-            fx = fmaf(c, dx, fx);
-            fy = fmaf(c, dy, fy);
-            fz = fmaf(c, dz, fz);
-        }
-        return make_float3(fx, fy, fz);
-    }
-    const float* row = gam + k * gamma_stride(N);
-    // x and y as one packed pair: d = x_k - x_j (a multiply by -1 is exact,
-    // so the fused form rounds like the subtraction), f += c d
-    float2 fxy = make_float2(0.0f, 0.0f);
-    const float2 xky = make_float2(xk.x, xk.y), m1 = make_float2(-1.0f, -1.0f);
-#pragma unroll 5
     for (int j = 0; j < N; ++j) {
-        const float c = row[j];
+        if (j == k) continue;
+        const int p = k < j ? pair_id(k, j, N) : pair_id(j, k, N);
         const float4 xj = xs4[j];
-        const float2 d = __ffma2_rn(m1, make_float2(xj.x, xj.y), xky);
-        fxy = __ffma2_rn(make_float2(c, c), d, fxy);
-        fz = fmaf(c, xk.z - xj.z, fz);
+        const float dx = xk.x - xj.x, dy = xk.y - xj.y, dz = xk.z - xj.z;
+        const float ir = rsqrtf(fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
+        const float c = gam[p] * ir * ir * ir;
+        fx = fmaf(c, dx, fx);
+        fy = fmaf(c, dy, fy);
+        fz = fmaf(c, dz, fz);
     }
-    return make_float3(fxy.x, fxy.y, fz);
-}
-
-// the terms j0 <= j < j1 of atom_force4's matrix-form sum (same arithmetic)
-__device__ __forceinline__ float3 atom_force4_range(int k, const float4* xs4, const float* gam, int N, int j0,
-                                                    int j1) {
-    const float4 xk = xs4[k];
-    const float* row = gam + k * gamma_stride(N);
-    float2 fxy = make_float2(0.0f, 0.0f);
-    float fz = 0.0f;
-    const float2 xky = make_float2(xk.x, xk.y), m1 = make_float2(-1.0f, -1.0f);
-#pragma unroll 5
-    for (int j = j0; j < j1; ++j) {
-        const float c = row[j];
-        const float4 xj = xs4[j];
-        const float2 d = __ffma2_rn(m1, make_float2(xj.x, xj.y), xky);
-        fxy = __ffma2_rn(make_float2(c, c), d, fxy);
-        fz = fmaf(c, xk.z - xj.z, fz);
-    }
-    return make_float3(fxy.x, fxy.y, fz);
+    return make_float3(fx, fy, fz);
 }
 
 // normalised energy e = b3 + sum of the layer-2 partial sums

@@ -5,7 +5,11 @@ batch size (one, two or eight configurations to a block) or on the batch's
 last odd one: equal bit for bit.  Forces against the FP64 oracle with
 BF16-rounded weights, over the sizes where the row sums split differently and
 at the limit of the matrix form, to 2e-2 of the RMS force (BF16 roundings of
-2^-9 each on a path of three layers).
+2^-9 each on a path of three layers); loss gradients to 3e-2 of each block's
+norm, as two more products lie on their path.  MD steps: a replica's path does
+not depend on its partner or on an odd last one, bit for bit, and follows the
+oracle's to 1e-4 nm (a relative force error of 2e-2 at the 1e4 kJ/mol/nm of
+this model moves 1 u by 2e-4 (dt theta)^2 = 1.8e-9 x 1e4 nm in three steps).
 """
 import numpy as np
 import pytest
@@ -77,5 +81,56 @@ def test_large_batches_equal_small_ones(env, n):
         assert torch.equal(E[last], e[last % 37]) and torch.equal(F[last], f[last % 37])
         E2, _ = model.energy_forces(xd, forces=False)
         assert torch.equal(E, E2)
+    finally:
+        model.close()
+
+
+@pytest.mark.parametrize("n", [31, 48, 97, 128, 130])
+def test_loss_gradients_over_the_row_splits(env, n):
+    torch, S = env
+    M = 8
+    x = pi.perturbed_positions(pi.make_chain(n, 4), M, 0.02, 2).astype(np.float32)
+    model, q = _model(S, n, x)
+    try:
+        rng = np.random.default_rng(M)
+        E = -40.0 + 15.0 * rng.normal(0, 1, M)
+        F = rng.normal(0, 200.0, (M, n, 3)).astype(np.float32)
+        loss = model.loss_grads(torch.from_numpy(x).cuda(), torch.from_numpy(E).cuda(), torch.from_numpy(F).cuda(), lam=0.8)
+        got = model.get_grads()
+        want_loss, want = omlp.loss_and_grads(q, x.astype(np.float64), E, F.astype(np.float64), 0.8)
+        assert abs(loss - want_loss) <= 3e-2 * abs(want_loss)
+        for k in ("W1", "b1", "W2", "b2", "w3"):
+            assert np.linalg.norm(got[k] - want[k]) <= 3e-2 * np.linalg.norm(want[k]), k
+    finally:
+        model.close()
+
+
+@pytest.mark.parametrize("n", [5, 21, 22, 42, 43, 85, 86, 128, 129])
+def test_steps_at_block_sizes(env, n):
+    torch, S = env
+    from paper_1806_06016_gb300 import pamd
+    theta, dt, T, seed = 3, 0.001, 600.0, 31
+    top = pi.make_chain(n, 2)
+    model, q = _model(S, n, pi.perturbed_positions(top, 32, 0.03, 5).astype(np.float32))
+    out = {}
+    try:
+        for R in (6, 7):
+            ctx = pamd.pamd_init(top, R, T, seed)
+            try:
+                x0, v0, _, _ = pamd.pamd_get_state(ctx)
+                S.attach(ctx, model)
+                pamd.pamd_propagate(ctx, theta, dt, T)
+                out[R] = (x0, v0) + pamd.pamd_get_state(ctx)[:3] + (pamd.pamd_observables(ctx, T),)
+            finally:
+                pamd.pamd_destroy(ctx)
+        for a, b in zip(out[6][:5], out[7][:5]):
+            np.testing.assert_array_equal(a, b[:6])
+        x0, v0, x1, _, E1, obs = out[7]
+        slots = np.arange(7)
+        xo, _, Eo = omlp.propagate(q, x0, v0, top.mass, theta, dt, T, 1.0, seed, 0, slots=slots)
+        assert np.abs(x1 - xo).max() < 1e-4
+        assert np.abs(E1 - Eo).max() <= 2e-2 * q["sigma_E"]
+        rg = np.sqrt(((x1 - x1.mean(1, keepdims=True)) ** 2).sum(-1).mean(1))
+        assert abs(obs["rg"] - rg.mean()) <= 1e-6 * rg.mean()
     finally:
         model.close()

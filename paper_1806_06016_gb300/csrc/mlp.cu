@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_forces_kernel(const ForceArgs
 // nu_a = dL/d(de/da) = (J u) / sd with (J u)_p = (x_i - x_j).(u_i - u_j) / r^3.
 // Two samples at a time like the force kernel, with a second pass over the
 // pairs for J u; bound likewise by shared-memory wavefronts and barriers.
-// 2048 samples of 75 atoms: 61 us (one at a time, 75 of 128 threads at the
+// 2048 samples of 75 atoms: 44 us (one at a time, 75 of 128 threads at the
 // force rows: 70).
 // Shared memory: that of the force kernel with dL/df in the place of the partial sums.
 __host__ __device__ __forceinline__ size_t loss_duo_smem(int N, int Pp) {
@@ -536,14 +536,25 @@ __global__ void __launch_bounds__(T, T == 384 ? 3 : 1024 / T) mlp_loss_duo_kerne
             sq0 = (double)d0 * d0;
             sq1 = (double)d1 * d1;
         }
-        sq0 = block_sum(sq0, red);
-        sq1 = block_sum(sq1, red);  // also orders the writes of us before the reads below
+        // the two sums of squares: half a warp each, then one thread each adds the
+        // warps' (FP64 instructions cost 20 clocks of the SM: block-wide sums in
+        // every warp were half of this kernel)
+        const int lane = threadIdx.x & 31, nw = (3 * N + 31) / 32;
+        if ((int)(threadIdx.x >> 5) < nw) {
+            const bool hi = lane & 16;
+            double t = (hi ? sq1 : sq0) + __shfl_xor_sync(0xffffffffu, hi ? sq0 : sq1, 16);
+            for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if ((lane & 15) == 0) red[lane + (threadIdx.x >> 5)] = t;
+        }
+        __syncthreads();  // also orders the writes of us before the reads below
         if ((threadIdx.x & 31) == 0 && threadIdx.x < 64 && (threadIdx.x == 0 || m1 != m0)) {
             const int m = threadIdx.x ? m1 : m0;
+            double sq = 0.0;
+            for (int w = 0; w < nw; ++w) sq += red[(threadIdx.x ? 16 : 0) + w];
             const double e = head_energy(A.part, A.nparts, m, A.b3);
             const double de = e - (A.E_ref[threadIdx.x ? src1 : src0] - A.mu_E) * inv_sE;
             A.ebar[m] = (float)(2.0 * de / (double)A.M);
-            A.loss_part[m] = de * de + A.lam / (3.0 * N) * (threadIdx.x ? sq1 : sq0);
+            A.loss_part[m] = de * de + A.lam / (3.0 * N) * sq;
         }
         __nv_bfloat16* nrow = A.nu_a + (size_t)m0 * A.Pp;
 #pragma unroll 2

@@ -23,7 +23,7 @@
 //     commits the accumulator when a tile's last product is issued;
 //   * warps 2..9 drain a finished accumulator with tcgen05.ld (warp w reads
 //     tensor-memory lanes 32 (w mod 4) ..), apply the bias and the layer's
-//     output transform, store with 16-byte vector stores, and hand the
+//     output transform, store through shared memory, and hand the
 //     accumulator back -- so the epilogue of one tile runs while the tensor
 //     core works on the next.
 //
@@ -33,7 +33,7 @@
 // the ring as a whole with an elected lane issuing, which spares the issue
 // loops over lanes that a single-lane branch costs (per 64 of K at BN = 64:
 // 0.41 us before, 0.15 now; 512 x 8192 x 64: 59.5 -> 28.8 us; 65536 x 512 x
-// 2776 at BN = 256: 178 -> 169 us, 1.10 PFLOP/s).
+// 2776 at BN = 256: 178 -> 169 us, and 150 with the stores below, 1.24 PFLOP/s).
 //
 // Every wait on an mbarrier is bounded: after kWaitLimit polls the waiting
 // role records PAMD_ETIMEOUT and raises a shared abort flag, the others stop
@@ -61,6 +61,7 @@ constexpr int kBK = 64;   // contraction depth of one operand tile (128 bytes of
 constexpr int kEpiWarps = 8, kThreads = 64 + 32 * kEpiWarps, kEpiThreads = 32 * kEpiWarps;
 constexpr int kTileA = kBM * kBK * 2;  // 16 KiB
 constexpr int kRingBytes = 192 * 1024;
+constexpr int kEpiStage = 4096;  // shared memory of one epilogue warp, after the ring
 constexpr uint32_t kWaitLimit = 1u << 22;
 
 // Per tile width BN: bytes of a B tile and a stage [A A | B B], stages of the
@@ -249,49 +250,102 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
 
 __device__ __forceinline__ float sigmoid(float z) { return __fdividef(1.0f, 1.0f + __expf(-z)); }
 
-// 32 consecutive FP32 values of one row: vector stores when the whole chunk
-// is inside the matrix and 16-byte aligned, else element by element
-__device__ __forceinline__ void store_row32(float* dst, const float (&v)[32], int n, bool vec) {
-    if (vec && n == 32) {
-        float4* d = reinterpret_cast<float4*>(dst);
+// the first n of 32 consecutive values of one row
+__device__ __forceinline__ void store_row32(float* dst, const float (&v)[32], int n) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) d[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-    } else {
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-            if (j < n) dst[j] = v[j];
-    }
+    for (int j = 0; j < 32; ++j)
+        if (j < n) dst[j] = v[j];
 }
 
-__device__ __forceinline__ void store_row32_bf16(__nv_bfloat16* dst, const float (&v)[32], int n,
-                                                 bool vec) {
-    if (vec && n == 32) {
-        uint4* d = reinterpret_cast<uint4*>(dst);
+__device__ __forceinline__ void store_row32_bf16(__nv_bfloat16* dst, const float (&v)[32], int n) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            uint32_t w[4];
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const __nv_bfloat162 h = __floats2bfloat162_rn(v[8 * q + 2 * t], v[8 * q + 2 * t + 1]);
-                w[t] = *reinterpret_cast<const uint32_t*>(&h);
-            }
-            d[q] = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-            if (j < n) dst[j] = __float2bfloat16(v[j]);
-    }
+    for (int j = 0; j < 32; ++j)
+        if (j < n) dst[j] = __float2bfloat16(v[j]);
 }
 
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
+// 32 rows x 32 columns of a warp through its 4 KiB of shared memory, so that
+// global memory sees whole 128- (FP32) or 64-byte (BF16) row pieces instead of
+// 16 bytes in each of 32 rows.  The 16-byte slots of a row are swizzled: writes
+// by row and reads across rows are both free of bank conflicts.  65536 x 2776 x
+// 512 with FP32 results: 331 -> 182 us, 65536 x 512 x 512: 64 -> 43 us.
+__device__ __forceinline__ uint4* slot_f32(unsigned char* st, int r, int q) {
+    return reinterpret_cast<uint4*>(st + r * 128 + ((q ^ (r & 7)) << 4));
+}
+__device__ __forceinline__ uint4* slot_b16(unsigned char* st, int r, int q) {
+    return reinterpret_cast<uint4*>(st + r * 64 + ((q ^ ((r >> 1) & 3)) << 4));
+}
+
+// dst: row 0 of the warp's 32, column 0 of the 32; rows of them exist
+__device__ __forceinline__ void store_block_f32(float* dst, int ld, int rows, const float (&v)[32], unsigned char* st) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+        *reinterpret_cast<float4*>(slot_f32(st, lane, q)) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    __syncwarp();
+#pragma unroll
+    for (int it = 0; it < 8; ++it) {
+        const int r = 4 * it + (lane >> 3);
+        const uint4 w = *slot_f32(st, r, lane & 7);
+        if (r < rows) *reinterpret_cast<uint4*>(dst + (size_t)r * ld + 4 * (lane & 7)) = w;
+    }
+}
+
+__device__ __forceinline__ void store_block_bf16(__nv_bfloat16* dst, int ld, int rows, const float (&v)[32], unsigned char* st) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        uint32_t w[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const __nv_bfloat162 h = __floats2bfloat162_rn(v[8 * q + 2 * t], v[8 * q + 2 * t + 1]);
+            w[t] = *reinterpret_cast<const uint32_t*>(&h);
+        }
+        *slot_b16(st, lane, q) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+        const int r = 8 * it + (lane >> 2);
+        const uint4 w = *slot_b16(st, r, lane & 3);
+        if (r < rows) *reinterpret_cast<uint4*>(dst + (size_t)r * ld + 8 * (lane & 3)) = w;
+    }
+}
+
+// v *= the same block of src
+__device__ __forceinline__ void mul_block_f32(const float* src, int ld, int rows, float (&v)[32], unsigned char* st) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+#pragma unroll
+    for (int it = 0; it < 8; ++it) {
+        const int r = 4 * it + (lane >> 3);
+        if (r < rows) *slot_f32(st, r, lane & 7) = *reinterpret_cast<const uint4*>(src + (size_t)r * ld + 4 * (lane & 7));
+    }
+    __syncwarp();
+    if (lane < rows) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float4 t = *reinterpret_cast<const float4*>(slot_f32(st, lane, q));
+            v[4 * q] *= t.x;
+            v[4 * q + 1] *= t.y;
+            v[4 * q + 2] *= t.z;
+            v[4 * q + 3] *= t.w;
+        }
+    }
+}
+
 // Epilogue of `chunks` x 32 columns of a tile: accumulator columns of this
-// warp's 32 tensor-memory lanes (rows m0 + 32q + lane); taddr and n0 point at
-// the first column.
-__device__ __forceinline__ void epilogue_tile(const GemmArgs& g, uint32_t taddr, int row, int n0, int chunks) {
+// warp's 32 tensor-memory lanes (rows row0 + lane); taddr and n0 point at the
+// first column, st at the warp's shared memory.  Full, aligned blocks of 32
+// columns go to memory through it; the rest element by element.
+__device__ __forceinline__ void epilogue_tile(const GemmArgs& g, uint32_t taddr, int row0, int n0, int chunks,
+                                              unsigned char* st) {
+    const int row = row0 + (threadIdx.x & 31), rows = g.M - row0;
     const bool row_ok = row < g.M;
     float head = 0.0f;
     __nv_bfloat16* Cb = static_cast<__nv_bfloat16*>(g.Cb);
@@ -302,13 +356,18 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs& g, uint32_t taddr,
         tmem_ld32(taddr + (uint32_t)(cc * 32), v);
         const int col0 = n0 + cc * 32;
         const int n = min(32, g.N - col0);
-        if (!row_ok || n <= 0) continue;
+        if (rows <= 0 || n <= 0) continue;
+        const bool bf = vf && n == 32, bb = vb && n == 32;
+        const int ns = row_ok ? n : 0;  // of the element-wise forms
         if (g.bias) {
 #pragma unroll
             for (int j = 0; j < 32; ++j) v[j] += (j < n) ? g.bias[col0 + j] : 0.0f;
         }
-        const size_t o = (size_t)row * g.ldc + col0;
-        if (g.C) store_row32(g.C + o, v, n, vf);
+        const size_t o = (size_t)row * g.ldc + col0, o0 = (size_t)row0 * g.ldc + col0;
+        if (g.C) {
+            if (bf) store_block_f32(g.C + o0, g.ldc, rows, v, st);
+            else store_row32(g.C + o, v, ns);
+        }
         if (g.epi == kEpiSilu || g.epi == kEpiHead) {
             float ds[32];
 #pragma unroll
@@ -317,7 +376,10 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs& g, uint32_t taddr,
                 ds[j] = sg * (1.0f + v[j] * (1.0f - sg));
                 v[j] *= sg;  // silu
             }
-            if (g.Cs) store_row32(g.Cs + o, ds, n, vf);
+            if (g.Cs) {
+                if (bf) store_block_f32(g.Cs + o0, g.ldc, rows, ds, st);
+                else store_row32(g.Cs + o, ds, ns);
+            }
             if (g.epi == kEpiHead) {
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
@@ -327,22 +389,17 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs& g, uint32_t taddr,
                 }
             }
         } else if (g.epi == kEpiMul) {
-            const float* mr = g.mul + o;
-            if (vf && n == 32) {
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const float4 t = reinterpret_cast<const float4*>(mr)[q];
-                    v[4 * q] *= t.x;
-                    v[4 * q + 1] *= t.y;
-                    v[4 * q + 2] *= t.z;
-                    v[4 * q + 3] *= t.w;
-                }
+            if (bf) {
+                mul_block_f32(g.mul + o0, g.ldc, rows, v, st);
             } else {
 #pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] *= (j < n) ? mr[j] : 0.0f;
+                for (int j = 0; j < 32; ++j) v[j] *= (j < ns) ? g.mul[o + j] : 0.0f;
             }
         }
-        if (Cb) store_row32_bf16(Cb + (size_t)row * g.ldcb + col0, v, n, vb);
+        if (Cb) {
+            if (bb) store_block_bf16(Cb + (size_t)row0 * g.ldcb + col0, g.ldcb, rows, v, st);
+            else store_row32_bf16(Cb + (size_t)row * g.ldcb + col0, v, ns);
+        }
     }
     // one partial sum of the head per 128 columns; a tile of 128 columns that
     // is the last one writes the zero of the missing other half as well
@@ -367,7 +424,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     __shared__ int s_abort, s_issued, s_consumed;
     // 1024-byte aligned stages: [A0 | B0 | A1 | B1 | ...]
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = tid >> 5;
     // The two CTAs of a cluster take row blocks 2p and 2p + 1 of the same
     // column block: each loads its A tile and half of the shared B tile,
     // multicast to both.
@@ -528,6 +585,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     } else {  // epilogue warps 2..9
         const int q = warp & 3;  // tensor-memory lane quarter this warp may access
         const int half = (warp - 2) >> 2;
+        unsigned char* stage = smem_raw + (base - smem_u32(smem_raw)) + kRingBytes + (warp - 2) * kEpiStage;
         int i = 0;
         for (int t = cid; t < tiles; t += ncl, ++i) {
             const int acc = i & 1;
@@ -541,10 +599,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             // the head's partial sums run over 128 columns: with a tile that
             // narrow one warp per quarter takes them all
             if (BN == 128 && g.epi == kEpiHead) {
-                if (half == 0) epilogue_tile(g, taddr, m0 + q * 32 + lane, nt * kBN, BN / 32);
+                if (half == 0) epilogue_tile(g, taddr, m0 + q * 32, nt * kBN, BN / 32, stage);
             } else {
-                epilogue_tile(g, taddr + (uint32_t)(half * (kBN / 2)), m0 + q * 32 + lane, nt * kBN + half * (kBN / 2),
-                              BN / 64);
+                epilogue_tile(g, taddr + (uint32_t)(half * (kBN / 2)), m0 + q * 32, nt * kBN + half * (kBN / 2),
+                              BN / 64, stage);
             }
             tc_fence_before();
             mbar_arrive(smem_u32(&acce_bar[acc]));
@@ -616,7 +674,7 @@ bool on_device(const void* p, int dev) {
 constexpr int kMaxDevices = 64;
 
 using GemmKernel = void (*)(const CUtensorMap, const CUtensorMap, const GemmArgs);
-constexpr size_t kGemmSmem = kRingBytes + 1024;
+constexpr size_t kGemmSmem = kRingBytes + kEpiWarps * kEpiStage + 1024;
 
 template <int MODE>
 GemmKernel gemm_kernel_of(int bn) {
@@ -675,7 +733,8 @@ long long gemm_tiles(const GemmArgs& g, int bn) {
 //   N 512,  K 2776: M 2048 16.5 / 18.6 / 24.6, 4096 28.8 / 19.9 / 24.7,
 //                   8192 53 / 34.9 / 25.4, 65536 346 / 229 / 169;
 //   N 512,  K 512:  M 2048 8.3 / 10.3 / 12.4, 8192 14.5 / 12.5 / 12.4;
-//   N 2776, K 512:  M 256 8.3 / 10.3 / 12.4, 512 10.4 / 10.3 / 12.4.
+//   N 2776, K 512:  M 256 8.3 / 10.3 / 12.4, 512 10.4 / 10.3 / 12.4
+// (before the stores through shared memory, which the wide tiles gain from).
 // The head sums over 128 columns in one thread: not below that.
 int tile_width(const GemmArgs& g, int max_clusters) {
     int bn = 256;

@@ -442,7 +442,7 @@ cudaError_t propagate_dispatch_any(const TopoLayout& lay, const PropParams* p, i
                                    size_t smem, cudaStream_t s, int* occ) {
     const bool chain = lay.chain != 0;
     const bool table = lay.ptab != 0;
-    if (lay.packed) return propagate_x2_dispatch(lay.per_lane, p, warps, grid, smem, s, occ);
+    if (lay.packed) return propagate_x2_dispatch(lay.per_lane, p, warps, grid, smem, s, lay.split != 0, occ);
     if (lay.paired) {
         switch (lay.per_lane) {
             case 2: return propagate2_b2(p, chain, warps, grid, smem, s, occ);
@@ -477,7 +477,8 @@ int slot_f4(const TopoLayout& lay) {
 size_t prop_smem_units(const TopoLayout& lay, int units) {
     const size_t table = lay.packed ? (size_t)x2_topo_bytes(lay) + (size_t)x2_table_f4(lay) * 16
                                     : (size_t)lay.bytes;
-    return table + (size_t)units * slot_f4(lay) * 16;
+    // the split kernel's pair forces: 3 B words of 32 lanes
+    return table + (size_t)units * slot_f4(lay) * 16 + (lay.split ? 384 * (size_t)lay.per_lane : 0);
 }
 
 size_t prop_smem(const pamd_ctx* c) {
@@ -753,20 +754,30 @@ int set_launch_shape(pamd_ctx* c, const TopoLayout& lay_in, int warps_req, int v
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     const int groups_per_warp = 32 / lay.lanes;  // idle lanes when L does not divide 32
     int warps = warps_req ? warps_req : 4;
+    // One warp per replica group for throughput; two where every warp gets a
+    // scheduler of its own (an SM has four): up to two groups per SM.  us a step,
+    // one / two warps: 22 atoms 608 replicas (one group per SM) 2.32 / 1.61, 1216
+    // (two) 2.33 / 1.65, 75 atoms 304 6.18 / 5.44, 608 6.59 / 5.47, but 912 (three)
+    // 6.99 / 7.78; 200 atoms 304 20.4 / 15.0, 456 21.0 / 25.5.  An explicit block
+    // size keeps the one-warp kernel.
+    const long long groups = (c->R + groups_per_warp - 1) / groups_per_warp;
+    lay.split = lay.packed && !warps_req && lay.per_lane <= kSplitMaxAtoms && groups <= 2 * (long long)c->num_sms;
     // the single-replica kernel of some atoms-per-lane counts takes smaller blocks
     if (lay.packed)
         warps = std::min(warps, kPackedMaxThreads / 32);
     else if (!lay.paired && lay.per_lane >= 1 && lay.per_lane <= 8)
         warps = std::min(warps, prop_max_threads(lay.per_lane) / 32);
+    if (lay.split) warps = 1;  // of replicas, and one beside it
     auto smem = [&](int w) { return (long long)prop_smem_units(lay, w * groups_per_warp); };
     while (smem(warps) > max_smem && warps > 1) --warps;
     if (smem(warps) > max_smem) return fail(PAMD_EUNSUPPORTED, "molecule tables exceed shared memory");
     int occ = 0;
-    cudaError_t e = propagate_dispatch_any(lay, nullptr, warps, 0, (size_t)smem(warps), nullptr, &occ);
+    const int block_warps = lay.split ? 2 : warps;
+    cudaError_t e = propagate_dispatch_any(lay, nullptr, block_warps, 0, (size_t)smem(warps), nullptr, &occ);
     if (e != cudaSuccess || occ < 1)
         return fail(PAMD_ECUDA, std::string("propagate occupancy: ") + cudaGetErrorString(e));
     c->lay = lay;
-    c->warps_per_block = warps;
+    c->warps_per_block = block_warps;
     c->rpb = warps * groups_per_warp * (lay.paired ? 2 : 1);
     const long long batches = (c->R + c->rpb - 1) / c->rpb;
     c->grid_prop = (int)std::min<long long>(batches, (long long)c->num_sms * occ);

@@ -54,6 +54,7 @@ struct TopoLayout {
     float s14_lj, s14_c;       // chain: 1-4 scale factors
     int paired;                // launch: 1 = two replicas per lane group (packed FP32x2)
     int packed;                // launch: 1 = own-atom pairs in packed FP32x2 (chain, B = 3..8)
+    int split;                 // launch: 1 = packed, pairs and the rest of a step in two warps
     int ptab, off_ptab;        // chain: 1 if float4 [L/2][B][B][L] {sigma_ij^2, eps_ij, qq_ij, 0}
                                //   of the half-ring tiles follows (entry ((t-1) B^2 + b B + a) L + g)
     int bytes;                 // total, multiple of 16
@@ -336,9 +337,10 @@ PAMD_DECLARE_PROPAGATE(8)
 // kernels with the pair arithmetic in packed FP32x2 (own atoms in register
 // pairs; linear chains, 3..8 atoms per lane)
 cudaError_t propagate_x2_dispatch(int B, const PropParams* p, int warps, int grid, size_t smem,
-                                  cudaStream_t s, int* blocks_per_sm);
+                                  cudaStream_t s, bool split, int* blocks_per_sm);
 // launch variants of the single-molecule propagate kernel
 constexpr int kVarScalar = 0, kVarPaired = 1, kVarPacked = 2;
+constexpr int kSplitMaxAtoms = 7;        // atoms per lane of the two-warp packed kernel (8: 255 registers do not hold a tile)
 constexpr int kPackedMaxThreads = 128;  // block-size cap of the packed-pair kernel
 // paired kernels (two replicas per lane group), 2..4 atoms per lane
 cudaError_t propagate2_b2(const PropParams* p, bool chain, int warps, int grid, size_t smem,

@@ -255,11 +255,14 @@ __device__ __forceinline__ void partner_x2(const Own<B>& r, const Own<B>& hs, co
 // table has one entry per atom slot), and padding atoms and the missing next
 // block of the last lane sit at distinct, non-collinear points far away (so a
 // term with zero parameters gives exactly zero, never 0 * inf).
-template <int B>
+// meet(), if any, runs between the evaluation of all terms and the sums onto
+// f; without it each term is added as it is evaluated.
+struct NoMeet {};
+
+template <int B, typename Meet>
 __device__ __forceinline__ void bonded_chain_x2(const unsigned char* sm, const TopoLayout& lay,
-                                                const float4* prm, const float4* posA,
-                                                const float4* posB, int L, int g, const Own<B>& r,
-                                                Own<B>& f, float3 (&sf)[3]) {
+                                                const float4* posA, const float4* posB, int L, int g,
+                                                const Own<B>& r, Own<B>& f, float3 (&sf)[3], Meet meet) {
     using C = X2Cfg<B>;
     const int i0 = g * B;
     const bool has_next = (g + 1 < L);
@@ -315,56 +318,96 @@ __device__ __forceinline__ void bonded_chain_x2(const unsigned char* sm, const T
         rc[k] = rsqrtf(cc[k]);
         dd[k] = dot3(bv[k], bv[k + 1]);
     }
+    // bond (d, d+1): 1/2 k (r - r0)^2, force on d is +g b_a
+    auto bond = [&](int a) {
+        const float2 q = cb[i0 + a];
+        const float r = bb[a] * rb[a];
+        return (q.x == 0.0f) ? q.y : q.y * (r - q.x) * rb[a];
+    };
+    auto add_bond = [&](int a, float gk) {
+        const float3 fb = f3scale(gk, bv[a]);
+        F(a, fb);
+        F(a + 1, make_float3(-fb.x, -fb.y, -fb.z));
+    };
+    // angle (d, d+1, d+2) at d+1: u = -b_a, w = b_{a+1}, |u x w| = |c_a|, u.w = -d_a
+    struct Angle {
+        float is, cu, cv;
+    };
+    auto angle = [&](int a) {
+        const float2 q = ca[i0 + a];
+        const float cw = -dd[a];
+        const float dth = atan2_nonneg(cc[a] * rc[a], cw) - q.x;
+        const float is = q.y * dth * rc[a];
+        const float cu = cw * (rb[a] * rb[a]), cvv = cw * (rb[a + 1] * rb[a + 1]);
+        return Angle{is, cu, cvv};
+    };
+    auto add_angle = [&](int a, const Angle& t) {
+        // F_i = is (w - cu u), F_k = is (u - cv w), F_j = -F_i - F_k
+        const float3 fi = f3scale(t.is, f3axpby(1.0f, bv[a + 1], t.cu, bv[a]));
+        const float3 fk = f3scale(-t.is, f3axpby(1.0f, bv[a], t.cv, bv[a + 1]));
+        F(a, fi);
+        F(a + 1, make_float3(-fi.x - fk.x, -fi.y - fk.y, -fi.z - fk.z));
+        F(a + 2, fk);
+    };
+    // dihedral (d..d+3), gradient of phi after Blondel & Karplus (1996): dE/dphi
+    // and the factors of A and B
+    struct Dihedral {
+        float dE, ia, ib, pa, pb;
+    };
+    auto dihedral = [&](int a) {
+        const float4 prm_d = cd[i0 + a];
+        const float kd = prm_d.x, nn = prm_d.y, cph = prm_d.z, sph = prm_d.w;
+        const float3 A = cv[a], Bn = cv[a + 1];
+        const float rlg = rb[a + 1], lg = bb[a + 1] * rlg;
+        const float rA2 = rc[a] * rc[a], rB2 = rc[a + 1] * rc[a + 1];
+        const float rab = rc[a] * rc[a + 1];
+        const float cphi = dot3(A, Bn) * rab;
+        // sin phi = -(F . B) |G| / (|A||B|) with F = -b_a
+        const float sphi = dot3(bv[a], Bn) * lg * rab;
+        const int n = (int)nn;
+        const float c2 = fmaf(cphi + cphi, cphi, -1.0f), s2 = (sphi + sphi) * cphi;
+        const float c3 = fmaf(c2, cphi, -s2 * sphi), s3 = fmaf(s2, cphi, c2 * sphi);
+        const int m = (n > 3) ? n - 3 : n;
+        const float cA = (m == 1) ? cphi : ((m == 2) ? c2 : c3);
+        const float sA = (m == 1) ? sphi : ((m == 2) ? s2 : s3);
+        const float cn = (n > 3) ? fmaf(c3, cA, -s3 * sA) : cA;
+        const float sn = (n > 3) ? fmaf(s3, cA, c3 * sA) : sA;
+        const float dEdphi = -kd * nn * (sn * cph - cn * sph);
+        const float ia = lg * rA2, ib = lg * rB2;
+        // F.G = d_a, H.G = -d_{a+1} (F = -b_a, G = -b_{a+1}, H = b_{a+2})
+        const float pa = dd[a] * rA2 * rlg, pb = -dd[a + 1] * rB2 * rlg;
+        return Dihedral{dEdphi, ia, ib, pa, pb};
+    };
+    auto add_dihedral = [&](int a, const Dihedral& t) {
+        const float3 A = cv[a], Bn = cv[a + 1];
+        F(a, f3scale(t.dE * t.ia, A));
+        F(a + 1, f3axpby(-t.dE * (t.ia + t.pa), A, t.dE * t.pb, Bn));
+        F(a + 2, f3axpby(t.dE * t.pa, A, -t.dE * (t.pb - t.ib), Bn));
+        F(a + 3, f3scale(-t.dE * t.ib, Bn));
+    };
+    if constexpr (std::is_same<Meet, NoMeet>::value) {
 #pragma unroll
-    for (int a = 0; a < B; ++a) {
-        const int d = i0 + a;
-        {  // bond (d, d+1): 1/2 k (r - r0)^2, force on d is +g b_a
-            const float2 q = cb[d];
-            const float r = bb[a] * rb[a];
-            const float gk = (q.x == 0.0f) ? q.y : q.y * (r - q.x) * rb[a];
-            const float3 fb = f3scale(gk, bv[a]);
-            F(a, fb);
-            F(a + 1, make_float3(-fb.x, -fb.y, -fb.z));
+        for (int a = 0; a < B; ++a) {
+            add_bond(a, bond(a));
+            add_angle(a, angle(a));
+            add_dihedral(a, dihedral(a));
         }
-        {  // angle (d, d+1, d+2) at d+1: u = -b_a, w = b_{a+1}, |u x w| = |c_a|, u.w = -d_a
-            const float2 q = ca[d];
-            const float cw = -dd[a];
-            const float dth = atan2_nonneg(cc[a] * rc[a], cw) - q.x;
-            const float is = q.y * dth * rc[a];
-            const float cu = cw * (rb[a] * rb[a]), cvv = cw * (rb[a + 1] * rb[a + 1]);
-            // F_i = is (w - cu u), F_k = is (u - cv w), F_j = -F_i - F_k
-            const float3 fi = f3scale(is, f3axpby(1.0f, bv[a + 1], cu, bv[a]));
-            const float3 fk = f3scale(-is, f3axpby(1.0f, bv[a], cvv, bv[a + 1]));
-            F(a, fi);
-            F(a + 1, make_float3(-fi.x - fk.x, -fi.y - fk.y, -fi.z - fk.z));
-            F(a + 2, fk);
+    } else {
+        float tb[B];
+        Angle ta[B];
+        Dihedral td[B];
+#pragma unroll
+        for (int a = 0; a < B; ++a) {
+            tb[a] = bond(a);
+            ta[a] = angle(a);
+            td[a] = dihedral(a);
         }
-        {  // dihedral (d..d+3), gradient of phi after Blondel & Karplus (1996)
-            const float4 prm_d = cd[d];
-            const float kd = prm_d.x, nn = prm_d.y, cph = prm_d.z, sph = prm_d.w;
-            const float3 A = cv[a], Bn = cv[a + 1];
-            const float rlg = rb[a + 1], lg = bb[a + 1] * rlg;
-            const float rA2 = rc[a] * rc[a], rB2 = rc[a + 1] * rc[a + 1];
-            const float rab = rc[a] * rc[a + 1];
-            const float cphi = dot3(A, Bn) * rab;
-            // sin phi = -(F . B) |G| / (|A||B|) with F = -b_a
-            const float sphi = dot3(bv[a], Bn) * lg * rab;
-            const int n = (int)nn;
-            const float c2 = fmaf(cphi + cphi, cphi, -1.0f), s2 = (sphi + sphi) * cphi;
-            const float c3 = fmaf(c2, cphi, -s2 * sphi), s3 = fmaf(s2, cphi, c2 * sphi);
-            const int m = (n > 3) ? n - 3 : n;
-            const float cA = (m == 1) ? cphi : ((m == 2) ? c2 : c3);
-            const float sA = (m == 1) ? sphi : ((m == 2) ? s2 : s3);
-            const float cn = (n > 3) ? fmaf(c3, cA, -s3 * sA) : cA;
-            const float sn = (n > 3) ? fmaf(s3, cA, c3 * sA) : sA;
-            const float dEdphi = -kd * nn * (sn * cph - cn * sph);
-            const float ia = lg * rA2, ib = lg * rB2;
-            // F.G = d_a, H.G = -d_{a+1} (F = -b_a, G = -b_{a+1}, H = b_{a+2})
-            const float pa = dd[a] * rA2 * rlg, pb = -dd[a + 1] * rB2 * rlg;
-            F(a, f3scale(dEdphi * ia, A));
-            F(a + 1, f3axpby(-dEdphi * (ia + pa), A, dEdphi * pb, Bn));
-            F(a + 2, f3axpby(dEdphi * pa, A, -dEdphi * (pb - ib), Bn));
-            F(a + 3, f3scale(-dEdphi * ib, Bn));
+        meet();
+#pragma unroll
+        for (int a = 0; a < B; ++a) {
+            add_bond(a, tb[a]);
+            add_angle(a, ta[a]);
+            add_dihedral(a, td[a]);
         }
     }
 }
@@ -380,11 +423,11 @@ __device__ __forceinline__ void hand_over(Own<B>& f, int b, float gx, float gy, 
     f.add(b, -rx, -ry, -rz);
 }
 
-// Forces on the lane's own atoms (f).  Positions must be in shared memory
-// (posA/posB of the replica), published by a __syncwarp.  Every lane of the
-// group must call this (the hand-over of partner forces is a warp shuffle).
+// Nonbonded forces on the lane's own atoms (f).  Positions must be in shared
+// memory (posA/posB of the replica), published by a __syncwarp.  Every lane of
+// the group must call this (the hand-over of partner forces is a warp shuffle).
 template <int B>
-__device__ __forceinline__ void forces_x2(const unsigned char* sm, const TopoLayout& lay,
+__device__ __forceinline__ void pairs_x2(const unsigned char* sm, const TopoLayout& lay,
                                           const float4* prm, const float4* dprm,
                                           const unsigned long long* masks, const float4* posA,
                                           const float4* posB, int L, int g, int base,
@@ -503,19 +546,23 @@ __device__ __forceinline__ void forces_x2(const unsigned char* sm, const TopoLay
 #pragma unroll
         for (int b = 0; b < B; ++b) hand_over<B>(f, b, gx[b], gy[b], gz[b], gmask, base + src);
     }
-    // bonded terms; forces on the next block's first atoms go to lane g + 1
+}
+
+// Bonded terms onto f; forces on the next block's first atoms go to lane g + 1.
+template <int B, typename Meet>
+__device__ __forceinline__ void bonded_x2(const unsigned char* sm, const TopoLayout& lay, const float4* posA,
+                                          const float4* posB, int L, int g, int base, unsigned gmask,
+                                          const Own<B>& r, Own<B>& f, Meet meet) {
     float3 sf[3];
-    bonded_chain_x2<B>(sm, lay, prm, posA, posB, L, g, r, f, sf);
-    {
-        int src = g - 1;
-        src = (src < 0) ? src + L : src;  // lane L-1 has no next block and sends zeros
+    bonded_chain_x2<B>(sm, lay, posA, posB, L, g, r, f, sf, meet);
+    int src = g - 1;
+    src = (src < 0) ? src + L : src;  // lane L-1 has no next block and sends zeros
 #pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            const float rx = __shfl_sync(gmask, sf[m].x, base + src);
-            const float ry = __shfl_sync(gmask, sf[m].y, base + src);
-            const float rz = __shfl_sync(gmask, sf[m].z, base + src);
-            if (g > 0) f.add(m, rx, ry, rz);
-        }
+    for (int m = 0; m < 3; ++m) {
+        const float rx = __shfl_sync(gmask, sf[m].x, base + src);
+        const float ry = __shfl_sync(gmask, sf[m].y, base + src);
+        const float rz = __shfl_sync(gmask, sf[m].z, base + src);
+        if (g > 0) f.add(m, rx, ry, rz);
     }
 }
 
@@ -525,6 +572,66 @@ __device__ __forceinline__ void store_pos_x2(float4* posA, float4* posB, int s, 
                                              float z) {
     posA[s] = make_float4(-x, -x, -y, -y);
     *reinterpret_cast<float2*>(&posB[s]) = make_float2(-z, -z);
+}
+
+// Write-back and observables of replica k.
+template <int B>
+__device__ __forceinline__ void write_replica_x2(const PropParams& p, double e_acc, long long k, int N, int Np, int g,
+                                                 int base, unsigned gmask, int L, const Own<B>& r, const Own<B>& v,
+                                                 const Own<B>& f) {
+    // write back and per-replica observables
+    float* so = p.state_out + (size_t)k * 6 * Np;
+    double ek = 0.0, cx = 0.0, cy = 0.0, cz = 0.0;
+#pragma unroll
+    for (int a = 0; a < B; ++a) {
+        const int i = g * B + a;
+        if (i < N) {
+            const float xa = r.gx(a), ya = r.gy(a), za = r.gz(a);
+            const float vxa = v.gx(a), vya = v.gy(a), vza = v.gz(a);
+            if (p.theta > 0) {
+                so[i] = xa;
+                so[Np + i] = ya;
+                so[2 * Np + i] = za;
+                so[3 * Np + i] = vxa;
+                so[4 * Np + i] = vya;
+                so[5 * Np + i] = vza;
+            }
+            if (p.fout) {
+                float* fo = p.fout + (size_t)k * 3 * Np;
+                fo[i] = f.gx(a);
+                fo[Np + i] = f.gy(a);
+                fo[2 * Np + i] = f.gz(a);
+            }
+            const double m = (double)p.masses[i];
+            ek += 0.5 * m * ((double)vxa * vxa + (double)vya * vya + (double)vza * vza);
+            cx += xa;
+            cy += ya;
+            cz += za;
+        }
+    }
+    const double E = group_sum(e_acc, gmask, base, L);
+    ek = group_sum(ek, gmask, base, L);
+    cx = group_sum(cx, gmask, base, L) / N;
+    cy = group_sum(cy, gmask, base, L) / N;
+    cz = group_sum(cz, gmask, base, L) / N;
+    double r2 = 0.0;
+#pragma unroll
+    for (int a = 0; a < B; ++a) {
+        const int i = g * B + a;
+        if (i < N) {
+            const double dx = r.gx(a) - cx, dy = r.gy(a) - cy, dz = r.gz(a) - cz;
+            r2 += dx * dx + dy * dy + dz * dz;
+        }
+    }
+    r2 = group_sum(r2, gmask, base, L);
+    if (g == 0) {
+        p.E[k] = E;
+        p.ke[k] = ek;
+        p.rg[k] = sqrt(r2 / N);
+        if (!isfinite(E) && atomicCAS(&p.status[0], 0, PAMD_ENONFINITE) == 0)
+            p.status[1] = (int)k;
+    }
+    __syncwarp(gmask);
 }
 
 // theta BAOAB steps of replica k by the L lanes of one group.  Velocities
@@ -608,7 +715,8 @@ __device__ __forceinline__ void advance_replica_x2(const PropParams& p, const un
             for (int a = 0; a < B; ++a) store_pos_x2<B>(posA, posB, s0 + a, r.gx(a), r.gy(a), r.gz(a));
             __syncwarp(gmask);
         }
-        forces_x2<B>(sm, lay, prm, dprm, masks, posA, posB, L, g, base, gmask, r, hs, nse, qq, f);
+        pairs_x2<B>(sm, lay, prm, dprm, masks, posA, posB, L, g, base, gmask, r, hs, nse, qq, f);
+        bonded_x2<B>(sm, lay, posA, posB, L, g, base, gmask, r, f, NoMeet{});
     }
     // closing B of the last step
     Own<B> v;
@@ -632,59 +740,7 @@ __device__ __forceinline__ void advance_replica_x2(const PropParams& p, const un
     __syncwarp(gmask);
     const double e_acc = energy_pass<B, true>(sm, lay, prm, posA, masks, L, g);
 
-    // write back and per-replica observables
-    float* so = p.state_out + (size_t)k * 6 * Np;
-    double ek = 0.0, cx = 0.0, cy = 0.0, cz = 0.0;
-#pragma unroll
-    for (int a = 0; a < B; ++a) {
-        const int i = g * B + a;
-        if (i < N) {
-            const float xa = r.gx(a), ya = r.gy(a), za = r.gz(a);
-            const float vxa = v.gx(a), vya = v.gy(a), vza = v.gz(a);
-            if (p.theta > 0) {
-                so[i] = xa;
-                so[Np + i] = ya;
-                so[2 * Np + i] = za;
-                so[3 * Np + i] = vxa;
-                so[4 * Np + i] = vya;
-                so[5 * Np + i] = vza;
-            }
-            if (p.fout) {
-                float* fo = p.fout + (size_t)k * 3 * Np;
-                fo[i] = f.gx(a);
-                fo[Np + i] = f.gy(a);
-                fo[2 * Np + i] = f.gz(a);
-            }
-            const double m = (double)p.masses[i];
-            ek += 0.5 * m * ((double)vxa * vxa + (double)vya * vya + (double)vza * vza);
-            cx += xa;
-            cy += ya;
-            cz += za;
-        }
-    }
-    const double E = group_sum(e_acc, gmask, base, L);
-    ek = group_sum(ek, gmask, base, L);
-    cx = group_sum(cx, gmask, base, L) / N;
-    cy = group_sum(cy, gmask, base, L) / N;
-    cz = group_sum(cz, gmask, base, L) / N;
-    double r2 = 0.0;
-#pragma unroll
-    for (int a = 0; a < B; ++a) {
-        const int i = g * B + a;
-        if (i < N) {
-            const double dx = r.gx(a) - cx, dy = r.gy(a) - cy, dz = r.gz(a) - cz;
-            r2 += dx * dx + dy * dy + dz * dz;
-        }
-    }
-    r2 = group_sum(r2, gmask, base, L);
-    if (g == 0) {
-        p.E[k] = E;
-        p.ke[k] = ek;
-        p.rg[k] = sqrt(r2 / N);
-        if (!isfinite(E) && atomicCAS(&p.status[0], 0, PAMD_ENONFINITE) == 0)
-            p.status[1] = (int)k;
-    }
-    __syncwarp(gmask);
+    write_replica_x2<B>(p, e_acc, k, N, Np, g, base, gmask, L, r, v, f);
 }
 
 template <int B>
@@ -732,10 +788,177 @@ __global__ void __launch_bounds__(X2Cfg<B>::MAX_THREADS, X2Cfg<B>::MIN_BLOCKS)
         advance_replica_x2<B>(p, sm, prm, dprm, aux, masks, posA, posB, vel, k, L, g, base, gmask);
 }
 
+// Small populations: two warps per group of replicas.  One evaluates the
+// nonbonded pairs; the other meanwhile the bonded terms and the next step's
+// noise, then adds the bonded forces to the pairs' in the same order as the
+// one-warp kernel, integrates and publishes the new positions.  The chain of
+// dependent instructions of a step, which is all that counts when a warp has
+// its scheduler to itself, loses the bonded terms, the noise and the
+// integrator's loads.
+// Same instructions on every value: the trajectories are those of
+// propagate_x2_kernel, bit for bit.
+// Bound by the latency of the pair warp's chain: 22 atoms, 256 replicas: 2.33 ->
+// 1.61 us a step; 75 atoms, 152 replicas 6.47 -> 5.18; 200 atoms 20.2 -> 15.0.
+// (Two or four tiles in flight: 1.85 and 5.4, 1.85 and 5.9: the code then
+// outgrows the instruction cache.)
+template <int B>
+__global__ void __launch_bounds__(64) propagate_x2_split_kernel(const PropParams p) {
+    using C = X2Cfg<B>;
+    extern __shared__ float4 smem4[];
+    unsigned char* sm = reinterpret_cast<unsigned char*>(smem4);
+    const TopoLayout& lay = p.lay;
+    const int tb = x2_topo_bytes(lay), N = lay.n_atoms, Np = lay.n_pad;
+    {
+        const float4* src = reinterpret_cast<const float4*>(p.topo);
+        for (int i = threadIdx.x; i < tb / 16; i += blockDim.x) smem4[i] = src[i];
+    }
+    __syncthreads();
+    const float4* prm = reinterpret_cast<const float4*>(sm + lay.off_params);
+    float4* dprm = smem4 + tb / 16;
+    for (int i = threadIdx.x; i < lay.nk; i += blockDim.x) {
+        const float4 c = prm[i];
+        dprm[i] = make_float4(c.x, c.x, c.y, c.y);
+    }
+    const unsigned long long* masks = reinterpret_cast<const unsigned long long*>(sm + lay.off_masks);
+    float4* slots = dprm + x2_table_f4(lay);
+    const int L = lay.lanes, G = 32 / L;
+    const int lane = threadIdx.x & 31, grp = lane / L, g = lane - grp * L, base = grp * L;
+    const unsigned gmask = (L == 32) ? 0xffffffffu : (((1u << L) - 1u) << base);
+    float4* posA = slots + (grp < G ? grp : 0) * x2_slot_f4(lay);  // idle lanes read, never write, group 0's
+    float4* posB = posA + lay.nk;
+    float* fx = reinterpret_cast<float*>(slots + G * x2_slot_f4(lay)) + lane;  // pair forces, 32 lanes apart
+    const int s0 = g * C::BS;
+    const uint32_t step_base = (p.dev_counters ? p.dev_counters[0] : 0u) + p.step0;
+    const float hdt = p.hdt, c1 = p.c1;
+    const long long R = p.live ? (long long)*p.live : p.R;
+    for (long long k0 = (long long)blockIdx.x * G; k0 < R; k0 += (long long)gridDim.x * G) {
+        const long long k = k0 + grp;
+        const bool on = grp < G && k < R;
+        if (threadIdx.x < 32) {  // nonbonded pairs
+            Own<B> r, f, hs, nse, qq;
+            if (on) {
+#pragma unroll
+                for (int a = 0; a < B; ++a) {
+                    const float4 c = prm[s0 + a];
+                    hs.set(a, c.x, 0.f, 0.f);
+                    nse.set(a, -c.y, 0.f, 0.f);
+                    qq.set(a, c.z, 0.f, 0.f);
+                }
+            }
+            for (int s = -1; s < p.theta; ++s) {
+                __syncthreads();  // the positions of step s are in shared memory
+                if (on) {
+#pragma unroll
+                    for (int a = 0; a < B; ++a) {
+                        const float4 pa = posA[s0 + a];
+                        r.set(a, -pa.x, -pa.z, -posB[s0 + a].x);
+                    }
+                    pairs_x2<B>(sm, lay, prm, dprm, masks, posA, posB, L, g, base, gmask, r, hs, nse, qq, f);
+#pragma unroll
+                    for (int a = 0; a < B; ++a) {
+                        fx[96 * a] = f.gx(a);
+                        fx[96 * a + 32] = f.gy(a);
+                        fx[96 * a + 64] = f.gz(a);
+                    }
+                }
+                __syncwarp();
+                asm volatile("bar.sync 1, 64;" ::: "memory");  // the pair forces are in shared memory
+            }
+        } else {  // bonded terms, noise and integration
+            Own<B> r, v, f;
+            float2 cf[B];
+            float3 w[B];
+            const float* st = p.state_in + (size_t)k * 6 * Np;
+#pragma unroll
+            for (int a = 0; a < B; ++a) {
+                const int i = g * B + a;
+                const float3 q = far_point(i);
+                r.set(a, q.x, q.y, q.z);
+                v.set(a, 0.f, 0.f, 0.f);
+            }
+            f.zero();
+            if (on) {
+#pragma unroll
+                for (int a = 0; a < B; ++a) {
+                    const int i = g * B + a;
+                    if (i < N) {
+                        r.set(a, st[i], st[Np + i], st[2 * Np + i]);
+                        v.set(a, st[3 * Np + i], st[4 * Np + i], st[5 * Np + i]);
+                    }
+                    const float4 c = prm[s0 + a];
+                    cf[a] = make_float2(hdt * c.w, p.c2kT * sqrtf(c.w));
+                    posA[s0 + a] = make_float4(-r.gx(a), -r.gx(a), -r.gy(a), -r.gy(a));
+                    posB[s0 + a] = make_float4(-r.gz(a), -r.gz(a), c.z, c.z);
+                }
+            }
+            for (int s = -1; s < p.theta; ++s) {
+                if (s >= 0 && on) {
+#pragma unroll
+                    for (int a = 0; a < B; ++a) {
+                        float x = r.gx(a), y = r.gy(a), z = r.gz(a);
+                        float vx = v.gx(a), vy = v.gy(a), vz = v.gz(a);
+                        const float fx_ = f.gx(a), fy_ = f.gy(a), fz_ = f.gz(a);
+                        if (s > 0) {  // closing B of the previous step
+                            vx = fmaf(cf[a].x, fx_, vx);
+                            vy = fmaf(cf[a].x, fy_, vy);
+                            vz = fmaf(cf[a].x, fz_, vz);
+                        }
+                        vx = fmaf(cf[a].x, fx_, vx);  // B
+                        vy = fmaf(cf[a].x, fy_, vy);
+                        vz = fmaf(cf[a].x, fz_, vz);
+                        x = fmaf(hdt, vx, x);  // A
+                        y = fmaf(hdt, vy, y);
+                        z = fmaf(hdt, vz, z);
+                        vx = fmaf(c1, vx, cf[a].y * w[a].x);  // O
+                        vy = fmaf(c1, vy, cf[a].y * w[a].y);
+                        vz = fmaf(c1, vz, cf[a].y * w[a].z);
+                        x = fmaf(hdt, vx, x);  // A
+                        y = fmaf(hdt, vy, y);
+                        z = fmaf(hdt, vz, z);
+                        r.set(a, x, y, z);
+                        v.set(a, vx, vy, vz);
+                        store_pos_x2<B>(posA, posB, s0 + a, x, y, z);
+                    }
+                }
+                __syncthreads();  // the positions of step s are in shared memory
+                if (on && s + 1 < p.theta) {
+#pragma unroll
+                    for (int a = 0; a < B; ++a)
+                        w[a] = normal3_fast(p.seed, (uint32_t)(g * B + a), (uint32_t)k, step_base + (uint32_t)(s + 1),
+                                            p.purpose_mol);
+                }
+                bonded_x2<B>(sm, lay, posA, posB, L, g, base, gmask, r, f, [&] {
+                    __syncwarp();
+                    asm volatile("bar.sync 1, 64;" ::: "memory");  // the pair forces are in shared memory
+#pragma unroll
+                    for (int a = 0; a < B; ++a) f.set(a, fx[96 * a], fx[96 * a + 32], fx[96 * a + 64]);
+                });
+            }
+            if (on) {
+                if (p.theta > 0) {  // closing B of the last step
+#pragma unroll
+                    for (int a = 0; a < B; ++a)
+                        v.set(a, fmaf(cf[a].x, f.gx(a), v.gx(a)), fmaf(cf[a].x, f.gy(a), v.gy(a)),
+                              fmaf(cf[a].x, f.gz(a), v.gz(a)));
+                }
+                // scalar energy pass on {x, y, z, 0} records
+#pragma unroll
+                for (int a = 0; a < B; ++a) posA[s0 + a] = make_float4(r.gx(a), r.gy(a), r.gz(a), 0.f);
+                __syncwarp(gmask);
+                const double e_acc = energy_pass<B, true>(sm, lay, prm, posA, masks, L, g);
+                write_replica_x2<B>(p, e_acc, k, N, Np, g, base, gmask, L, r, v, f);
+            }
+            __syncwarp();
+        }
+    }
+}
+
 template <int B>
 cudaError_t propagate_x2_launch(const PropParams* p, int warps, int grid, size_t smem,
-                                cudaStream_t s, int* blocks_per_sm) {
+                                cudaStream_t s, bool split, int* blocks_per_sm) {
     auto kern = propagate_x2_kernel<B>;
+    if constexpr (B <= kSplitMaxAtoms)
+        if (split) kern = propagate_x2_split_kernel<B>;
     const cudaError_t e = ensure_dyn_smem((const void*)kern, smem);
     if (e != cudaSuccess) return e;
     if (!p) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kern, warps * 32, smem);

@@ -362,9 +362,8 @@ __global__ void __launch_bounds__(kFeatThreads) mlp_features_kernel(const FeatAr
 // cp.async and their positions in registers.  Bound by shared-memory
 // wavefronts (8 per 32 pairs and configuration in the first pass, 2 per 32
 // elements in the second) and by the barriers between the passes.
-// 65536 configurations of 75 atoms: 471 us (one configuration at a time, 75 of
-// 128 threads in the second pass: 796); shared-memory pipe 72 % busy.
-// 16384 of 128 atoms with the rest of the call: 2062 -> 895 us.
+// 65536 configurations of 75 atoms: 431 us (one configuration at a time, 75 of
+// 128 threads in the second pass: 796); shared-memory pipe three quarters busy.
 // byte offsets: matrix, de/da rows, positions, partial force sums [part][2][N][3]
 struct DuoSmem {
     size_t ga, pos, part, total;
@@ -404,7 +403,7 @@ __device__ __forceinline__ void energies(const ForceArgs& f) {
 }
 
 template <int T>
-__global__ void __launch_bounds__(T, T == 384 ? 3 : 1024 / T) mlp_forces_duo_kernel(const ForceArgs f) {
+__global__ void __launch_bounds__(T, duo_blocks(T)) mlp_forces_duo_kernel(const ForceArgs f) {
     extern __shared__ __align__(16) unsigned char dsm[];
     const int N = f.N, D = (f.M + 1) / 2;
     const DuoSmem L = duo_smem(N, f.Pp);
@@ -445,7 +444,10 @@ __global__ void __launch_bounds__(T, T == 384 ? 3 : 1024 / T) mlp_forces_duo_ker
 using ForceKernel = void (*)(const ForceArgs);
 ForceKernel forces_duo_kernel(int N) {
     const int t = duo_threads(N);
-    return t == 64 ? mlp_forces_duo_kernel<64> : t == 128 ? mlp_forces_duo_kernel<128> : mlp_forces_duo_kernel<384>;
+    return t == 64    ? mlp_forces_duo_kernel<64>
+           : t == 128 ? mlp_forces_duo_kernel<128>
+           : t == 256 ? mlp_forces_duo_kernel<256>
+                      : mlp_forces_duo_kernel<384>;
 }
 
 // The same for molecules past gamma_matrix(N), whose matrix does not fit.
@@ -485,7 +487,7 @@ __host__ __device__ __forceinline__ size_t loss_duo_smem(int N, int Pp) {
 }
 
 template <int T>
-__global__ void __launch_bounds__(T, T == 384 ? 3 : 1024 / T) mlp_loss_duo_kernel(const LossArgs A) {
+__global__ void __launch_bounds__(T, T == 384 ? 3 : duo_blocks(T)) mlp_loss_duo_kernel(const LossArgs A) {
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ double red[32];
     const int N = A.N, D = (A.M + 1) / 2;
@@ -579,7 +581,7 @@ __global__ void __launch_bounds__(T, T == 384 ? 3 : 1024 / T) mlp_loss_duo_kerne
 
 using LossKernel = void (*)(const LossArgs);
 LossKernel loss_duo_kernel(int N) {
-    const int t = duo_threads(N);
+    const int t = duo_threads_wide(N);
     return t == 64 ? mlp_loss_duo_kernel<64> : t == 128 ? mlp_loss_duo_kernel<128> : mlp_loss_duo_kernel<384>;
 }
 
@@ -1206,7 +1208,7 @@ int pamd_mlp_energy_forces(pamd_mlp* m, const float* x_dev, int64_t M, double* E
     f.F = F_dev;
     if (gamma_matrix(m->N)) {
         const int t = duo_threads(m->N);
-        const int grid = F_dev ? grid_for((M + 1) / 2 * t, t, 152 * (t == 384 ? 3 : 1024 / t)) : grid_for(M, t);
+        const int grid = F_dev ? grid_for((M + 1) / 2 * t, t, 152 * duo_blocks(t)) : grid_for(M, t);
         forces_duo_kernel(m->N)<<<grid, t, duo_smem(m->N, m->Pp).total, m->stream>>>(f);
     } else {
         mlp_forces_kernel<<<F_dev ? grid_for(M * kMlpThreads, kMlpThreads, 152 * 16) : grid_for(M, kMlpThreads), kMlpThreads,
@@ -1275,8 +1277,8 @@ int pamd_mlp_loss_grads(pamd_mlp* m, const float* x_dev, const double* E_dev, co
     L.ebar = w.ebar;
     L.loss_part = w.loss_part;
     if (gamma_matrix(m->N)) {
-        const int t = duo_threads(m->N);
-        loss_duo_kernel(m->N)<<<grid_for((M + 1) / 2 * t, t, 152 * (t == 384 ? 3 : 1024 / t)), t,
+        const int t = duo_threads_wide(m->N);
+        loss_duo_kernel(m->N)<<<grid_for((M + 1) / 2 * t, t, 152 * (t == 384 ? 3 : duo_blocks(t))), t,
                                 loss_duo_smem(m->N, m->Pp), s>>>(L);
     } else {
         mlp_loss_kernel<<<grid_for(M * kMlpThreads, kMlpThreads, 152 * 16), kMlpThreads, loss_smem(m), s>>>(L);

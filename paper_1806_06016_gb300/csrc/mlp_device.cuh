@@ -172,15 +172,24 @@ __device__ __forceinline__ Duo3 duo_force(int k, const DuoPos& q, const float2* 
     return f;
 }
 
-// Block size: as many threads as a row split over up to eight keeps busy.
-// Small molecules in 384 threads leave most idle at the barriers (65536
-// configurations of 9 atoms, whole call: 210 us, in 64 threads 131; 16384 of
-// 22: 102 and, in 128, 87).
+// Block size and the blocks per SM it is compiled for: as many threads as a row
+// split over up to eight keeps busy.  Small molecules in 384 threads leave
+// most idle at the barriers (65536 configurations of 9 atoms, whole call: 210
+// us, in 64 threads 131; 16384 of 22: 102 and, in 128, 87).  Three blocks' shared
+// memory fits an SM up to 82 atoms; 256 threads with 85 registers then beat 384
+// with 56 (75 atoms, 65536 configurations: forces 475 -> 432 us), and past it
+// 384 at two blocks do (16384 of 97 atoms, whole call: 456 -> 391 us).
 constexpr int kDuoPartsMax = 8;
 constexpr int kDuoElems = 2;  // coordinates per thread: 6 N <= 2 threads
 
-__host__ __device__ __forceinline__ int duo_threads(int N) { return N <= 21 ? 64 : N <= 42 ? 128 : 384; }
-static_assert(6 * 21 <= kDuoElems * 64 && 6 * 42 <= kDuoElems * 128 && 6 * kGammaMatrixMax <= kDuoElems * 384, "");
+__host__ __device__ __forceinline__ int duo_threads(int N) { return N <= 21 ? 64 : N <= 42 ? 128 : N <= 82 ? 256 : 384; }
+// The loss and MD step kernels run 384 from 43 atoms on: their work beside the
+// pairs uses the warps (loss of 2048 samples of 75 atoms: 44 us in 384 threads,
+// 49 in 256; a step of 16384 replicas of 75, H = 64: 286 and 294).
+__host__ __device__ __forceinline__ int duo_threads_wide(int N) { return N <= 42 ? duo_threads(N) : 384; }
+__host__ __device__ constexpr int duo_blocks(int threads) { return threads == 384 ? 2 : threads == 256 ? 3 : 1024 / threads; }
+static_assert(6 * 21 <= kDuoElems * 64 && 6 * 42 <= kDuoElems * 128 && 6 * 82 <= kDuoElems * 256 &&
+                  6 * kGammaMatrixMax <= kDuoElems * 384, "");
 __host__ __device__ __forceinline__ int duo_parts(int N) {
     return duo_threads(N) / N < kDuoPartsMax ? duo_threads(N) / N : kDuoPartsMax;
 }

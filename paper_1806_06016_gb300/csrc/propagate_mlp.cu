@@ -306,7 +306,7 @@ StepKernel step_kernel(int N, int* threads) {
         *threads = kStepThreads;
         return mlp_step_large_kernel;
     }
-    *threads = duo_threads(N);
+    *threads = duo_threads_wide(N);
     return *threads == 64 ? mlp_step_duo_kernel<64> : *threads == 128 ? mlp_step_duo_kernel<128> : mlp_step_duo_kernel<384>;
 }
 

@@ -48,7 +48,7 @@ def _model(S, n, x):
     return model, q
 
 
-@pytest.mark.parametrize("n", [4, 31, 48, 49, 97, 128, 129])
+@pytest.mark.parametrize("n", [4, 21, 22, 31, 42, 43, 48, 49, 82, 83, 97, 128, 129])
 def test_forces_over_the_row_splits(env, n):
     torch, S = env
     x = pi.perturbed_positions(pi.make_chain(n, 4), 7, 0.02, 2).astype(np.float32)

@@ -1,5 +1,6 @@
 """Resampling at the edges of its one-launch form (chunks of 512, 1024 and 2048
-replicas in up to eight CTAs, 16384 replicas at most) and just above it.
+replicas in up to eight CTAs, 16384 replicas at most), just above it, and over
+several blocks of the separate launches.
 
 Counts, families and energies are integer work or copies: exact.  ln Q is an
 FP64 sum in another order than the oracle's: 1e-12 relative.
@@ -26,7 +27,7 @@ def lib():
 @pytest.mark.parametrize("rule", [0, 1])
 @pytest.mark.parametrize("R,spread", [(1, 10.0), (31, 30.0), (511, 30.0), (512, 1e5), (513, 30.0), (2049, 0.0),
                                       (4096, 30.0), (4097, 2000.0), (8192, 30.0), (8193, 30.0), (16383, 60.0),
-                                      (16384, 1e4), (16385, 30.0)])
+                                      (16384, 1e4), (16385, 30.0), (49153, 1e4), (262144, 0.0), (262145, 60.0)])
 def test_two_resamplings(lib, orc, R, spread, rule):
     from oracle import adaptive as oa
     n, seed = 3, 17 + R

@@ -107,6 +107,9 @@ NCU_TRAFFIC = {
     # after the t = 1 tile's masks became compile-time constants: 15.18 MB
     # read, 26 KB written
     "3be35c0f8ab35a11": 15205120,
+    # the same kernel after the two-warp form of small populations joined the
+    # header (theta = 1000): 15.36 MB read, 27 KB written
+    "e0d6ff45d4fd3965": 15383808,
 }
 
 
@@ -1186,7 +1189,7 @@ def run_surrogate(args, w):
     out["force_evaluation_ms"] = {"total": per_eval, "gemms": gemm_ms, "step_kernel": step_ms}
     out["roofline"] = {"bound": "hbm", "achieved": step_bytes / (step_ms / 1e3) / 1e9, "peak": hbm,
                        "unit": "GB/s", "frac": step_bytes / (step_ms / 1e3) / 1e9 / hbm if hbm else None,
-                       "traffic": None, "kernel": "mlp_step_kernel (largest time share)",
+                       "traffic": None, "kernel": "mlp_step_duo_kernel (largest time share)",
                        "bytes_per_launch": step_bytes,
                        "launch_ms_basis": "event-timed force evaluation minus the event-timed GEMMs",
                        "peak_basis": "measured copy bandwidth (MEASURED_PEAKS.json)"}

@@ -140,7 +140,8 @@ typedef struct pamd_options {
     int32_t precision;          /* PAMD_PREC_MIXED or PAMD_PREC_FP64 */
     int32_t lanes_per_replica;  /* 0 = choose; else 1..32 lanes, with at most 8 atoms
                                    per lane (ceil(n_atoms / lanes) <= 8) */
-    int32_t warps_per_block;    /* 0 = choose (4); else 1..8, lowered to the kernel's
+    int32_t warps_per_block;    /* 0 = choose (4, or 2 that share each step of a small
+                                   population of chains); else 1..8, lowered to the kernel's
                                    block-size cap (4 warps for the packed-pair kernel
                                    and for 5 atoms per lane) and to shared memory */
     int32_t mol_id;             /* molecule index mixed into the random counters */

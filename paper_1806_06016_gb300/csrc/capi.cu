@@ -757,8 +757,8 @@ int set_launch_shape(pamd_ctx* c, const TopoLayout& lay_in, int warps_req, int v
     // One warp per replica group for throughput; two where every warp gets a
     // scheduler of its own (an SM has four): up to two groups per SM.  us a step,
     // one / two warps: 22 atoms 608 replicas (one group per SM) 2.32 / 1.61, 1216
-    // (two) 2.33 / 1.65, 75 atoms 304 6.18 / 5.44, 608 6.59 / 5.47, but 912 (three)
-    // 6.99 / 7.78; 200 atoms 304 20.4 / 15.0, 456 21.0 / 25.5.  An explicit block
+    // (two) 2.42 / 1.67, 75 atoms 304 7.2 / 5.5, 608 7.2 / 5.6, but 912 (three) 7.0 /
+    // 7.8; 200 atoms 304 21.2 / 15.2, 456 21.0 / 25.5.  An explicit block
     // size keeps the one-warp kernel.
     const long long groups = (c->R + groups_per_warp - 1) / groups_per_warp;
     lay.split = lay.packed && !warps_req && lay.per_lane <= kSplitMaxAtoms && groups <= 2 * (long long)c->num_sms;

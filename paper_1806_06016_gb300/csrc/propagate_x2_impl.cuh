@@ -30,6 +30,9 @@
 //   evaluated there with their scale factors instead of being masked out and
 //   recomputed with the bonded terms.
 //
+// * Populations too small to fill the chip run each step in two warps
+//   (propagate_x2_split_kernel).
+//
 // Linear-chain layouts only (B >= 3); other topologies use propagate_impl.cuh.
 #pragma once
 
@@ -797,10 +800,10 @@ __global__ void __launch_bounds__(X2Cfg<B>::MAX_THREADS, X2Cfg<B>::MIN_BLOCKS)
 // integrator's loads.
 // Same instructions on every value: the trajectories are those of
 // propagate_x2_kernel, bit for bit.
-// Bound by the latency of the pair warp's chain: 22 atoms, 256 replicas: 2.33 ->
-// 1.61 us a step; 75 atoms, 152 replicas 6.47 -> 5.18; 200 atoms 20.2 -> 15.0.
-// (Two or four tiles in flight: 1.85 and 5.4, 1.85 and 5.9: the code then
-// outgrows the instruction cache.)
+// Bound by the latency of the pair warp's chain.  us a step, before and now: 256
+// replicas of 22 atoms 2.33, 1.63; 152 of 75 atoms 6.5, 5.5; 152 of 200 atoms
+// 20.2, 15.1.  (Two or four tiles in flight at once: 1.85 and up to 2.2 times the
+// time, as the code then outgrows the instruction cache.)
 template <int B>
 __global__ void __launch_bounds__(64) propagate_x2_split_kernel(const PropParams p) {
     using C = X2Cfg<B>;

@@ -191,6 +191,8 @@ struct GraphKey {
     int K = -1, theta = -1, resample = -1;
     double dt = 0;
     std::vector<double> T;
+    // the captured kernels hold each population's seed by value
+    std::vector<unsigned long long> seeds;
     const double* rec = nullptr;  // energy recording target (pamd_record_energies)
     int rec_rows = 0;
     // force model: which one, the generation of its workspace, its energy scale
@@ -199,7 +201,7 @@ struct GraphKey {
     double mu_E = 0, sigma_E = 0;
     bool operator==(const GraphKey& o) const {
         return K == o.K && theta == o.theta && resample == o.resample && dt == o.dt && T == o.T &&
-               rec == o.rec && rec_rows == o.rec_rows && model == o.model && model_gen == o.model_gen &&
+               seeds == o.seeds && rec == o.rec && rec_rows == o.rec_rows && model == o.model && model_gen == o.model_gen &&
                mu_E == o.mu_E && sigma_E == o.sigma_E;
     }
 };

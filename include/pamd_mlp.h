@@ -120,7 +120,9 @@ int pamd_mlp_get_params(pamd_mlp* mlp, pamd_mlp_params* p);
  * Set the normalisation from data: mu_p and sd_p as the mean and standard
  * deviation (population, n in the denominator) of g_p over the n
  * configurations x_dev [n][N][3], mu_E and sigma_E those of E_dev [n];
- * a zero standard deviation becomes 1.  Computed in FP64 on the GPU.
+ * a zero standard deviation becomes 1.  mu_E and sigma_E in FP64; mu_p and sd_p
+ * are the FP32 roundings of sums that hold g_p to 2^-44 of its value, or, where
+ * the spread of a feature is below 2^-16 of its mean, of FP64 sums.
  * Synchronous.  Errors: PAMD_EINVAL (n < 2, null pointer), PAMD_ECUDA.
  */
 int pamd_mlp_fit_normalization(pamd_mlp* mlp, const float* x_dev, const double* E_dev, int64_t n);

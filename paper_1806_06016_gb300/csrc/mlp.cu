@@ -137,28 +137,38 @@ __global__ void mlp_adam_kernel(float* p, const float* __restrict__ g, float* m,
 // Mean and sum of squared deviations of every feature g_p = 1 / r over n
 // configurations (and of the energies), merged from slices of the data.
 //
-// The result is that of 64-bit arithmetic, but GB300's FP64 units do a 64th
-// of the FP32 rate, and a reciprocal square root per sample and pair is all
-// the work there is.  So a sample's g is formed in pairs of FP32 numbers
-// (TwoSum: Knuth 1969; exact products by fma): coordinate differences are
-// exact, r^2 carries its rounding errors, and one Newton step on the hardware
-// reciprocal square root leaves g = y0 + corr with a relative error of about
-// 2^-44.  Deviations from the slice's first sample (exactly zero for an equal
-// one, so that a constant feature has no spurious deviation) are summed, with
-// their squares, in compensated FP32; slices become (mean,
-// M2) in FP64 and are merged by Chan, Golub & LeVeque's (1979) formula.
-// A distance outside [1e-10, 1e10] nm (coincident atoms, non-finite input)
-// marks its pair with a NaN, and the merge kernel then does that pair in plain
-// FP64.
+// GB300's FP64 units do a 64th of the FP32 rate, and a reciprocal square root
+// per sample and pair is all the work there is.  So a sample's g is formed in
+// pairs of FP32 numbers (TwoSum: Knuth 1969; exact products by fma):
+// coordinate differences are exact, r^2 carries its rounding errors, and one
+// Newton step on the hardware reciprocal square root leaves g = y0 + corr
+// within 2^-44 of its value.  Deviations from the slice's first sample
+// (exactly zero for an equal one, so that a constant feature has no spurious
+// deviation) are pairs as well; they and their squares are added in
+// compensated FP32 over kStatHold samples or a tile, then in FP64.  Slices become
+// (mean, M2) in FP64 and are merged by Chan, Golub & LeVeque's (1979) formula.
+// A spread below 2^-16 of the mean, of which 2^-44 of g would be 2^-28 or more,
+// and a distance outside [1e-10, 1e10] nm (coincident atoms, non-finite input;
+// its pair is marked with a NaN) are left to the merge kernel, which does that
+// pair in plain FP64.  mu and sd are then the FP32 roundings of values within
+// 2^-40 and 2^-28 of the 64-bit ones (a slice whose first sample lies far from
+// the rest loses log2 of its length of these bits).
 //
 // One thread per pair, the positions of a tile of configurations in shared
 // memory as float4 (consecutive pairs read consecutive atoms: no bank
 // conflicts), the data cut into as many slices as fill the chip.
-// 65536 configurations of 75 atoms: 611 + 29 us, bound by the FP32 issue rate
-// (about 85 instructions per sample and pair); one thread per pair looping
-// twice over all configurations in FP64 (22 blocks) took 151.0 ms.
+// 65536 configurations of 75 atoms: 661 + 30 us, bound by the FP32 issue rate
+// (about 90 instructions per sample and pair).  Deviations rounded to FP32
+// took 611 us and lost up to half the last bit of sd; one thread per pair
+// looping twice over all configurations in FP64 (22 blocks) took 151.0 ms.
+// Against 64-bit torch, 27 sets of 9..75 atoms x 100..65536 samples: mu and sd
+// are as far from it as that FP64 loop's, to five digits.
 constexpr int kStatThreads = 256;
 constexpr int kStatTileBytes = 24 * 1024;
+constexpr int kStatHold = 64;  // samples added in FP32 pairs before they join the FP64 sums
+// block columns (the last one for the energies), and slices that give every SM six blocks
+int stat_columns(int P) { return (P + kStatThreads - 1) / kStatThreads + 1; }
+int stat_slices(int P, int sms) { return (6 * sms + stat_columns(P) - 1) / stat_columns(P); }
 
 // a + b = s + e exactly
 __device__ __forceinline__ float two_sum(float a, float b, float& e) {
@@ -212,8 +222,32 @@ __global__ void __launch_bounds__(kStatThreads) mlp_moments_kernel(const float* 
     }
     const int p = blockIdx.x * kStatThreads + threadIdx.x;
     const ushort2 ij = pairs[p < P ? p : 0];
-    float g0 = 0.0f, c0 = 0.0f, s = 0.0f, sl = 0.0f, q = 0.0f, ql = 0.0f;
-    bool first = true, bad = false;
+    float g0 = 0.0f, c0 = 0.0f;
+    double S = 0.0, Q = 0.0;  // of the deviations from g0 + c0
+    float s = 0.0f, sl = 0.0f, q = 0.0f, ql = 0.0f;
+    int held = 0;  // samples in the FP32 sums
+    float h_min = 1.0f, h_max = 1.0f;  // squared distances (a NaN reaches the sums)
+    // g = y + corr of sample c of the tile
+    auto feature = [&](int c, float& y, float& corr) {
+        const float4 a = sx[c * N + ij.x], b = sx[c * N + ij.y];
+        float ex, ey, ez, l1, l2;
+        const float dx = two_sum(a.x, -b.x, ex), dy = two_sum(a.y, -b.y, ey), dz = two_sum(a.z, -b.z, ez);
+        const float px = __fmul_rn(dx, dx), py = __fmul_rn(dy, dy), pz = __fmul_rn(dz, dz);
+        const float h = two_sum(two_sum(px, py, l1), pz, l2);
+        // the squares' errors and the cross terms 2 d e
+        const float qe = __fadd_rn(__fmaf_rn(dx, dx, -px), __fadd_rn(__fmaf_rn(dy, dy, -py), __fmaf_rn(dz, dz, -pz)));
+        const float qc = __fmaf_rn(dx, ex, __fmaf_rn(dy, ey, __fmul_rn(dz, ez)));
+        const float lo = __fadd_rn(__fadd_rn(l1, l2), __fmaf_rn(2.0f, qc, qe));
+        h_min = fminf(h_min, h);
+        h_max = fmaxf(h_max, h);
+        y = rsqrtf(h);
+        // e = 1 - r^2 y^2
+        const float u = __fmul_rn(h, y), ue = __fmaf_rn(h, y, -u);
+        float e = __fmaf_rn(-u, y, 1.0f);
+        e = __fmaf_rn(-ue, y, e);
+        e = __fmaf_rn(-__fmul_rn(lo, y), y, e);
+        corr = __fmul_rn(y, __fmaf_rn(__fmul_rn(0.375f, e), e, __fmul_rn(0.5f, e)));
+    };
     for (long long t0 = m0; t0 < m1; t0 += tile) {
         const int nt = (int)(m1 - t0 < tile ? m1 - t0 : tile);
         __syncthreads();
@@ -221,39 +255,34 @@ __global__ void __launch_bounds__(kStatThreads) mlp_moments_kernel(const float* 
         for (int a = threadIdx.x; a < nt * N; a += kStatThreads)
             sx[a] = make_float4(src[3 * a], src[3 * a + 1], src[3 * a + 2], 0.0f);
         __syncthreads();
+        if (t0 == m0) feature(0, g0, c0);
 #pragma unroll 2
         for (int c = 0; c < nt; ++c) {
-            const float4 a = sx[c * N + ij.x], b = sx[c * N + ij.y];
-            float ex, ey, ez, qx, qy, qz, l1, l2;
-            const float dx = two_sum(a.x, -b.x, ex), dy = two_sum(a.y, -b.y, ey), dz = two_sum(a.z, -b.z, ez);
-            const float px = square_err(dx, ex, qx), py = square_err(dy, ey, qy), pz = square_err(dz, ez, qz);
-            const float h = two_sum(two_sum(px, py, l1), pz, l2);
-            const float lo = __fadd_rn(__fadd_rn(l1, l2), __fadd_rn(qx, __fadd_rn(qy, qz)));
-            bad = bad || !(h > 1e-20f && h < 1e20f);
-            const float y = rsqrtf(h);
-            // e = 1 - r^2 y^2
-            const float u = __fmul_rn(h, y), ue = __fmaf_rn(h, y, -u);
-            float e = __fmaf_rn(-u, y, 1.0f);
-            e = __fmaf_rn(-ue, y, e);
-            e = __fmaf_rn(-__fmul_rn(lo, y), y, e);
-            const float corr = __fmul_rn(y, __fmaf_rn(__fmul_rn(0.375f, e), e, __fmul_rn(0.5f, e)));
-            if (first) {
-                g0 = y;
-                c0 = corr;
-                first = false;
-            }
-            const float d = __fadd_rn(__fsub_rn(y, g0), __fsub_rn(corr, c0));
-            float err;
+            float y, corr, ey0, dl, err;
+            feature(c, y, corr);
+            const float dy0 = two_sum(y, -g0, ey0);
+            const float dc = __fadd_rn(__fsub_rn(corr, c0), ey0);
+            const float d = __fadd_rn(dy0, dc);
+            dl = __fsub_rn(dc, __fsub_rn(d, dy0));  // dy0 is 0 or at least an ulp of g, dc a few: lost are 2^-22 of these
             s = two_sum(s, d, err);
-            sl = __fadd_rn(sl, err);
-            const float d2 = __fmul_rn(d, d);
+            sl = __fadd_rn(sl, __fadd_rn(err, dl));
+            float e2;
+            const float d2 = square_err(d, dl, e2);
             q = two_sum(q, d2, err);
-            ql = __fadd_rn(ql, __fadd_rn(err, __fmaf_rn(d, d, -d2)));
+            ql = __fadd_rn(ql, __fadd_rn(err, e2));
+        }
+        held += nt;
+        if (held >= kStatHold || t0 + tile >= m1) {
+            S += (double)s + (double)sl;
+            Q += (double)q + (double)ql;
+            s = sl = q = ql = 0.0f;
+            held = 0;
         }
     }
     if (p < P) {
-        const double cnt = (double)(m1 - m0), S = (double)s + (double)sl, Q = (double)q + (double)ql;
+        const double cnt = (double)(m1 - m0);
         const double m2 = Q - S * (S / cnt);
+        const bool bad = !(h_min > 1e-20f && h_max < 1e20f);
         out[p] = bad ? make_double2(NAN, NAN) : make_double2(((double)g0 + (double)c0) + S / cnt, m2 > 0.0 ? m2 : 0.0);
     }
 }
@@ -287,7 +316,8 @@ __global__ void __launch_bounds__(128) mlp_moments_merge_kernel(const float* __r
         }
         return;
     }
-    if (isnan(mean)) {  // a distance out of the fast path's range: this pair in FP64
+    // a distance out of the fast path's range, or a spread too small for its bits: this pair in FP64
+    if (isnan(mean) || (m2 > 0.0 && m2 < 0x1p-32 * (double)n * mean * mean)) {
         const ushort2 ij = pairs[p];
         auto g_of = [&](long long m) {
             const float* c = x + m * 3 * N;
@@ -979,10 +1009,18 @@ int pamd_mlp_create(pamd_mlp** out, int32_t n_atoms, int32_t hidden, uint64_t se
     m->ow3 = m->ob2 + H;
     m->ob3 = m->ow3 + H;
     m->n_params = m->ob3 + 4;
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        delete m;
+        return mfail(PAMD_ECUDA, "pamd_mlp_create: no CUDA device");
+    }
+    m->max_slices = stat_slices(m->P, sms);
     const size_t pbytes = align256(4 * m->n_params);
     const size_t sizes[] = {pbytes, pbytes, pbytes, pbytes, align256(4 * Pp), align256(4 * Pp),
                             align256(4 * Pp), align256(2 * H * Pp), align256(2 * H * H), align256(4 * Pp),
-                            align256(sizeof(int)), align256(8 * 4)};
+                            align256(sizeof(int)), align256(8 * 4),
+                            align256(sizeof(double2) * (size_t)m->max_slices * (m->P + 1))};
     size_t total = 0;
     for (size_t s : sizes) total += s;
     if (stream) {
@@ -1018,6 +1056,7 @@ int pamd_mlp_create(pamd_mlp** out, int32_t n_atoms, int32_t hidden, uint64_t se
     m->pairs = reinterpret_cast<ushort2*>(take());
     m->status = reinterpret_cast<int*>(take());
     m->scratch = reinterpret_cast<double*>(take());
+    m->moments = reinterpret_cast<double2*>(take());
     // pair table, identity normalisation, zero moments
     std::vector<ushort2> pr(Pp, make_ushort2(0, 0));
     for (int i = 0, q = 0; i < n_atoms; ++i)
@@ -1143,28 +1182,12 @@ int pamd_mlp_fit_normalization(pamd_mlp* m, const float* x_dev, const double* E_
     int rc = check_model(m);
     if (rc) return rc;
     if (!x_dev || !E_dev || n < 2) return mfail(PAMD_EINVAL, "pamd_mlp_fit_normalization: null pointer or n < 2");
-    int dev = 0, sms = 0;
-    MLP_CU(m, cudaGetDevice(&dev));
-    MLP_CU(m, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    // slices: six blocks per SM over all block columns, at least a tile each
-    const int cols = (m->P + kStatThreads - 1) / kStatThreads + 1;
+    const int cols = stat_columns(m->P);
     const int tile = kStatTileBytes / (16 * m->N) > 0 ? kStatTileBytes / (16 * m->N) : 1;
-    const long long max_slices = (6LL * sms + cols - 1) / cols;
-    long long slices = (n + tile - 1) / tile;
-    if (slices > max_slices) slices = max_slices;
+    long long slices = (n + tile - 1) / tile;  // a tile each at least
+    if (slices > m->max_slices) slices = m->max_slices;
     const long long per = (n + slices - 1) / slices;
     slices = (n + per - 1) / per;  // no empty slice
-    if (m->moments_cap < max_slices) {  // kept with the model
-        if (m->moments) cudaFree(m->moments);
-        m->moments = nullptr;
-        m->moments_cap = 0;
-        if (cudaMalloc(&m->moments, sizeof(double2) * (size_t)max_slices * (m->P + 1)) != cudaSuccess) {
-            cudaGetLastError();
-            m->moments = nullptr;
-            return mfail(PAMD_ENOMEM, "pamd_mlp_fit_normalization: workspace");
-        }
-        m->moments_cap = max_slices;
-    }
     mlp_moments_kernel<<<dim3(cols, (unsigned)slices), kStatThreads, sizeof(float4) * (size_t)tile * m->N, m->stream>>>(
         x_dev, E_dev, n, per, m->N, m->P, tile, m->pairs, m->moments);
     if ((rc = launch_check(m, "feature statistics"))) return rc;
@@ -1470,7 +1493,6 @@ void pamd_mlp_destroy(pamd_mlp* m) {
     if (m->loop_ctr) cudaFree(m->loop_ctr);
     if (m->body_stream) cudaStreamDestroy(m->body_stream);
     if (m->w.base) cudaFree(m->w.base);
-    if (m->moments) cudaFree(m->moments);
     if (m->base) cudaFree(m->base);
     if (m->own_stream && m->stream) cudaStreamDestroy(m->stream);
     delete m;

@@ -146,10 +146,10 @@ struct pamd_mlp {
     ushort2* pairs = nullptr;       // [Pp]
     int* status = nullptr;
     double* scratch = nullptr;      // [4] loss and statistics
+    double2* moments = nullptr;  // [max_slices][P + 1] (mean, M2) of pamd_mlp_fit_normalization
+    int max_slices = 0;
     void* base = nullptr;           // allocation holding the members above
     pamd::MlpWork w;
-    double2* moments = nullptr;     // slices' (mean, M2) of pamd_mlp_fit_normalization, kept once allocated
-    long long moments_cap = 0;      // slices it holds
     long long work_gen = 0;         // incremented whenever the workspace is reallocated
     int* loop_ctr = nullptr;        // step index of a captured MD loop (device int)
     cudaStream_t body_stream = nullptr;  // captures the body of that loop

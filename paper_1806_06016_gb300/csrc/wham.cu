@@ -710,14 +710,22 @@ extern "C" int pamd_wham(const pamd_wham_args* a, pamd_wham_result* r) {
     const size_t o_st = off; off += align256(sizeof(SweepState));
     const size_t o_edges = off; off += align256(sizeof(long long) * (size_t)std::min(nb, kEdgeBins));
     // the table is laid out where it may be used; the energy range, known
-    // below, decides whether it is
+    // below, decides whether it is.  One allocation, as each costs tens of
+    // microseconds; a device without room for the table still sweeps with every
+    // exponential evaluated.
     const size_t cells = (size_t)nT * nb;
-    const bool table_fits = cells * kCellBytes <= kTableBytes;
+    bool table_fits = cells * kCellBytes <= kTableBytes;
     const size_t o_tab = off;
     if (table_fits)
         off += 2 * align256(sizeof(double) * cells) + 2 * align256(sizeof(int) * cells) + 2 * align256(sizeof(double) * nT) +
                2 * align256(sizeof(int) * nT) + align256(sizeof(double) * nb) + align256(sizeof(int) * nb);
     e = cudaMalloc(&wk.base, off);
+    if (e != cudaSuccess && table_fits) {
+        cudaGetLastError();
+        table_fits = false;
+        off = o_tab;
+        e = cudaMalloc(&wk.base, off);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         wk.base = nullptr;

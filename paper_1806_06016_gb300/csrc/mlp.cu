@@ -8,6 +8,7 @@
 // Everything between the products (features, the pair Jacobian and its
 // transpose, second-derivative terms, column sums) is FP32 here; energies and
 // loss sums are FP64.
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -903,7 +904,10 @@ int mlp_ensure_work(pamd_mlp* m, long long M, bool train) {
         cudaStreamSynchronize(m->stream);
         cudaFree(w.base);
     }
-    m->work_gen += 1;  // graphs captured over the old workspace are stale
+    // graphs captured over another workspace are stale: also one of a model
+    // that was destroyed and whose address this one took
+    static std::atomic<long long> generations{0};
+    m->work_gen = ++generations;
     MlpWork nw;
     nw.cap = cap;
     nw.train = tr;

@@ -150,7 +150,7 @@ struct pamd_mlp {
     int max_slices = 0;
     void* base = nullptr;           // allocation holding the members above
     pamd::MlpWork w;
-    long long work_gen = 0;         // incremented whenever the workspace is reallocated
+    long long work_gen = 0;         // of the workspace, unique in the process (0: none)
     int* loop_ctr = nullptr;        // step index of a captured MD loop (device int)
     cudaStream_t body_stream = nullptr;  // captures the body of that loop
 };

@@ -88,3 +88,32 @@ def test_batch_seeds(lib):
         _equal(_run(lib, ctx), fresh([(None, 2), (1, 3)]))
     finally:
         lib.pamd_destroy(ctx)
+
+
+def test_force_model_at_a_freed_models_address(lib):
+    """A model made after another was destroyed often takes its host address;
+    the anneal captured with the first must not stand for the second."""
+    import torch
+    from paper_1806_06016_gb300 import surrogate
+    n, R = 12, 70
+    top = pi.make_chain(n, 2)
+
+    def anneal(p, model):
+        p.reset(TEMPS[0], 5)
+        surrogate.attach(p.ctx, model)
+        got = _run(lib, p.ctx)
+        surrogate.attach(p.ctx, None)
+        return got
+
+    with lib.Population(top, R, TEMPS[0], 5, lib.torch_options()) as p, \
+            lib.Population(top, R, TEMPS[0], 5, lib.torch_options()) as q:
+        first = surrogate.MLP(n, 64, seed=1)
+        a = anneal(p, first)
+        first.close()
+        hold = torch.empty(32 << 20, dtype=torch.uint8, device="cuda")  # the device memory it gave back is taken
+        second = surrogate.MLP(n, 64, seed=2)
+        b = anneal(p, second)
+        _equal(b, anneal(q, second))
+        assert not np.array_equal(a[1][0][0], b[1][0][0])
+        second.close()
+        del hold

@@ -909,7 +909,10 @@ int anneal_batch(pamd_ctx* c, int32_t K, const double* T, int32_t theta, double 
     key.resample = resample ? 1 : 0;
     key.dt = dt_ps;
     key.T.assign(T, T + K + 1);
-    for (const pamd_ctx* sub : c->subs) key.seeds.push_back(sub->seed);
+    for (const pamd_ctx* sub : c->subs) {
+        key.seeds.push_back(sub->seed);
+        key.obs.push_back(sub->b.obs);
+    }
     if (c->mlp) {
         // A force model issues five launches per MD step: queue the anneal
         // directly instead of capturing a graph of that size.
@@ -1533,6 +1536,7 @@ int pamd_anneal(pamd_ctx* c, int32_t K, const double* T, int32_t theta, double d
     key.dt = dt_ps;
     key.T.assign(T, T + K + 1);
     key.seeds.assign(1, c->seed);
+    key.obs.assign(1, c->b.obs);
     key.rec = c->rec_E;
     key.rec_rows = c->rec_rows;
     // the captured graph starts from the main buffers

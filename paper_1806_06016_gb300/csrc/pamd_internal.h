@@ -191,8 +191,10 @@ struct GraphKey {
     int K = -1, theta = -1, resample = -1;
     double dt = 0;
     std::vector<double> T;
-    // the captured kernels hold each population's seed by value
+    // the captured kernels hold each population's seed by value and write its
+    // observables buffer, which a longer anneal moves
     std::vector<unsigned long long> seeds;
+    std::vector<const void*> obs;
     const double* rec = nullptr;  // energy recording target (pamd_record_energies)
     int rec_rows = 0;
     // force model: which one, the generation of its workspace, its energy scale
@@ -201,8 +203,8 @@ struct GraphKey {
     double mu_E = 0, sigma_E = 0;
     bool operator==(const GraphKey& o) const {
         return K == o.K && theta == o.theta && resample == o.resample && dt == o.dt && T == o.T &&
-               seeds == o.seeds && rec == o.rec && rec_rows == o.rec_rows && model == o.model && model_gen == o.model_gen &&
-               mu_E == o.mu_E && sigma_E == o.sigma_E;
+               seeds == o.seeds && obs == o.obs && rec == o.rec && rec_rows == o.rec_rows &&
+               model == o.model && model_gen == o.model_gen && mu_E == o.mu_E && sigma_E == o.sigma_E;
     }
 };
 

@@ -117,3 +117,19 @@ def test_force_model_at_a_freed_models_address(lib):
         assert not np.array_equal(a[1][0][0], b[1][0][0])
         second.close()
         del hold
+
+
+def test_batch_after_a_longer_anneal_of_one_molecule(lib):
+    """The longer anneal moves that molecule's observables buffer."""
+    ctx = lib.pamd_init_batch([pi.make_chain(12, 3), pi.make_chain(20, 4)], [70, 40], [TEMPS[0]] * 2, 1, lib.torch_options())
+    try:
+        first = _run(lib, ctx)
+        lib.pamd_anneal(lib.pamd_batch_sub(ctx, 0), np.linspace(900.0, 700.0, 9), THETA, DT)
+        lib.pamd_reset(ctx, TEMPS[0], 1)
+        again = _run(lib, ctx)
+        for obs in (first[0], again[0]):  # a reset does not clear what the last resampling reported
+            for o in obs[0]:
+                del o["lnQ"], o["max_copies"]
+        _equal(again, first)
+    finally:
+        lib.pamd_destroy(ctx)

@@ -339,8 +339,10 @@ typedef struct pamd_tune {
  * population, energies, counters and observables are left unchanged.  The
  * choice is cached in the process per (N, R, chain layout) and, when the
  * environment variable PAMD_TUNE_CACHE names a file, in that file.
- * theta_probe: 1..1000.  out: chosen shape, or NULL.  Synchronises the
- * stream; must not be called while the stream is being captured.
+ * A molecule of a batch keeps the shape the batch's launches are laid out
+ * for, which is reported.  theta_probe: 1..1000.  out: chosen shape, or NULL.
+ * Synchronises the stream; must not be called while the stream is being
+ * captured.
  */
 int pamd_autotune(pamd_ctx* ctx, int32_t theta_probe, pamd_tune* out);
 

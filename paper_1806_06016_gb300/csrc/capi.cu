@@ -1271,6 +1271,7 @@ int pamd_init_batch(pamd_ctx** out, int32_t n_mol, const pamd_topology* tops, co
             const std::string msg = "molecule " + std::to_string(m) + ": " + g_err;
             return bail(rc, msg);
         }
+        sub->in_batch = true;
         c->subs.push_back(sub);
         if (o.autotune && sub->N >= 3) {
             // measured choice among the batched kernel's shapes
@@ -1805,6 +1806,7 @@ int pamd_autotune(pamd_ctx* c, int32_t theta_probe, pamd_tune* out) {
     if (rc) return rc;
     if (is_batch(c)) return fail(PAMD_EINVAL, "batch context: call this on pamd_batch_sub(ctx, m)");
     if (theta_probe < 1 || theta_probe > 1000) return fail(PAMD_EINVAL, "theta_probe must be 1..1000");
+    if (c->in_batch) return out ? pamd_get_shape(c, out) : PAMD_OK;  // the batch's launches are laid out for this shape
     return autotune_with(c, theta_probe, TuneLimits{1, 8, true, true, {2, 4, 8}, 0}, out);
 }
 

@@ -293,6 +293,7 @@ struct pamd_ctx {
     pamd::TopoF64 top64{};        // all-FP64 mode tables (precision == PAMD_PREC_FP64)
     // batch context (pamd_init_batch): one sub-context per molecule
     std::vector<pamd_ctx*> subs;
+    bool in_batch = false;        // one of those
     void* staging = nullptr;      // rows of the state on their way to or from the host, kept once allocated
     size_t staging_bytes = 0;
     int4* items = nullptr;        // device work lists of the batched propagate, group by group

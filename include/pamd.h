@@ -320,7 +320,7 @@ int pamd_forces(pamd_ctx* ctx, double* f, double* E);
 typedef struct pamd_tune {
     int32_t lanes_per_replica; /* L: lanes of one warp that share a replica */
     int32_t atoms_per_lane;    /* B: atoms each lane owns */
-    int32_t warps_per_block;
+    int32_t warps_per_block;   /* 2 also where two warps share each step (no block size asked for) */
     int32_t replicas_per_lane; /* 1, or 2 for the packed two-replica kernels */
     int32_t from_cache;        /* 1 if the shape came from the cache */
     double ms;                 /* probe time of the chosen shape (0 if cached) */
@@ -334,7 +334,8 @@ typedef struct pamd_tune {
  * shape -- B = 1..8 atoms per lane with L = ceil(N/B) <= 32 lanes per replica
  * (fixed to the requested lanes_per_replica if one was given), one or two
  * replicas per lane group (two only for B = 2..4), and 2, 4 or 8 warps per
- * block -- one propagate launch of theta_probe steps over the whole
+ * block or, for small populations of chains (B = 3..7), two warps that share
+ * each step -- one propagate launch of theta_probe steps over the whole
  * population is timed on a scratch copy; the fastest shape is kept.  The
  * population, energies, counters and observables are left unchanged.  The
  * choice is cached in the process per (N, R, chain layout) and, when the

@@ -667,7 +667,9 @@ int build_topo_f64(pamd_ctx* c, const pamd_topology* t, std::vector<unsigned cha
 }
 
 // In-process cache of tuned shapes, mirrored to the file named by
-// PAMD_TUNE_CACHE ("N R chain lanes_req -> L warps" per line).
+// PAMD_TUNE_CACHE ("N R chain lanes_req pair_arith L warps 10 + variant" per
+// line; without the 10, the two-warp kernel was not among the shapes timed).
+constexpr int kTuneFileTag = 10;
 struct TuneKey {
     int N;
     long long R;
@@ -676,7 +678,7 @@ struct TuneKey {
     int pair_arith;
 };
 struct TuneShape {
-    int L, W, variant;  // variant: kVarScalar, kVarPaired or kVarPacked
+    int L, W, variant;  // variant: kVarScalar, kVarPaired, kVarPacked or kVarSplit
 };
 // Shapes a tuning run may choose: atoms per lane bmin..bmax, the given warp
 // counts, two-replica kernels or not, packed-pair kernels or not.  The batched
@@ -686,6 +688,7 @@ struct TuneLimits {
     int bmin, bmax;
     bool paired_ok;
     bool packed_ok;
+    bool split_ok;
     std::vector<int> warps;
     int key_tag;  // separates the cache entries of restricted searches
 };
@@ -693,7 +696,8 @@ int autotune_with(pamd_ctx* c, int32_t theta_probe, const TuneLimits& lim, pamd_
 std::mutex g_tune_mu;
 std::vector<std::pair<TuneKey, TuneShape>> g_tune;
 
-bool tune_cache_lookup(const TuneKey& k, TuneShape* out) {
+// split: the two-warp kernel is one of the shapes to time
+bool tune_cache_lookup(const TuneKey& k, bool split, TuneShape* out) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto match = [&](const TuneKey& q) {
         return q.N == k.N && q.R == k.R && q.chain == k.chain && q.lanes_req == k.lanes_req &&
@@ -713,8 +717,10 @@ bool tune_cache_lookup(const TuneKey& k, TuneShape* out) {
     bool found = false;
     while (std::fscanf(f, "%d %lld %d %d %d %d %d %d", &q.N, &q.R, &q.chain, &q.lanes_req,
                        &q.pair_arith, &t.L, &t.W, &t.variant) == 8) {
-        if (match(q) && t.L >= 1 && t.L <= 32 && (t.W == 2 || t.W == 4 || t.W == 8) &&
-            (t.variant == kVarScalar || t.variant == kVarPaired || t.variant == kVarPacked)) {
+        const bool tagged = t.variant >= kTuneFileTag;
+        if (tagged) t.variant -= kTuneFileTag;
+        if (match(q) && t.L >= 1 && t.L <= 32 && (t.W == 2 || t.W == 4 || t.W == 8) && (tagged || !split) &&
+            t.variant >= kVarScalar && t.variant <= kVarSplit && (t.variant != kVarSplit || (split && t.W == 2))) {
             *out = t;
             found = true;
         }
@@ -731,7 +737,7 @@ void tune_cache_store(const TuneKey& k, const TuneShape& t) {
     if (!path || !*path) return;
     if (FILE* f = std::fopen(path, "a")) {
         std::fprintf(f, "%d %lld %d %d %d %d %d %d\n", k.N, k.R, k.chain, k.lanes_req, k.pair_arith,
-                     t.L, t.W, t.variant);
+                     t.L, t.W, kTuneFileTag + t.variant);
         std::fclose(f);
     }
 }
@@ -744,7 +750,7 @@ bool packed_ok(const TopoLayout& lay) { return lay.chain && lay.per_lane >= 3 &&
 int set_launch_shape(pamd_ctx* c, const TopoLayout& lay_in, int warps_req, int variant) {
     TopoLayout lay = lay_in;
     lay.paired = variant == kVarPaired ? 1 : 0;
-    lay.packed = variant == kVarPacked ? 1 : 0;
+    lay.packed = variant == kVarPacked || variant == kVarSplit ? 1 : 0;
     if (lay.paired && (lay.per_lane < 2 || lay.per_lane > 4))
         return fail(PAMD_EUNSUPPORTED, "two replicas per lane need 2..4 atoms per lane");
     if (lay.packed && !packed_ok(lay))
@@ -753,6 +759,8 @@ int set_launch_shape(pamd_ctx* c, const TopoLayout& lay_in, int warps_req, int v
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     const int groups_per_warp = 32 / lay.lanes;  // idle lanes when L does not divide 32
+    if (variant == kVarSplit && lay.per_lane > kSplitMaxAtoms)
+        return fail(PAMD_EUNSUPPORTED, "two warps per step need 3..7 atoms per lane");
     int warps = warps_req ? warps_req : 4;
     // One warp per replica group for throughput; two where every warp gets a
     // scheduler of its own (an SM has four): up to two groups per SM.  us a step,
@@ -761,7 +769,8 @@ int set_launch_shape(pamd_ctx* c, const TopoLayout& lay_in, int warps_req, int v
     // 7.8; 200 atoms 304 21.2 / 15.2, 456 21.0 / 25.5.  An explicit block
     // size keeps the one-warp kernel.
     const long long groups = (c->R + groups_per_warp - 1) / groups_per_warp;
-    lay.split = lay.packed && !warps_req && lay.per_lane <= kSplitMaxAtoms && groups <= 2 * (long long)c->num_sms;
+    lay.split = variant == kVarSplit || (lay.packed && !warps_req && lay.per_lane <= kSplitMaxAtoms &&
+                                         groups <= 2 * (long long)c->num_sms);
     // the single-replica kernel of some atoms-per-lane counts takes smaller blocks
     if (lay.packed)
         warps = std::min(warps, kPackedMaxThreads / 32);
@@ -1275,7 +1284,7 @@ int pamd_init_batch(pamd_ctx** out, int32_t n_mol, const pamd_topology* tops, co
         c->subs.push_back(sub);
         if (o.autotune && sub->N >= 3) {
             // measured choice among the batched kernel's shapes
-            const int trc = autotune_with(sub, 20, TuneLimits{3, 7, false, sub->pair_arith == PAMD_PAIRS_PACKED,
+            const int trc = autotune_with(sub, 20, TuneLimits{3, 7, false, sub->pair_arith == PAMD_PAIRS_PACKED, false,
                                                                   {kBatchThreads / 32}, -2}, nullptr);
             if (trc && trc != PAMD_EUNSUPPORTED) {
                 const std::string msg = "molecule " + std::to_string(m) + ": " + g_err;
@@ -1807,7 +1816,7 @@ int pamd_autotune(pamd_ctx* c, int32_t theta_probe, pamd_tune* out) {
     if (is_batch(c)) return fail(PAMD_EINVAL, "batch context: call this on pamd_batch_sub(ctx, m)");
     if (theta_probe < 1 || theta_probe > 1000) return fail(PAMD_EINVAL, "theta_probe must be 1..1000");
     if (c->in_batch) return out ? pamd_get_shape(c, out) : PAMD_OK;  // the batch's launches are laid out for this shape
-    return autotune_with(c, theta_probe, TuneLimits{1, 8, true, true, {2, 4, 8}, 0}, out);
+    return autotune_with(c, theta_probe, TuneLimits{1, 8, true, true, true, {2, 4, 8}, 0}, out);
 }
 
 }  // extern "C"
@@ -1833,7 +1842,15 @@ int autotune_with(pamd_ctx* c, int32_t theta_probe, const TuneLimits& lim, pamd_
                       lim.packed_ok ? c->pair_arith : PAMD_PAIRS_SCALAR};
     TuneShape best_shape{0, 0, 0};
     double best_ms = 0.0;
-    bool cached = tune_cache_lookup(key, &best_shape);
+    // the two-warp kernel, where the population may be small enough for it: up
+    // to twice the replica groups of the untuned rule in set_launch_shape
+    auto split_may_win = [&](int l) {
+        const long long groups = (c->R + 32 / l - 1) / (32 / l);
+        return groups <= 4 * (long long)c->num_sms;
+    };
+    const bool split = lim.split_ok && lim.packed_ok && chain && c->pair_arith != PAMD_PAIRS_SCALAR &&
+                       c->N <= 32 * kSplitMaxAtoms && split_may_win((c->N + kSplitMaxAtoms - 1) / kSplitMaxAtoms);
+    bool cached = tune_cache_lookup(key, split, &best_shape);
     std::vector<unsigned char> blob;
     TopoLayout lay;
     auto apply = [&](const TuneShape& sh) -> int {
@@ -1861,18 +1878,20 @@ int autotune_with(pamd_ctx* c, int32_t theta_probe, const TuneLimits& lim, pamd_
         PAMD_CU(c, cudaEventCreate(&e1));
         double best = 1e300;
         std::vector<TuneShape> shapes;
+        const std::vector<int> two{2};
         for (int b = lim.bmin; b <= lim.bmax; ++b) {
             int l = c->lanes_req ? c->lanes_req : (c->N + b - 1) / b;
             if (l > 32) continue;
             const int bb = (c->N + l - 1) / l;
             if (bb < lim.bmin || bb > lim.bmax) continue;
             l = (c->N + bb - 1) / bb;
-            for (int var = kVarScalar; var <= kVarPacked; ++var) {
+            for (int var = kVarScalar; var <= kVarSplit; ++var) {
                 if (var == kVarPaired && (!lim.paired_ok || bb < 2 || bb > 4)) continue;
                 if (var == kVarPacked && (!lim.packed_ok || !chain || bb < 3 || bb > 8)) continue;
                 if (var == kVarScalar && c->pair_arith == PAMD_PAIRS_PACKED) continue;
                 if (var == kVarPacked && c->pair_arith == PAMD_PAIRS_SCALAR) continue;
-                for (int w : lim.warps) {
+                if (var == kVarSplit && (!split || bb < 3 || bb > kSplitMaxAtoms || !split_may_win(l))) continue;
+                for (int w : var == kVarSplit ? two : lim.warps) {
                     bool dup = false;
                     for (auto& s2 : shapes) dup = dup || (s2.L == l && s2.W == w && s2.variant == var);
                     if (!dup) shapes.push_back({l, w, var});

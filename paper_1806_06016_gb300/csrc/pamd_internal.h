@@ -344,7 +344,7 @@ PAMD_DECLARE_PROPAGATE(8)
 cudaError_t propagate_x2_dispatch(int B, const PropParams* p, int warps, int grid, size_t smem,
                                   cudaStream_t s, bool split, int* blocks_per_sm);
 // launch variants of the single-molecule propagate kernel
-constexpr int kVarScalar = 0, kVarPaired = 1, kVarPacked = 2;
+constexpr int kVarScalar = 0, kVarPaired = 1, kVarPacked = 2, kVarSplit = 3;
 constexpr int kSplitMaxAtoms = 7;        // atoms per lane of the two-warp packed kernel (8: 255 registers do not hold a tile)
 constexpr int kPackedMaxThreads = 128;  // block-size cap of the packed-pair kernel
 // paired kernels (two replicas per lane group), 2..4 atoms per lane

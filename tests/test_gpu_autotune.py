@@ -41,17 +41,17 @@ def test_tuning_one_molecule_leaves_the_batch_alone(lib):
             np.testing.assert_array_equal(u, w)
 
 
-def _block_ms(lib, pop, steps=400):
-    """Best of five propagate blocks."""
+def _block_seconds(pop, steps=400):
+    """Best of five propagate blocks, by the host's clock: the population has a stream of its own."""
+    import time
     import torch
-    a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
     best = 1e9
     for _ in range(5):
-        a.record()
+        torch.cuda.synchronize()
+        start = time.perf_counter()
         pop.propagate(steps, 0.001, 600.0)
-        b.record()
-        b.synchronize()
-        best = min(best, a.elapsed_time(b))
+        torch.cuda.synchronize()
+        best = min(best, time.perf_counter() - start)
     return best
 
 
@@ -60,9 +60,9 @@ def test_tuned_is_not_slower_than_default(lib, n, R):
     """The default is among the shapes timed, so that the choice is at most as
     slow as the default (a tenth is left for the timing)."""
     with lib.Population(pi.make_chain(n, 1), R, 600.0, 3, lib.torch_options()) as pop:
-        default = _block_ms(lib, pop)
+        default = _block_seconds(pop)
         pop.autotune(100)
-        assert _block_ms(lib, pop) <= 1.1 * default
+        assert _block_seconds(pop) <= 1.1 * default
 
 
 def test_cached_shapes(lib, tmp_path, monkeypatch):

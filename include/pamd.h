@@ -340,8 +340,9 @@ typedef struct pamd_tune {
  * population, energies, counters and observables are left unchanged.  The
  * choice is cached in the process per (N, R, chain layout) and, when the
  * environment variable PAMD_TUNE_CACHE names a file, in that file.
- * A molecule of a batch keeps the shape the batch's launches are laid out
- * for, which is reported.  theta_probe: 1..1000.  out: chosen shape, or NULL.
+ * An all-FP64 population has one shape, which follows from N, R and
+ * lanes_per_replica, and a molecule of a batch keeps the shape the batch's
+ * launches are laid out for; either is only reported.  theta_probe: 1..1000.  out: chosen shape, or NULL.
  * Synchronises the stream; must not be called while the stream is being
  * captured.
  */

@@ -795,6 +795,25 @@ int set_launch_shape(pamd_ctx* c, const TopoLayout& lay_in, int warps_req, int v
 
 bool is_batch(const pamd_ctx* c) { return !c->subs.empty(); }
 
+// Shape of the propagate kernel that runs.
+pamd_tune shape_of(const pamd_ctx* c) {
+    pamd_tune t{};
+    t.replicas_per_lane = 1;
+    t.pair_arith = PAMD_PAIRS_SCALAR;
+    if (is_f64(c)) {
+        t.lanes_per_replica = c->top64.lanes;
+        t.atoms_per_lane = c->top64.per_lane;
+        t.warps_per_block = 1;
+        return t;
+    }
+    t.lanes_per_replica = c->lay.lanes;
+    t.atoms_per_lane = c->lay.per_lane;
+    t.warps_per_block = c->warps_per_block;
+    if (c->lay.paired) t.replicas_per_lane = 2;
+    if (c->lay.packed) t.pair_arith = PAMD_PAIRS_PACKED;
+    return t;
+}
+
 // One launch of the batched kernel per group (atoms per lane, pair
 // arithmetic), the groups on streams of their own forked from and joined back
 // to the context's stream (parallel branches when the anneal is captured as
@@ -1832,8 +1851,8 @@ int autotune_with(pamd_ctx* c, int32_t theta_probe, const TuneLimits& lim, pamd_
         ~ModelDetach() { c->mlp = m; }
     } detach{c, c->mlp};
     c->mlp = nullptr;
-    if (is_f64(c)) {  // one fixed shape (a warp per replica)
-        if (out) *out = pamd_tune{32, (c->N + 31) / 32, 4, 1, 0, 0.0};
+    if (is_f64(c)) {  // its shape is chosen by instruction counts (choose_lanes_f64)
+        if (out) *out = shape_of(c);
         return PAMD_OK;
     }
     const pamd_topology t = c->host_top.view();
@@ -1939,11 +1958,7 @@ int autotune_with(pamd_ctx* c, int32_t theta_probe, const TuneLimits& lim, pamd_
         c->graph_key = GraphKey{};
     }
     if (out) {
-        out->lanes_per_replica = c->lay.lanes;
-        out->atoms_per_lane = c->lay.per_lane;
-        out->warps_per_block = c->warps_per_block;
-        out->replicas_per_lane = c->lay.paired ? 2 : 1;
-        out->pair_arith = c->lay.packed ? PAMD_PAIRS_PACKED : PAMD_PAIRS_SCALAR;
+        *out = shape_of(c);
         out->from_cache = cached ? 1 : 0;
         out->ms = best_ms;
     }
@@ -1991,9 +2006,10 @@ int pamd_info(pamd_ctx* c, int64_t* R, int32_t* n_atoms, int32_t* lanes, int32_t
     }
     if (R) *R = c->R;
     if (n_atoms) *n_atoms = c->N;
-    if (lanes) *lanes = c->lay.lanes;
-    if (per_lane) *per_lane = c->lay.per_lane;
-    if (rpb) *rpb = c->rpb;
+    const pamd_tune t = shape_of(c);
+    if (lanes) *lanes = t.lanes_per_replica;
+    if (per_lane) *per_lane = t.atoms_per_lane;
+    if (rpb) *rpb = is_f64(c) ? 32 / t.lanes_per_replica : c->rpb;
     return PAMD_OK;
 }
 
@@ -2016,12 +2032,7 @@ int pamd_population_size(pamd_ctx* c, int64_t* live, int64_t* capacity) {
 int pamd_get_shape(pamd_ctx* c, pamd_tune* out) {
     if (!c || !out) return fail(PAMD_EINVAL, "null argument");
     if (is_batch(c)) return fail(PAMD_EINVAL, "batch context: call this on pamd_batch_sub(ctx, m)");
-    *out = pamd_tune{};
-    out->lanes_per_replica = c->lay.lanes;
-    out->atoms_per_lane = c->lay.per_lane;
-    out->warps_per_block = c->warps_per_block;
-    out->replicas_per_lane = c->lay.paired ? 2 : 1;
-    out->pair_arith = c->lay.packed ? PAMD_PAIRS_PACKED : PAMD_PAIRS_SCALAR;
+    *out = shape_of(c);
     return PAMD_OK;
 }
 

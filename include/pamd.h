@@ -298,6 +298,10 @@ int pamd_anneal(pamd_ctx* ctx, int32_t K, const double* T, int32_t theta, double
 /*
  * Copy the population to the host.  x, v: [R][N][3] double (the FP32 device
  * values widened), E: [R], fam: [R]; any may be NULL.  Synchronises.
+ * pamd_get_state, pamd_set_state and pamd_forces convert through device memory
+ * that the context takes on the first of these calls and keeps: up to 64 MiB,
+ * for a batch up to 64 MiB over all its molecules.  Without it (the allocation
+ * fails) they convert on the host.
  */
 int pamd_get_state(pamd_ctx* ctx, double* x, double* v, double* E, int32_t* fam);
 

@@ -1300,6 +1300,7 @@ int pamd_init_batch(pamd_ctx** out, int32_t n_mol, const pamd_topology* tops, co
             return bail(rc, msg);
         }
         sub->in_batch = true;
+        sub->staging_max = kStagingBytes / (size_t)n_mol & ~size_t(255);
         c->subs.push_back(sub);
         if (o.autotune && sub->N >= 3) {
             // measured choice among the batched kernel's shapes
@@ -1651,14 +1652,10 @@ int pamd_anneal(pamd_ctx* c, int32_t K, const double* T, int32_t theta, double d
 
 namespace {
 
-// Staging memory of the state calls: up to kStagingBytes of device memory,
-// kept with the context.  Larger populations go through it in chunks.
-constexpr size_t kStagingBytes = (size_t)64 << 20;
-
 // Replicas per chunk with `row_bytes` of staging each; 0 if there is no
 // memory for staging.  The first 256 bytes hold the finiteness flag.
 long long staging_chunk(pamd_ctx* c, size_t row_bytes) {
-    const size_t want = std::min(kStagingBytes, 256 + row_bytes * (size_t)c->R);
+    const size_t want = std::min(c->staging_max, 256 + row_bytes * (size_t)c->R);
     if (c->staging_bytes < want) {
         void* p = dalloc(c, want);
         if (!p) return 0;

@@ -187,6 +187,12 @@ struct Buffers {
     float* fout = nullptr;        // [R][3][Np] allocated on demand
 };
 
+// Staging memory of the state calls: at most this much device memory, kept
+// with the context; the molecules of a batch have equal parts of it.  Larger
+// populations go through it in chunks, at about 30 us each: 8192 replicas of
+// 75 atoms, set_state and forces, 1620 us, with 16 MiB 1660, with 8 MiB 1750.
+constexpr size_t kStagingBytes = (size_t)64 << 20;
+
 struct GraphKey {
     int K = -1, theta = -1, resample = -1;
     double dt = 0;
@@ -296,6 +302,7 @@ struct pamd_ctx {
     bool in_batch = false;        // one of those
     void* staging = nullptr;      // rows of the state on their way to or from the host, kept once allocated
     size_t staging_bytes = 0;
+    size_t staging_max = pamd::kStagingBytes;
     int4* items = nullptr;        // device work lists of the batched propagate, group by group
     int n_items = 0;
     int* queue = nullptr;         // device work counters, one per group

@@ -1652,6 +1652,14 @@ int pamd_anneal(pamd_ctx* c, int32_t K, const double* T, int32_t theta, double d
 
 namespace {
 
+// A population this small is converted on the host: one copy and a loop take
+// less than the launches and copies of a staging buffer.  us, host / device (the
+// staging buffer), by replicas x atoms: set_state 3: 15 / 34, 3000: 37 / 52, 6000:
+// 55 / 56, 12000: 89 / 57; positions and velocities read 3: 38 / 54, 6000: 61 / 67,
+// 8000: 66 / 67, 12000: 78 / 72; positions alone 3: 17 / 19, 4000: 26 / 23, 8000: 34 / 25.
+constexpr long long kHostAtoms = 4000;
+bool convert_on_host(const pamd_ctx* c, int arrays) { return c->R * c->N <= kHostAtoms * arrays; }
+
 // Replicas per chunk with `row_bytes` of staging each; 0 if there is no
 // memory for staging.  The first 256 bytes hold the finiteness flag.
 long long staging_chunk(pamd_ctx* c, size_t row_bytes) {
@@ -1698,27 +1706,35 @@ int rows_to_host(pamd_ctx* c, const void* src, int planes, int first, double* ro
     return PAMD_OK;
 }
 
-// The same on the host, for a context without staging memory.
-int rows_to_host_slow(pamd_ctx* c, const void* src, int planes, int first, double* rows) {
-    const int N = c->N, Np = c->Np;
-    const size_t es = is_f64(c) ? 8 : 4;
-    std::vector<unsigned char> buf(es * (size_t)planes * Np * (size_t)c->R);
-    PAMD_CU(c, cudaMemcpyAsync(buf.data(), src, buf.size(), cudaMemcpyDeviceToHost, c->stream));
-    PAMD_CU(c, cudaStreamSynchronize(c->stream));
-    const float* f = reinterpret_cast<const float*>(buf.data());
-    const double* d = reinterpret_cast<const double*>(buf.data());
-    for (long long k = 0; k < c->R; ++k)
+// x and v (either may be null) on the host: planes 0..2 and 3..5 of the records.
+template <typename T>
+void unpack_on_host(const T* rec, long long R, int N, int Np, int planes, double* x, double* v) {
+    for (long long k = 0; k < R; ++k)
         for (int i = 0; i < N; ++i)
             for (int q = 0; q < 3; ++q) {
-                const size_t at = ((size_t)k * planes + first + q) * Np + i;
-                rows[((size_t)k * N + i) * 3 + q] = es == 8 ? d[at] : (double)f[at];
+                const size_t at = ((size_t)k * planes + q) * Np + i, row = ((size_t)k * N + i) * 3 + q;
+                if (x) x[row] = (double)rec[at];
+                if (v) v[row] = (double)rec[at + 3 * (size_t)Np];
             }
+}
+
+int rows_on_host(pamd_ctx* c, const void* src, int planes, double* x, double* v) {
+    std::vector<unsigned char> buf((is_f64(c) ? 8 : 4) * (size_t)planes * c->Np * (size_t)c->R);
+    PAMD_CU(c, cudaMemcpyAsync(buf.data(), src, buf.size(), cudaMemcpyDeviceToHost, c->stream));
+    PAMD_CU(c, cudaStreamSynchronize(c->stream));
+    if (is_f64(c)) unpack_on_host(reinterpret_cast<const double*>(buf.data()), c->R, c->N, c->Np, planes, x, v);
+    else unpack_on_host(reinterpret_cast<const float*>(buf.data()), c->R, c->N, c->Np, planes, x, v);
     return PAMD_OK;
 }
 
-int read_rows(pamd_ctx* c, const void* src, int planes, int first, double* rows) {
-    const int rc = rows_to_host(c, src, planes, first, rows);
-    return rc == PAMD_ENOMEM ? rows_to_host_slow(c, src, planes, first, rows) : rc;
+// Synchronises.
+int read_rows(pamd_ctx* c, const void* src, int planes, double* x, double* v) {
+    if (convert_on_host(c, (x != nullptr) + (v != nullptr))) return rows_on_host(c, src, planes, x, v);
+    int rc = x ? rows_to_host(c, src, planes, 0, x) : PAMD_OK;
+    if (!rc && v) rc = rows_to_host(c, src, planes, 3, v);
+    if (rc == PAMD_ENOMEM) return rows_on_host(c, src, planes, x, v);
+    if (!rc) PAMD_CU(c, cudaStreamSynchronize(c->stream));
+    return rc;
 }
 
 // New population state from the host rows: packed into the alternate buffer
@@ -1750,7 +1766,7 @@ int rows_from_host(pamd_ctx* c, const double* x, const double* v) {
     return PAMD_OK;
 }
 
-int rows_from_host_slow(pamd_ctx* c, const double* x, const double* v) {
+int state_on_host(pamd_ctx* c, const double* x, const double* v) {
     const int N = c->N, Np = c->Np;
     for (size_t e = 0; e < (size_t)c->R * 3 * N; ++e)
         if (!std::isfinite(x[e]) || !std::isfinite(v[e])) return fail(PAMD_EINVAL, "non-finite state");
@@ -1779,8 +1795,6 @@ int pamd_get_state(pamd_ctx* c, double* x, double* v, double* E, int32_t* fam) {
     int rc = check_ctx(c);
     if (rc) return rc;
     if (is_batch(c)) return fail(PAMD_EINVAL, "batch context: call this on pamd_batch_sub(ctx, m)");
-    if (x && (rc = read_rows(c, cur_state(c), 6, 0, x))) return rc;
-    if (v && (rc = read_rows(c, cur_state(c), 6, 3, v))) return rc;
     if (E) {
         touch_pages(E, 8 * (size_t)c->R);
         PAMD_CU(c, cudaMemcpyAsync(E, cur_E(c), 8 * (size_t)c->R, cudaMemcpyDeviceToHost, c->stream));
@@ -1789,6 +1803,7 @@ int pamd_get_state(pamd_ctx* c, double* x, double* v, double* E, int32_t* fam) {
         touch_pages(fam, 4 * (size_t)c->R);
         PAMD_CU(c, cudaMemcpyAsync(fam, cur_fam(c), 4 * (size_t)c->R, cudaMemcpyDeviceToHost, c->stream));
     }
+    if (x || v) return read_rows(c, cur_state(c), 6, x, v);
     PAMD_CU(c, cudaStreamSynchronize(c->stream));
     return PAMD_OK;
 }
@@ -1798,8 +1813,8 @@ int pamd_set_state(pamd_ctx* c, const double* x, const double* v, const double* 
     if (rc) return rc;
     if (is_batch(c)) return fail(PAMD_EINVAL, "batch context: call this on pamd_batch_sub(ctx, m)");
     if (!x || !v) return fail(PAMD_EINVAL, "x and v are required");
-    rc = rows_from_host(c, x, v);
-    if (rc == PAMD_ENOMEM) rc = rows_from_host_slow(c, x, v);
+    rc = convert_on_host(c, 2) ? PAMD_ENOMEM : rows_from_host(c, x, v);
+    if (rc == PAMD_ENOMEM) rc = state_on_host(c, x, v);
     if (rc) return rc;
     if (E) PAMD_CU(c, cudaMemcpyAsync(cur_E(c), E, 8 * (size_t)c->R, cudaMemcpyHostToDevice, c->stream));
     if (fam) PAMD_CU(c, cudaMemcpyAsync(cur_fam(c), fam, 4 * (size_t)c->R, cudaMemcpyHostToDevice, c->stream));
@@ -1817,13 +1832,12 @@ int pamd_forces(pamd_ctx* c, double* f, double* E) {
         if (!c->b.fout) return fail(PAMD_ENOMEM, "force buffer");
     }
     if ((rc = launch_prop(c, 0, 0.001, 300.0, nullptr, c->step, c->b.fout))) return rc;
-    if (f && (rc = read_rows(c, c->b.fout, 3, 0, f))) return rc;
     if (E) {
         touch_pages(E, 8 * (size_t)c->R);
         PAMD_CU(c, cudaMemcpyAsync(E, cur_E(c), 8 * (size_t)c->R, cudaMemcpyDeviceToHost, c->stream));
     }
-    PAMD_CU(c, cudaStreamSynchronize(c->stream));
-    return read_status(c);
+    if (f && (rc = read_rows(c, c->b.fout, 3, f, nullptr))) return rc;
+    return read_status(c);  // synchronises
 }
 
 int pamd_autotune(pamd_ctx* c, int32_t theta_probe, pamd_tune* out) {

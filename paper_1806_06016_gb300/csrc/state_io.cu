@@ -7,6 +7,7 @@
 // arrays.  On one host core they took most of the call: 75 atoms, R = 8192,
 // set_state and forces with the results rounded to FP32, 6.4 ms; now 1.6 ms, of
 // which 0.2 ms is the force kernel and the rest 44 MB over the host link.
+// Small populations stay with the host loops (convert_on_host in capi.cu).
 #include "pamd_internal.h"
 
 namespace pamd {

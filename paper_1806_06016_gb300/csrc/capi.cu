@@ -1727,14 +1727,18 @@ int rows_on_host(pamd_ctx* c, const void* src, int planes, double* x, double* v)
     return PAMD_OK;
 }
 
-// Synchronises.
+// On the device if there is staging memory.  Queued, not waited for: the page
+// touching and what follows run beside the kernels before.
 int read_rows(pamd_ctx* c, const void* src, int planes, double* x, double* v) {
-    if (convert_on_host(c, (x != nullptr) + (v != nullptr))) return rows_on_host(c, src, planes, x, v);
     int rc = x ? rows_to_host(c, src, planes, 0, x) : PAMD_OK;
     if (!rc && v) rc = rows_to_host(c, src, planes, 3, v);
-    if (rc == PAMD_ENOMEM) return rows_on_host(c, src, planes, x, v);
-    if (!rc) PAMD_CU(c, cudaStreamSynchronize(c->stream));
-    return rc;
+    return rc == PAMD_ENOMEM ? rows_on_host(c, src, planes, x, v) : rc;
+}
+
+int read_energies(pamd_ctx* c, double* E) {
+    touch_pages(E, 8 * (size_t)c->R);
+    PAMD_CU(c, cudaMemcpyAsync(E, cur_E(c), 8 * (size_t)c->R, cudaMemcpyDeviceToHost, c->stream));
+    return PAMD_OK;
 }
 
 // New population state from the host rows: packed into the alternate buffer
@@ -1795,15 +1799,16 @@ int pamd_get_state(pamd_ctx* c, double* x, double* v, double* E, int32_t* fam) {
     int rc = check_ctx(c);
     if (rc) return rc;
     if (is_batch(c)) return fail(PAMD_EINVAL, "batch context: call this on pamd_batch_sub(ctx, m)");
-    if (E) {
-        touch_pages(E, 8 * (size_t)c->R);
-        PAMD_CU(c, cudaMemcpyAsync(E, cur_E(c), 8 * (size_t)c->R, cudaMemcpyDeviceToHost, c->stream));
-    }
+    // the rows first where they are long, last where the host's loop waits for them
+    const int rows = (x != nullptr) + (v != nullptr);
+    const bool on_host = rows && convert_on_host(c, rows);
+    if (rows && !on_host && (rc = read_rows(c, cur_state(c), 6, x, v))) return rc;
+    if (E && (rc = read_energies(c, E))) return rc;
     if (fam) {
         touch_pages(fam, 4 * (size_t)c->R);
         PAMD_CU(c, cudaMemcpyAsync(fam, cur_fam(c), 4 * (size_t)c->R, cudaMemcpyDeviceToHost, c->stream));
     }
-    if (x || v) return read_rows(c, cur_state(c), 6, x, v);
+    if (on_host) return rows_on_host(c, cur_state(c), 6, x, v);
     PAMD_CU(c, cudaStreamSynchronize(c->stream));
     return PAMD_OK;
 }
@@ -1832,11 +1837,10 @@ int pamd_forces(pamd_ctx* c, double* f, double* E) {
         if (!c->b.fout) return fail(PAMD_ENOMEM, "force buffer");
     }
     if ((rc = launch_prop(c, 0, 0.001, 300.0, nullptr, c->step, c->b.fout))) return rc;
-    if (E) {
-        touch_pages(E, 8 * (size_t)c->R);
-        PAMD_CU(c, cudaMemcpyAsync(E, cur_E(c), 8 * (size_t)c->R, cudaMemcpyDeviceToHost, c->stream));
-    }
-    if (f && (rc = read_rows(c, c->b.fout, 3, f, nullptr))) return rc;
+    const bool on_host = f && convert_on_host(c, 1);
+    if (f && !on_host && (rc = read_rows(c, c->b.fout, 3, f, nullptr))) return rc;
+    if (E && (rc = read_energies(c, E))) return rc;
+    if (on_host && (rc = rows_on_host(c, c->b.fout, 3, f, nullptr))) return rc;
     return read_status(c);  // synchronises
 }
 

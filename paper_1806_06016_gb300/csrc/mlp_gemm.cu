@@ -401,12 +401,12 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs& g, uint32_t taddr,
             else store_row32_bf16(Cb + (size_t)row * g.ldcb + col0, v, ns);
         }
     }
-    // one partial sum of the head per 128 columns; a tile of up to 128 columns
-    // that is the last one writes the zero of the missing other half as well
+    // one partial sum of the head per 128 columns; a tile of 128 columns that
+    // is the last one writes the zero of the missing other half as well
     if (g.epi == kEpiHead && row_ok) {
         const int np = gemm_head_parts(g.N), at = n0 / 128;
         g.part[(size_t)row * np + at] = head;
-        if (at + 1 < np && n0 + 128 >= g.N && chunks * 32 <= 128 && at % 2 == 0) g.part[(size_t)row * np + at + 1] = 0.0f;
+        if (at + 1 < np && n0 + 128 >= g.N && chunks * 32 == 128 && at % 2 == 0) g.part[(size_t)row * np + at + 1] = 0.0f;
     }
 }
 
@@ -596,9 +596,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             tc_fence_after();
             const int m0 = (2 * (t / NT) + crank) * kBM, nt = t % NT;
             const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kBN);
-            // the head's partial sums run over 128 columns: with a tile no
-            // wider than that one warp per quarter takes them all
-            if (BN <= 128 && g.epi == kEpiHead) {
+            // the head's partial sums run over 128 columns: with a tile that
+            // narrow one warp per quarter takes them all
+            if (BN == 128 && g.epi == kEpiHead) {
                 if (half == 0) epilogue_tile(g, taddr, m0 + q * 32, nt * kBN, BN / 32, stage);
             } else {
                 epilogue_tile(g, taddr + (uint32_t)(half * (kBN / 2)), m0 + q * 32, nt * kBN + half * (kBN / 2),
@@ -735,12 +735,10 @@ long long gemm_tiles(const GemmArgs& g, int bn) {
 //   N 512,  K 512:  M 2048 8.3 / 10.3 / 12.4, 8192 14.5 / 12.5 / 12.4;
 //   N 2776, K 512:  M 256 8.3 / 10.3 / 12.4, 512 10.4 / 10.3 / 12.4
 // (before the stores through shared memory, which the wide tiles gain from).
-// The head sums over 128 columns in one thread: not below that, unless one
-// narrow tile holds all of them; the products of a small model are then one
-// kernel (100 samples of 9 atoms, H = 64, calls in a stream: 42.8 -> 41.1 us).
+// The head sums over 128 columns in one thread: not below that.
 int tile_width(const GemmArgs& g, int max_clusters) {
     int bn = 256;
-    while (bn > (g.epi == kEpiHead && g.N > 64 ? 128 : 64) && gemm_tiles(g, bn / 2) <= max_clusters) bn /= 2;
+    while (bn > (g.epi == kEpiHead ? 128 : 64) && gemm_tiles(g, bn / 2) <= max_clusters) bn /= 2;
     return bn;
 }
 

@@ -158,9 +158,10 @@ __global__ void mlp_adam_kernel(float* p, const float* __restrict__ g, float* m,
 // One thread per pair, the positions of a tile of configurations in shared
 // memory as float4 (consecutive pairs read consecutive atoms: no bank
 // conflicts), the data cut into as many slices as fill the chip.
-// 65536 configurations of 75 atoms: 661 + 30 us, bound by the FP32 issue rate
-// (about 90 instructions per sample and pair).  Deviations rounded to FP32
-// took 611 us and lost up to half the last bit of sd; one thread per pair
+// 65536 configurations of 75 atoms: 624 + 31 us, bound by instruction issue
+// (about 100 per sample and pair, 83 % of the slots; 661 us with a subnormal-safe
+// reciprocal square root and a TwoSum for the squares).  Deviations rounded to
+// FP32 took 611 us and lost up to half the last bit of sd; one thread per pair
 // looping twice over all configurations in FP64 (22 blocks) took 151.0 ms.
 // Against 64-bit torch, 27 sets of 9..75 atoms x 100..65536 samples: mu and sd
 // are as far from it as that FP64 loop's, to five digits.
@@ -241,13 +242,13 @@ __global__ void __launch_bounds__(kStatThreads) mlp_moments_kernel(const float* 
         const float lo = __fadd_rn(__fadd_rn(l1, l2), __fmaf_rn(2.0f, qc, qe));
         h_min = fminf(h_min, h);
         h_max = fmaxf(h_max, h);
-        y = rsqrtf(h);
+        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(h));  // no subnormal h comes into the sums
         // e = 1 - r^2 y^2
         const float u = __fmul_rn(h, y), ue = __fmaf_rn(h, y, -u);
         float e = __fmaf_rn(-u, y, 1.0f);
         e = __fmaf_rn(-ue, y, e);
         e = __fmaf_rn(-__fmul_rn(lo, y), y, e);
-        corr = __fmul_rn(y, __fmaf_rn(__fmul_rn(0.375f, e), e, __fmul_rn(0.5f, e)));
+        corr = __fmul_rn(__fmul_rn(y, e), __fmaf_rn(0.375f, e, 0.5f));
     };
     for (long long t0 = m0; t0 < m1; t0 += tile) {
         const int nt = (int)(m1 - t0 < tile ? m1 - t0 : tile);
@@ -257,7 +258,7 @@ __global__ void __launch_bounds__(kStatThreads) mlp_moments_kernel(const float* 
             sx[a] = make_float4(src[3 * a], src[3 * a + 1], src[3 * a + 2], 0.0f);
         __syncthreads();
         if (t0 == m0) feature(0, g0, c0);
-#pragma unroll 2
+#pragma unroll 4
         for (int c = 0; c < nt; ++c) {
             float y, corr, ey0, dl, err;
             feature(c, y, corr);
@@ -269,8 +270,9 @@ __global__ void __launch_bounds__(kStatThreads) mlp_moments_kernel(const float* 
             sl = __fadd_rn(sl, __fadd_rn(err, dl));
             float e2;
             const float d2 = square_err(d, dl, e2);
-            q = two_sum(q, d2, err);
-            ql = __fadd_rn(ql, __fadd_rn(err, e2));
+            const float big = fmaxf(q, d2), small = fminf(q, d2);  // neither is negative
+            q = __fadd_rn(big, small);
+            ql = __fadd_rn(ql, __fadd_rn(__fsub_rn(small, __fsub_rn(q, big)), e2));
         }
         held += nt;
         if (held >= kStatHold || t0 + tile >= m1) {

@@ -343,7 +343,9 @@ typedef struct pamd_tune {
  * population is timed on a scratch copy; the fastest shape is kept.  The
  * population, energies, counters and observables are left unchanged.  The
  * choice is cached in the process per (N, R, chain layout) and, when the
- * environment variable PAMD_TUNE_CACHE names a file, in that file.
+ * environment variable PAMD_TUNE_CACHE names a file, in that file (an entry
+ * for which the two-warp kernel was not timed, though it could win, does not
+ * count).
  * An all-FP64 population has one shape, which follows from N, R and
  * lanes_per_replica, and a molecule of a batch keeps the shape the batch's
  * launches are laid out for; either is only reported.  theta_probe: 1..1000.  out: chosen shape, or NULL.
